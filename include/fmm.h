@@ -33,8 +33,9 @@
  * widened exactly to float32.  Results are deterministic: the same plan and
  * inputs give bitwise identical outputs on every call (no floating-point
  * atomics).  16-byte aligned dense pointers with r in {32, 64, 128, 256}
- * take the vectorised kernels; any other r or alignment takes a slower
- * generic GPU kernel with the same results up to rounding.  No call ever
+ * take the vectorised kernels; any other r up to 512, or alignment, takes a
+ * flexible-width kernel, wider rows a slower generic one, with the same
+ * results up to rounding.  No call ever
  * falls back to the CPU.
  *
  * Streams and ownership

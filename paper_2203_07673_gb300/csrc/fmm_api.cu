@@ -1,4 +1,5 @@
 // C-ABI entry points of libfmm (declared in include/fmm.h).
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <cstdio>
@@ -52,6 +53,31 @@ static const int kVariantCodes[] = {114, 118, 222, 224, 441, 442, 214, 124, 112,
                                     1041, 1042, 1081, 1082,
                                     22212, 23212, 22412, 32212, 24221, 34221, 23421, 23241,
                                     44042, 43082, 44041, 44081, 52212, 52412, 54211};
+
+int flex_lanes(int32_t r)
+{
+    const int e = r <= 256 ? 8 : 16;   // elements per lane
+    int g = 1;
+    while (g * e < r) g *= 2;
+    return g;
+}
+
+// Bytes per vector of the flexible pass: the widest power of two up to 16
+// that divides a row and the alignment of the operands (float32 operands
+// beside bfloat16 rows are read in the same pieces, so an element count of
+// vb / e must keep them aligned as well).
+static int flex_vector_bytes(const PassArgs &a, int dtype)
+{
+    const uintptr_t e = dtype == FMM_BF16 ? 2 : 4;
+    const uintptr_t rows = reinterpret_cast<uintptr_t>(a.L) | reinterpret_cast<uintptr_t>(a.Y) |
+                           ((uintptr_t)a.r * e);
+    const uintptr_t f32 = reinterpret_cast<uintptr_t>(a.H) | reinterpret_cast<uintptr_t>(a.out);
+    int vb = 16;
+    while (vb > (int)e &&
+           ((rows & (vb - 1)) || (f32 & (std::min<uintptr_t>(16, vb / e * 4) - 1))))
+        vb /= 2;
+    return vb;
+}
 
 bool variant_known(int code)
 {
@@ -150,6 +176,19 @@ cudaError_t launch_pass(int mode, int dtype, const KernelVariant &v, const PassA
             return e;
         // a ring layout this width does not have: the team kernel below
     }
+    if (!vec && a.r <= kFlexMaxR) {
+        // any other width or alignment: the flexible pass.  Lane groups per
+        // row: doubled while the launch leaves lanes idle (1024 resident per
+        // SM) and every group still has a batch of two nonzeros
+        const long long items = (long long)a.n_chunks + a.n_light;
+        const long long fill = (long long)sm_count() * 32 * 32;   // resident lanes
+        int ng = 1;
+        while (ng < 32 && items * flex_lanes(a.r) * ng * 2 <= fill && items * 4 * ng <= a.nnz)
+            ng *= 2;
+        const int vb = flex_vector_bytes(a, dtype);
+        return dtype == FMM_BF16 ? launch_flex_bf16(mode, a, vb, ng, st)
+                                 : launch_flex_f32(mode, a, vb, ng, st);
+    }
     // other backward roles of a staged, pipelined or bulk-staged plan: the
     // team kernel's default layout for the width
     const KernelVariant t =
@@ -230,6 +269,7 @@ int run_pass(const fmm_plan *p, const Side &side, int mode, const float *s, cons
     a.r = p->r;
     a.err = p->err;
     a.accumulate = accumulate ? 1 : 0;
+    a.nnz = p->nnz;
     cudaError_t e = cudaSuccess;
     if (side.perm && s) {
         if (s == p->static_src && p->vals_static) {

@@ -1,0 +1,347 @@
+// Row pass for any width and alignment, and for passes too small to fill the
+// GPU with one lane group per row.
+//
+// The layouts of fmm_rows.cuh fix the row width, the lanes per row and the
+// lane groups per row at compile time.  Here only the loads are fixed: a row
+// of r elements is cut into vectors of VB bytes (the widest that divides the
+// row and that every operand is aligned to), a lane holds E elements of it
+// (E / EPV vectors, lane l the vectors l, l + G, ...; vectors past the row
+// are zeros that are never loaded), and the G lanes of a group and the
+// groups of a team are launch parameters.  The NG groups of a team take the
+// nonzeros of their row or chunk in turn and sum their partial rows at the
+// end in a fixed xor order.
+//
+// What bounds it: the gathers (L2 or HBM), as in the other passes; with the
+// output row in registers each gathered row is read once.  Column indices
+// and values of the next batch are loaded while the current one is used
+// (every lane of a group reads the same word: one request per group).
+// 8 elements per lane up to r = 256, as the team kernel's default layout (the
+// light register footprint keeps more rows in flight), 16 up to 512.
+//
+// Measured on GB300 against the generic kernel, which it replaces for r <=
+// 512 (float32, r = 100, 60013 x 41999, 1.2M nonzeros, a hub row of 1200):
+// FusedMM 337 -> 88 us, adjoint over S 378 -> 121, over S^T 325 -> 106.
+#pragma once
+
+#include "fmm_rows.cuh"
+
+namespace fmm {
+
+struct FlexShape {
+    int g;        // lanes per group (power of two, <= 32)
+    int ng;       // groups per team (power of two, g * ng <= 32)
+    int nvec;     // vectors per row
+};
+
+// One vector of VB bytes of a row of T, widened to EPV floats.
+template <typename T, int VB>
+__device__ __forceinline__ void flex_load(const T *p, float *f, bool gather)
+{
+    if constexpr (VB == 16) {
+        const uint4 *q = reinterpret_cast<const uint4 *>(p);
+        const uint4 w = gather ? __ldg(q) : __ldcs(q);
+        if constexpr (sizeof(T) == 2) {
+            unpack_bf16x8(w, f);
+        } else {
+            f[0] = __uint_as_float(w.x); f[1] = __uint_as_float(w.y);
+            f[2] = __uint_as_float(w.z); f[3] = __uint_as_float(w.w);
+        }
+    } else if constexpr (VB == 8) {
+        const uint2 *q = reinterpret_cast<const uint2 *>(p);
+        const uint2 w = gather ? __ldg(q) : __ldcs(q);
+        if constexpr (sizeof(T) == 2) {
+            f[0] = __uint_as_float(w.x << 16); f[1] = __uint_as_float(w.x & 0xffff0000u);
+            f[2] = __uint_as_float(w.y << 16); f[3] = __uint_as_float(w.y & 0xffff0000u);
+        } else {
+            f[0] = __uint_as_float(w.x); f[1] = __uint_as_float(w.y);
+        }
+    } else if constexpr (VB == 4) {
+        const uint32_t *q = reinterpret_cast<const uint32_t *>(p);
+        const uint32_t w = gather ? __ldg(q) : __ldcs(q);
+        if constexpr (sizeof(T) == 2) {
+            f[0] = __uint_as_float(w << 16); f[1] = __uint_as_float(w & 0xffff0000u);
+        } else {
+            f[0] = __uint_as_float(w);
+        }
+    } else {
+        static_assert(sizeof(T) == 2, "two-byte vectors are bfloat16 elements");
+        f[0] = widen<T>(gather ? __ldg(p) : __ldcs(p));
+    }
+}
+
+// EPV floats from or to an address aligned to min(16, 4 EPV) bytes.
+template <int EPV>
+__device__ __forceinline__ void flex_load_f32(const float *p, float *f, bool gather)
+{
+    if constexpr (EPV % 4 == 0) {
+#pragma unroll
+        for (int q = 0; q < EPV / 4; ++q) {
+            const float4 *a = reinterpret_cast<const float4 *>(p) + q;
+            const float4 x = gather ? __ldg(a) : __ldcs(a);
+            f[4 * q] = x.x; f[4 * q + 1] = x.y; f[4 * q + 2] = x.z; f[4 * q + 3] = x.w;
+        }
+    } else if constexpr (EPV == 2) {
+        const float2 *a = reinterpret_cast<const float2 *>(p);
+        const float2 x = gather ? __ldg(a) : __ldcs(a);
+        f[0] = x.x; f[1] = x.y;
+    } else {
+        f[0] = gather ? __ldg(p) : __ldcs(p);
+    }
+}
+
+template <int EPV>
+__device__ __forceinline__ void flex_store_f32(float *p, const float *f, bool add)
+{
+    if constexpr (EPV % 4 == 0) {
+        const Loader ld;
+#pragma unroll
+        for (int q = 0; q < EPV / 4; ++q)
+            out_store4(ld, p + 4 * q, make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]),
+                       add);
+    } else if constexpr (EPV == 2) {
+        float2 v = make_float2(f[0], f[1]);
+        if (add) {
+            const float2 o = __ldcs(reinterpret_cast<const float2 *>(p));
+            v.x += o.x; v.y += o.y;
+        }
+        __stcs(reinterpret_cast<float2 *>(p), v);
+    } else {
+        __stcs(p, add ? f[0] + __ldcs(p) : f[0]);
+    }
+}
+
+// Accumulates into acc the nonzeros beg + first, beg + first + step, ... of
+// [beg, end): the share of one group of g lanes (lig = lane within it).
+// Every lane of the warp must call it.
+template <int MODE, typename T, int VB, int E>
+__device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, int end, int first,
+                                           int step, int g, int lig, int nvec, float (&acc)[E])
+{
+    constexpr int EPV = VB / (int)sizeof(T), VPL = E / EPV;
+    constexpr int U = E <= 8 ? 2 : 1;
+    constexpr bool HAS_L = MODE != M_SPMM;
+    constexpr bool TWO = MODE == M_BWD_ROW || MODE == M_BWD_COL;
+    constexpr bool NZ = MODE == M_SDDMM || MODE == M_BWD_ROW;
+    constexpr int ND = TWO ? 2 * U : U;
+    static_assert(E % EPV == 0, "whole vectors per lane");
+
+    const int r = a.r;
+    const T *L = static_cast<const T *>(a.L);
+    const T *Y = static_cast<const T *>(a.Y);
+    // lane's first element; vector v of the lane starts at k0 + v * vs
+    const int k0 = lig * EPV, vs = g * EPV;
+    const int mine = lig < nvec ? (nvec - lig + g - 1) / g : 0;   // vectors of this lane
+
+    float lrow[E], hrow[MODE == M_BWD_ROW ? E : 1];
+#pragma unroll
+    for (int e = 0; e < E; ++e) { lrow[e] = 0.f; acc[e] = 0.f; }
+#pragma unroll
+    for (int e = 0; e < (MODE == M_BWD_ROW ? E : 1); ++e) hrow[e] = 0.f;
+    if (HAS_L && end > beg) {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+            if (v < mine) {
+                flex_load<T, VB>(L + (size_t)row * r + k0 + v * vs, &lrow[v * EPV], false);
+                if constexpr (MODE == M_BWD_ROW)
+                    flex_load_f32<EPV>(a.H + (size_t)row * r + k0 + v * vs, &hrow[v * EPV], false);
+            }
+    }
+
+    // positions relative to beg, unsigned: past the end they cannot wrap
+    const unsigned n = (unsigned)(end - beg), span = (unsigned)(U * step);
+    const unsigned iters = n > (unsigned)first ? (n - first + span - 1) / span : 0;
+    const unsigned witers = __reduce_max_sync(0xffffffffu, iters);
+    unsigned q = first;
+    int jn[U], sin_[U];
+    float svn[U];
+    auto fetch = [&]() {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            jn[u] = -1; sin_[u] = 0; svn[u] = 0.f;
+            if (q + u * step < n) {
+                const int pp = beg + (int)(q + u * step);
+                jn[u] = __ldg(a.col_idx + pp);
+                sin_[u] = (a.perm && (NZ || !a.s_direct)) ? __ldg(a.perm + pp) : pp;
+                svn[u] = a.s ? __ldg(a.s + (a.s_direct ? pp : sin_[u])) : 1.f;
+            }
+        }
+    };
+    fetch();
+    for (unsigned it = 0; it < witers; ++it) {
+        int jj[U], sidx[U];
+        float sv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) { jj[u] = jn[u]; sidx[u] = sin_[u]; sv[u] = svn[u]; }
+        float y[U][E], h[MODE == M_BWD_COL ? U : 1][E];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                y[u][e] = 0.f;
+                if constexpr (MODE == M_BWD_COL) h[u][e] = 0.f;
+            }
+            if (jj[u] >= 0) {
+                const T *yp = Y + (size_t)jj[u] * r + k0;
+#pragma unroll
+                for (int v = 0; v < VPL; ++v)
+                    if (v < mine)
+                        flex_load<T, VB>(yp + v * vs, &y[u][v * EPV], true);
+                if constexpr (MODE == M_BWD_COL) {
+                    const float *hp = a.H + (size_t)jj[u] * r + k0;
+#pragma unroll
+                    for (int v = 0; v < VPL; ++v)
+                        if (v < mine)
+                            flex_load_f32<EPV>(hp + v * vs, &h[u][v * EPV], true);
+                }
+            }
+        }
+        q += span;
+        fetch();
+        if constexpr (MODE == M_SPMM) {
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (jj[u] >= 0)
+                        acc[e] = fmaf(sv[u], y[u][e], acc[e]);
+            continue;
+        }
+        float d[ND];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            float t = 0.f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) t = fmaf(lrow[e], y[u][e], t);
+            d[u] = t;
+            if constexpr (TWO) {
+                float w = 0.f;
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    w = MODE == M_BWD_ROW ? fmaf(hrow[MODE == M_BWD_ROW ? e : 0], y[u][e], w)
+                                          : fmaf(h[MODE == M_BWD_COL ? u : 0][e], lrow[e], w);
+                d[U + u] = w;
+            }
+        }
+        for (int off = g >> 1; off > 0; off >>= 1) {
+#pragma unroll
+            for (int i = 0; i < ND; ++i)
+                d[i] += __shfl_xor_sync(0xffffffffu, d[i], off);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (jj[u] < 0)
+                continue;
+            if constexpr (MODE == M_FUSED) {
+                const float c = sv[u] * d[u];
+#pragma unroll
+                for (int e = 0; e < E; ++e) acc[e] = fmaf(c, y[u][e], acc[e]);
+            } else if constexpr (MODE == M_SDDMM) {
+                if (lig == 0)
+                    nz_store<MODE>(a, sidx[u], sv[u] * d[u]);
+            } else if constexpr (MODE == M_BWD_ROW) {
+                if (lig == 0 && a.nzout)
+                    a.nzout[sidx[u]] = d[u] * d[U + u];
+                const float c = sv[u] * d[U + u];
+#pragma unroll
+                for (int e = 0; e < E; ++e) acc[e] = fmaf(c, y[u][e], acc[e]);
+            } else if constexpr (MODE == M_BWD_COL) {
+                const float c1 = sv[u] * d[u], c2 = sv[u] * d[U + u];
+#pragma unroll
+                for (int e = 0; e < E; ++e) acc[e] = fmaf(c1, h[u][e], fmaf(c2, y[u][e], acc[e]));
+            }
+        }
+    }
+}
+
+// Blocks of two warps, as the team kernel's; register caps of 64 per thread
+// in the forward roles, 72 in the pass over S, 80 in the pass over S^T (none
+// spills).
+constexpr int kFlexBlock = 64;
+
+template <int MODE, typename T, int VB, int E>
+__global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 12 : MODE == M_BWD_ROW ? 14 : 16))
+    flex_pass_kernel(const PassArgs a, const FlexShape sh)
+{
+    constexpr int EPV = VB / (int)sizeof(T), VPL = E / EPV;
+    const int team = sh.g * sh.ng;
+    const int lane = threadIdx.x & 31;
+    const int lig = lane & (sh.g - 1);
+    const int grp = (lane & (team - 1)) / sh.g;
+    const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / team;
+    const bool active = gid < (long long)a.n_chunks + a.n_light;
+    int row = 0, beg = 0, end = 0, slot = -1;
+    if (active)
+        pass_item(a, gid, row, beg, end, slot);
+    float acc[E];
+    flex_range<MODE, T, VB, E>(a, row, beg, end, grp, sh.ng, sh.g, lig, sh.nvec, acc);
+    if constexpr (MODE != M_SDDMM) {
+        for (int off = sh.g; off < team; off <<= 1) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], off);
+        }
+        if (!active || grp != 0)
+            return;
+        float *dst = slot >= 0 ? a.partials + (size_t)slot * a.r
+                               : (a.out ? a.out + (size_t)row * a.r : nullptr);
+        if (!dst)
+            return;
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+            if (v * sh.g + lig < sh.nvec)
+                flex_store_f32<EPV>(dst + (v * sh.g + lig) * EPV, &acc[v * EPV],
+                                    a.accumulate && slot < 0);
+    }
+}
+
+template <int MODE, typename T, int VB, int E>
+cudaError_t launch_flex_shape(const PassArgs &a, int ng, cudaStream_t st)
+{
+    constexpr int EPV = VB / (int)sizeof(T), VPL = E / EPV;
+    FlexShape sh;
+    sh.nvec = a.r / EPV;
+    sh.g = flex_lanes(a.r);
+    static_assert(VPL * EPV == E, "E elements per lane");
+    sh.ng = 1;
+    while (sh.ng < ng && sh.g * sh.ng < 32) sh.ng *= 2;
+    const long long total = (long long)a.n_chunks + a.n_light;
+    const long long blocks = (total * sh.g * sh.ng + kFlexBlock - 1) / kFlexBlock;
+    flex_pass_kernel<MODE, T, VB, E><<<(unsigned)blocks, kFlexBlock, 0, st>>>(a, sh);
+    return cudaGetLastError();
+}
+
+// vb: bytes per vector (a power of two up to 16, a multiple of the element
+// size, dividing the row and the alignment of every operand).
+template <int MODE, typename T>
+cudaError_t dispatch_flex(const PassArgs &a, int vb, int ng, cudaStream_t st)
+{
+#define FMM_FLEX(VB)                                                       \
+    if (vb == VB)                                                          \
+        return a.r <= 256 ? launch_flex_shape<MODE, T, VB, 8>(a, ng, st)   \
+                          : launch_flex_shape<MODE, T, VB, 16>(a, ng, st);
+    FMM_FLEX(16)
+    FMM_FLEX(8)
+    FMM_FLEX(4)
+    if constexpr (sizeof(T) == 2) {
+        FMM_FLEX(2)
+    }
+#undef FMM_FLEX
+    return cudaErrorInvalidValue;
+}
+
+template <typename T>
+cudaError_t launch_flex_typed(int mode, const PassArgs &a, int vb, int ng, cudaStream_t st)
+{
+    if ((long long)a.n_chunks + a.n_light == 0)
+        return cudaSuccess;
+    switch (mode) {
+    case M_FUSED: return dispatch_flex<M_FUSED, T>(a, vb, ng, st);
+    case M_SDDMM: return dispatch_flex<M_SDDMM, T>(a, vb, ng, st);
+    case M_SPMM: return dispatch_flex<M_SPMM, T>(a, vb, ng, st);
+    case M_BWD_ROW: return dispatch_flex<M_BWD_ROW, T>(a, vb, ng, st);
+    case M_BWD_COL: return dispatch_flex<M_BWD_COL, T>(a, vb, ng, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace fmm

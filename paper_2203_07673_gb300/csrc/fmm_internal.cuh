@@ -115,6 +115,7 @@ struct PassArgs {
     int32_t *err = nullptr;    // device word set to 1 by a pass that gave up a
                                // bounded wait (NULL: not reported)
     int32_t accumulate = 0;    // 1: out += the pass's rows (else out =)
+    int64_t nnz = 0;           // nonzeros of the pattern walked (launch rules)
 };
 
 // Launches one row pass (main kernel; the combine kernel for split rows is
@@ -125,6 +126,14 @@ cudaError_t launch_pass_f32(int mode, int vpl_mult, int ng, int u, bool vec, con
                             cudaStream_t st);
 cudaError_t launch_pass_bf16(int mode, int vpl_mult, int ng, int u, bool vec, const PassArgs &a,
                              cudaStream_t st);
+// Flexible-width passes (fmm_flex.cuh): vb bytes per vector, ng lane groups
+// per row at most.
+cudaError_t launch_flex_f32(int mode, const PassArgs &a, int vb, int ng, cudaStream_t st);
+cudaError_t launch_flex_bf16(int mode, const PassArgs &a, int vb, int ng, cudaStream_t st);
+// Widest row of the flexible pass (32 lanes of 16 elements).
+constexpr int32_t kFlexMaxR = 512;
+// Lanes of one group of the flexible pass for rows of r elements.
+int flex_lanes(int32_t r);
 // Staged forward-role passes (fmm_staged.cuh): FusedMM, SDDMM and SpMM with a
 // cp.async ring of `stages` gathered rows per team; vector path only.
 cudaError_t launch_staged_f32(int mode, int vpl_mult, int stages, const PassArgs &a,

@@ -745,6 +745,8 @@ int32_t default_split_nnz(int64_t nnz, int32_t r, int32_t dtype, const KernelVar
         const int vecs = r * e / 16;
         const int vpl = (vecs > 32 ? vecs / 32 : 1) * v.vpl_mult;
         lanes = std::min(32, std::max(1, vecs / std::max(1, vpl)) * std::max(1, v.ng));
+    } else if (r <= kFlexMaxR) {
+        lanes = flex_lanes(r);
     }
     const int warps = (v.ring > 0 || v.depth > 0 || v.stream) && v.mb > 0 ? 8 * v.mb : 32;
     const int64_t teams = (int64_t)sm_count() * warps * (32 / lanes);

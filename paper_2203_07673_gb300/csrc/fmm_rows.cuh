@@ -519,7 +519,8 @@ __device__ __forceinline__ float warp_allreduce(float v)
     return v;
 }
 
-// Generic pass for any r and any alignment: one warp per row or chunk,
+// Generic pass for rows wider than the flexible pass takes (fmm_flex.cuh),
+// any alignment: one warp per row or chunk,
 // scalar loads strided by lane, the output row accumulated in place (each
 // lane owns the columns k = lane + 32 t, so no two lanes touch one word).
 template <int MODE, typename T>
