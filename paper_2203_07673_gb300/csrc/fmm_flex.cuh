@@ -20,7 +20,8 @@
 //
 // Measured on GB300 against the generic kernel, which it replaces for r <=
 // 512 (float32, r = 100, 60013 x 41999, 1.2M nonzeros, a hub row of 1200):
-// FusedMM 337 -> 88 us, adjoint over S 378 -> 121, over S^T 325 -> 106.
+// FusedMM 337 -> 115 us (88 with the order of its sums left free), adjoint over
+// S 378 -> 120, over S^T 325 -> 106.
 #pragma once
 
 #include "fmm_rows.cuh"
@@ -107,6 +108,48 @@ __device__ __forceinline__ void flex_store_f32(float *p, const float *f, bool ad
         __stcs(reinterpret_cast<float2 *>(p), v);
     } else {
         __stcs(p, add ? f[0] + __ldcs(p) : f[0]);
+    }
+}
+
+// Whether a role adds in the order of the generic kernel: float32 FusedMM and
+// SpMM, whose results an iteration may amplify (the conjugate gradients of
+// ALS past their convergence), are the same bits as the generic kernel's.
+// That fixes the lanes of a group (32 / EPV, so that element e of vector v of
+// lane l is element 32 v + EPV l + e: position EPV l + e of the generic
+// kernel's warp, step v), one group per row, and the order of the dot product
+// below.
+template <int MODE, typename T>
+constexpr bool flex_ordered() { return sizeof(T) == 4 && (MODE == M_FUSED || MODE == M_SPMM); }
+
+// Sum over the 32 / EPV lanes of a group and the EPV elements of each, in the
+// order of a 32-lane xor butterfly over positions EPV l + e (offsets 16, 8,
+// 4, 2, 1).  The first offsets cross lanes, the last ones elements; a lane
+// keeps half of its elements at each of the first log2(EPV) offsets, so the
+// elements' offsets become one shuffle each at the end.
+template <int EPV>
+__device__ __forceinline__ float ordered_sum(const float (&d)[EPV], int lig)
+{
+    constexpr unsigned ALL = 0xffffffffu;
+    if constexpr (EPV == 4) {
+        const bool b2 = lig & 4, b1 = lig & 2;
+        const float s0 = __shfl_xor_sync(ALL, b2 ? d[0] : d[2], 4);
+        const float s1 = __shfl_xor_sync(ALL, b2 ? d[1] : d[3], 4);
+        const float k0 = (b2 ? d[2] : d[0]) + s0, k1 = (b2 ? d[3] : d[1]) + s1;   // 16
+        float m = (b1 ? k1 : k0) + __shfl_xor_sync(ALL, b1 ? k0 : k1, 2);         // 8
+        m += __shfl_xor_sync(ALL, m, 1);                                          // 4
+        m += __shfl_xor_sync(ALL, m, 4);                                          // 2
+        m += __shfl_xor_sync(ALL, m, 2);                                          // 1
+        return m;
+    } else if constexpr (EPV == 2) {
+        const bool b3 = lig & 8;
+        float m = (b3 ? d[1] : d[0]) + __shfl_xor_sync(ALL, b3 ? d[0] : d[1], 8);   // 16
+        m += __shfl_xor_sync(ALL, m, 4);                                            // 8
+        m += __shfl_xor_sync(ALL, m, 2);                                            // 4
+        m += __shfl_xor_sync(ALL, m, 1);                                            // 2
+        m += __shfl_xor_sync(ALL, m, 8);                                            // 1
+        return m;
+    } else {
+        return warp_allreduce(d[0]);
     }
 }
 
@@ -207,25 +250,38 @@ __device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, 
             continue;
         }
         float d[ND];
+        if constexpr (flex_ordered<MODE, T>()) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            float t = 0.f;
+            for (int u = 0; u < U; ++u) {
+                float de[EPV] = {};
 #pragma unroll
-            for (int e = 0; e < E; ++e) t = fmaf(lrow[e], y[u][e], t);
-            d[u] = t;
-            if constexpr (TWO) {
-                float w = 0.f;
+                for (int v = 0; v < VPL; ++v)
 #pragma unroll
-                for (int e = 0; e < E; ++e)
-                    w = MODE == M_BWD_ROW ? fmaf(hrow[MODE == M_BWD_ROW ? e : 0], y[u][e], w)
-                                          : fmaf(h[MODE == M_BWD_COL ? u : 0][e], lrow[e], w);
-                d[U + u] = w;
+                    for (int e = 0; e < EPV; ++e)
+                        de[e] = fmaf(lrow[v * EPV + e], y[u][v * EPV + e], de[e]);
+                d[u] = ordered_sum<EPV>(de, lig);
             }
-        }
-        for (int off = g >> 1; off > 0; off >>= 1) {
+        } else {
 #pragma unroll
-            for (int i = 0; i < ND; ++i)
-                d[i] += __shfl_xor_sync(0xffffffffu, d[i], off);
+            for (int u = 0; u < U; ++u) {
+                float t = 0.f;
+#pragma unroll
+                for (int e = 0; e < E; ++e) t = fmaf(lrow[e], y[u][e], t);
+                d[u] = t;
+                if constexpr (TWO) {
+                    float w = 0.f;
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        w = MODE == M_BWD_ROW ? fmaf(hrow[MODE == M_BWD_ROW ? e : 0], y[u][e], w)
+                                              : fmaf(h[MODE == M_BWD_COL ? u : 0][e], lrow[e], w);
+                    d[U + u] = w;
+                }
+            }
+            for (int off = g >> 1; off > 0; off >>= 1) {
+#pragma unroll
+                for (int i = 0; i < ND; ++i)
+                    d[i] += __shfl_xor_sync(0xffffffffu, d[i], off);
+            }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -297,13 +353,12 @@ __global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 1
 template <int MODE, typename T, int VB, int E>
 cudaError_t launch_flex_shape(const PassArgs &a, int ng, cudaStream_t st)
 {
-    constexpr int EPV = VB / (int)sizeof(T), VPL = E / EPV;
+    constexpr int EPV = VB / (int)sizeof(T);
     FlexShape sh;
     sh.nvec = a.r / EPV;
-    sh.g = flex_lanes(a.r);
-    static_assert(VPL * EPV == E, "E elements per lane");
+    sh.g = flex_ordered<MODE, T>() ? 32 / EPV : flex_lanes(a.r);
     sh.ng = 1;
-    while (sh.ng < ng && sh.g * sh.ng < 32) sh.ng *= 2;
+    while (!flex_ordered<MODE, T>() && sh.ng < ng && sh.g * sh.ng < 32) sh.ng *= 2;
     const long long total = (long long)a.n_chunks + a.n_light;
     const long long blocks = (total * sh.g * sh.ng + kFlexBlock - 1) / kFlexBlock;
     flex_pass_kernel<MODE, T, VB, E><<<(unsigned)blocks, kFlexBlock, 0, st>>>(a, sh);
@@ -311,14 +366,22 @@ cudaError_t launch_flex_shape(const PassArgs &a, int ng, cudaStream_t st)
 }
 
 // vb: bytes per vector (a power of two up to 16, a multiple of the element
-// size, dividing the row and the alignment of every operand).
+// size, dividing the row and the alignment of every operand).  Roles that
+// keep the generic kernel's order hold 32 elements of a row per vector step,
+// so a lane's E elements cover r <= 32 E / EPV: narrower vectors for wider
+// rows.
 template <int MODE, typename T>
 cudaError_t dispatch_flex(const PassArgs &a, int vb, int ng, cudaStream_t st)
 {
-#define FMM_FLEX(VB)                                                       \
-    if (vb == VB)                                                          \
-        return a.r <= 256 ? launch_flex_shape<MODE, T, VB, 8>(a, ng, st)   \
-                          : launch_flex_shape<MODE, T, VB, 16>(a, ng, st);
+    int e = a.r <= 256 ? 8 : 16;
+    if constexpr (flex_ordered<MODE, T>()) {
+        while (vb > 4 && a.r > 32 * 16 / (vb / 4)) vb /= 2;
+        e = a.r <= 32 * 8 / (vb / 4) ? 8 : 16;
+    }
+#define FMM_FLEX(VB)                                                  \
+    if (vb == VB)                                                     \
+        return e == 8 ? launch_flex_shape<MODE, T, VB, 8>(a, ng, st)  \
+                      : launch_flex_shape<MODE, T, VB, 16>(a, ng, st);
     FMM_FLEX(16)
     FMM_FLEX(8)
     FMM_FLEX(4)

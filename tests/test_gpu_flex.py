@@ -56,3 +56,13 @@ def test_few_rows(m):
     """Fewer rows than one block of groups: every lane group of a team works."""
     S = wl.random_csr(m, 90, np.random.default_rng(m), mean_deg=40, empty_frac=0.0)
     run_all(S, {}, 12, torch.float32, seed=m)
+
+
+@pytest.mark.parametrize("r", [32, 12, 13, 132])
+@pytest.mark.parametrize("hub", [64, 65, 512, 513, 3000])
+def test_sums_of_partial_rows(hub, r):
+    """Rows of 1 to 47 chunks of 64: summed by one warp up to eight chunks,
+    by a block above, several of both kinds in one block."""
+    S = wl.random_csr(300, 280, np.random.default_rng(hub + r), mean_deg=6,
+                      hubs=((0, hub), (1, 700), (2, 100), (299, 600)))
+    run_all(S, {"split_nnz": 64}, r, torch.float32, seed=hub)
