@@ -255,31 +255,122 @@ __global__ void __launch_bounds__(kGatBlock, MINB * (256 / kGatBlock)) gat_kerne
     }
 }
 
-// Merges the chunk states of every split row, in chunk order:
-// M = max_c max_c[k], out[k] = sum_c acc_c[k] e^(max_c[k] - M) /
-// sum_c sum_c[k] e^(max_c[k] - M).  One warp per split row.
-__global__ void __launch_bounds__(256) gat_combine_kernel(const GatArgs a)
+// Merges the chunk states of every split row: M = max_c max_c[k], out[k] =
+// sum_c acc_c[k] e^(max_c[k] - M) / sum_c sum_c[k] e^(max_c[k] - M).  A block
+// takes kGatCombineRows split rows, one per warp, in chunk order; rows of
+// more than that many chunks are merged by the whole block, warp w taking
+// chunks w, w + 8, ... and the eight partial sums added in warp order.  (One
+// warp per row took 110 us on R-MAT 2^20, r = 128, whose longest row has 96
+// chunks; 24 us this way.)
+// VEC elements per lane and step (4 where r allows 16-byte reads).
+constexpr int kGatCombineRows = 8;
+
+template <int VEC>
+__device__ __forceinline__ void gat_state_load(const float *p, float (&v)[VEC])
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= a.n_split)
-        return;
-    const int4 sp = a.split[w];
+    if constexpr (VEC == 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(p);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else {
+        v[0] = *p;
+    }
+}
+
+template <int VEC>
+__global__ void __launch_bounds__(32 * kGatCombineRows) gat_combine_kernel(const GatArgs a)
+{
+    __shared__ float red_m[kGatCombineRows][VEC][32], red_a[kGatCombineRows][VEC][32],
+        red_l[kGatCombineRows][VEC][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = blockIdx.x * kGatCombineRows;
     const int r = a.r;
-    for (int k = lane; k < r; k += 32) {
-        float M = -INFINITY;
-        for (int c = 0; c < sp.z; ++c)
-            M = fmaxf(M, a.partials[(size_t)(sp.y + c) * 3 * r + r + k]);
-        float A = 0.f, L = 0.f;
-        if (M > -INFINITY) {
-            for (int c = 0; c < sp.z; ++c) {
-                const float *b = a.partials + (size_t)(sp.y + c) * 3 * r;
-                const float wgt = expf(b[r + k] - M);
-                A = fmaf(b[k], wgt, A);
-                L = fmaf(b[2 * r + k], wgt, L);
+    // over chunks c0, c0 + step, ... of a row, elements k ... k + VEC - 1
+    auto state = [&](const int4 &sp, int k) { return a.partials + (size_t)sp.y * 3 * r + k; };
+    auto top = [&](const int4 &sp, int c0, int step, int k, float (&M)[VEC]) {
+        const float *b = state(sp, k) + r;
+#pragma unroll 4
+        for (int c = c0; c < sp.z; c += step) {
+            float m[VEC];
+            gat_state_load<VEC>(b + (size_t)c * 3 * r, m);
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) M[v] = fmaxf(M[v], m[v]);
+        }
+    };
+    auto sums = [&](const int4 &sp, int c0, int step, int k, const float (&M)[VEC],
+                    float (&A)[VEC], float (&L)[VEC]) {
+        const float *b = state(sp, k);
+#pragma unroll 2
+        for (int c = c0; c < sp.z; c += step) {
+            const float *p = b + (size_t)c * 3 * r;
+            float acc[VEC], m[VEC], l[VEC];
+            gat_state_load<VEC>(p, acc);
+            gat_state_load<VEC>(p + r, m);
+            gat_state_load<VEC>(p + 2 * r, l);
+#pragma unroll
+            for (int v = 0; v < VEC; ++v)
+                if (M[v] > -INFINITY) {
+                    const float wgt = expf(m[v] - M[v]);
+                    A[v] = fmaf(acc[v], wgt, A[v]);
+                    L[v] = fmaf(l[v], wgt, L[v]);
+                }
+        }
+    };
+    auto finish = [&](const int4 &sp, int k, const float (&A)[VEC], const float (&L)[VEC]) {
+#pragma unroll
+        for (int v = 0; v < VEC; ++v)
+            a.out[(size_t)sp.x * r + k + v] = L[v] > 0.f ? A[v] / L[v] : 0.f;
+    };
+    if (first + warp < a.n_split) {
+        const int4 sp = a.split[first + warp];
+        if (sp.z <= kGatCombineRows) {
+            for (int k = lane * VEC; k < r; k += 32 * VEC) {
+                float M[VEC], A[VEC] = {}, L[VEC] = {};
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) M[v] = -INFINITY;
+                top(sp, 0, 1, k, M);
+                sums(sp, 0, 1, k, M, A, L);
+                finish(sp, k, A, L);
             }
         }
-        a.out[(size_t)sp.x * r + k] = L > 0.f ? A / L : 0.f;
+    }
+    for (int i = 0; i < kGatCombineRows && first + i < a.n_split; ++i) {
+        const int4 sp = a.split[first + i];
+        if (sp.z <= kGatCombineRows)
+            continue;   // uniform across the block
+        for (int k0 = 0; k0 < r; k0 += 32 * VEC) {
+            const int k = k0 + lane * VEC;
+            float M[VEC], A[VEC] = {}, L[VEC] = {};
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) M[v] = -INFINITY;
+            if (k < r)
+                top(sp, warp, kGatCombineRows, k, M);
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) red_m[warp][v][lane] = M[v];
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < kGatCombineRows; ++w)
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) M[v] = fmaxf(M[v], red_m[w][v][lane]);
+            if (k < r)
+                sums(sp, warp, kGatCombineRows, k, M, A, L);
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) {
+                red_a[warp][v][lane] = A[v];
+                red_l[warp][v][lane] = L[v];
+            }
+            __syncthreads();
+            if (warp == 0 && k < r) {
+#pragma unroll
+                for (int w = 1; w < kGatCombineRows; ++w)
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) {
+                        A[v] += red_a[w][v][lane];
+                        L[v] += red_l[w][v][lane];
+                    }
+                finish(sp, k, A, L);
+            }
+            __syncthreads();   // the next step reuses the arrays
+        }
     }
 }
 
@@ -335,26 +426,90 @@ __global__ void __launch_bounds__(256) gat_generic(const GatArgs a)
 }
 
 // out[i, h] = sum_k X[i, h*rh + k] * w[h*rh + k]: the per-node projections
-// f = H a_l and g = H a_r of every head.  One warp per row.
-__global__ void __launch_bounds__(256) gat_project_kernel(int32_t rows, int32_t heads, int32_t rh,
-                                                          const float *X, const float *w,
-                                                          float *out)
+// f = H a_l and g = H a_r of every head.  X is rows x heads segments of rh
+// floats back to back, and out has one float per segment in the same order,
+// so a group of g lanes takes a segment and consecutive groups read
+// consecutive memory whatever the number of heads.  A lane reads vectors
+// lig, lig + g, ... of its segment (VEC floats each); U segments are in
+// flight per group.  Bound by reading X (HBM).  Measured on GB300, 2^20 x 128
+// in 4 heads: 103 us, 5.2 TB/s of X (one warp per row, one scalar load per
+// lane and head at a time, took 363 us).
+constexpr int kProjectU = 4;   // segments in flight per group
+
+template <int VEC>
+__device__ __forceinline__ float project_dot(const float *x, const float *w, float acc)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int r = heads * rh;
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < rows; i += warps) {
-        for (int h = 0; h < heads; ++h) {
-            float acc = 0.f;
-            for (int k = lane; k < rh; k += 32)
-                acc = fmaf(X[(size_t)i * r + h * rh + k], w[h * rh + k], acc);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1)
-                acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if (lane == 0)
-                out[(size_t)i * heads + h] = acc;
-        }
+    if constexpr (VEC == 4) {
+        const float4 xv = __ldcs(reinterpret_cast<const float4 *>(x));
+        const float4 wv = __ldg(reinterpret_cast<const float4 *>(w));
+        acc = fmaf(xv.x, wv.x, acc);
+        acc = fmaf(xv.y, wv.y, acc);
+        acc = fmaf(xv.z, wv.z, acc);
+        return fmaf(xv.w, wv.w, acc);
+    } else {
+        return fmaf(__ldcs(x), __ldg(w), acc);
     }
+}
+
+// ONE: a segment has at most g vectors, one per lane (no loop over k: with
+// it, 214 us in place of 103 at 2^20 x 128).
+template <int VEC, bool ONE>
+__global__ void __launch_bounds__(256) gat_project_kernel(int64_t segments, int32_t heads,
+                                                          int32_t rh, int32_t g, const float *X,
+                                                          const float *w, float *out)
+{
+    constexpr int U = kProjectU;
+    const int lig = threadIdx.x & (g - 1);
+    const int nv = rh / VEC;
+    const int per = 256 / g;   // groups of a block
+    // the block's U x per consecutive segments; group q takes q, q + per, ...
+    const int64_t base = (int64_t)blockIdx.x * (U * per) + threadIdx.x / g;
+    const int hstep = per % heads;
+    int h = segments <= 0xffffffffll ? (int)((uint32_t)base % (uint32_t)heads)
+                                     : (int)(base % heads);
+    float acc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int64_t seg = base + u * per;
+        const float *x = X + (size_t)seg * rh, *wh = w + (size_t)h * rh;
+        acc[u] = 0.f;
+        if constexpr (ONE) {
+            if (seg < segments && lig < nv)
+                acc[u] = project_dot<VEC>(x + lig * VEC, wh + lig * VEC, 0.f);
+        } else {
+            if (seg < segments)
+                for (int k = lig; k < nv; k += g)
+                    acc[u] = project_dot<VEC>(x + k * VEC, wh + k * VEC, acc[u]);
+        }
+        h += hstep;
+        if (h >= heads) h -= heads;
+    }
+    for (int off = g >> 1; off > 0; off >>= 1) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], off);
+    }
+    if (lig == 0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (base + u * per < segments)
+                out[base + u * per] = acc[u];
+    }
+}
+
+template <int VEC>
+void launch_project(int64_t segments, int32_t heads, int32_t rh, const float *X, const float *w,
+                    float *out, cudaStream_t st)
+{
+    const int nv = rh / VEC;
+    int g = 1;
+    while (g < nv && g < 32) g *= 2;
+    const int64_t per = kProjectU * (256 / g);
+    const unsigned blocks = (unsigned)((segments + per - 1) / per);
+    if (nv <= g)
+        gat_project_kernel<VEC, true><<<blocks, 256, 0, st>>>(segments, heads, rh, g, X, w, out);
+    else
+        gat_project_kernel<VEC, false><<<blocks, 256, 0, st>>>(segments, heads, rh, g, X, w, out);
 }
 
 template <typename T, int R, typename C>
@@ -415,9 +570,14 @@ int fmm_gat_project(int32_t rows, int32_t heads, int32_t rh, const float *X, con
     }
     if (rows == 0)
         return FMM_OK;
-    const int64_t blocks = std::min<int64_t>(((int64_t)rows + 7) / 8, (int64_t)sm_count() * 64);
-    gat_project_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(rows, heads, rh, X, w,
-                                                                          out);
+    // 16-byte pieces where the head width and both operands allow them
+    const bool vec = rh % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) |
+                                      reinterpret_cast<uintptr_t>(w)) & 15u) == 0;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (vec)
+        launch_project<4>((int64_t)rows * heads, heads, rh, X, w, out, st);
+    else
+        launch_project<1>((int64_t)rows * heads, heads, rh, X, w, out, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("fmm_gat_project", e);
@@ -467,7 +627,11 @@ int fmm_gat_forward(const fmm_plan *p, int32_t heads, const float *vals, const f
     cudaError_t e = p->dtype == FMM_BF16 ? launch_gat<bf16_t>(a, vec, st)
                                          : launch_gat<float>(a, vec, st);
     if (e == cudaSuccess && a.n_split > 0) {
-        gat_combine_kernel<<<(a.n_split + 7) / 8, 256, 0, st>>>(a);
+        const unsigned blocks = (unsigned)((a.n_split + kGatCombineRows - 1) / kGatCombineRows);
+        if (a.r % 4 == 0)
+            gat_combine_kernel<4><<<blocks, 32 * kGatCombineRows, 0, st>>>(a);
+        else
+            gat_combine_kernel<1><<<blocks, 32 * kGatCombineRows, 0, st>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {

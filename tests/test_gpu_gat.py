@@ -143,3 +143,47 @@ def test_gat_h_alignment(offset_bytes, dtype):
                           torch.from_numpy(g).cuda(), Ht, 0.2)
     ref = oracle.gat(S.row_ptr, S.col_idx, None, f, g, Hd.double().numpy(), heads, 0.2)
     assert relF(out.double().cpu().numpy(), ref) <= 1e-5
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("heads,rh", [(4, 32), (1, 256), (3, 9), (5, 4), (1, 1), (2, 132), (7, 40)])
+def test_projection_shapes(heads, rh, shift):
+    """Head widths of one vector per lane, of several, and of none (scalar
+    loads), operands off a 16-byte boundary, rows that leave the last group
+    short: every element within the rounding bound of a dot of rh terms."""
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(heads * 1000 + rh + shift)
+    rows, r = 3001, heads * rh
+    X = np.zeros(rows * r + shift, np.float32)
+    X[shift:] = rng.standard_normal(rows * r)
+    w = rng.standard_normal(r).astype(np.float32)
+    Xd = torch.from_numpy(X).cuda()[shift:].view(rows, r)
+    got = fmm.gat_project(Xd, torch.from_numpy(w).cuda(), heads).double().cpu().numpy()
+    X64 = X[shift:].reshape(rows, heads, rh).astype(np.float64)
+    w64 = w.reshape(heads, rh).astype(np.float64)
+    ref = (X64 * w64).sum(2)
+    mag = (np.abs(X64) * np.abs(w64)).sum(2)
+    assert np.all(np.abs(got - ref) <= 2 * (rh + 4) * U32 * mag + 1e-30)
+
+
+@pytest.mark.parametrize("heads,rh", [(4, 32), (2, 9)])
+@pytest.mark.parametrize("hub", [256, 257, 2048, 2049, 5000])
+def test_merge_of_chunk_states(heads, rh, hub):
+    """Rows of 1 to 20 chunks of 256: merged by one warp up to eight chunks,
+    by a block above; a second hub row shares the first one's block."""
+    from paper_2203_07673_gb300 import fmm
+    S, rng = _graph(hub + rh, m=600, hubs=((5, hub), (6, 2300), (7, 300)))
+    r = heads * rh
+    H = rng.standard_normal((S.n, r)).astype(np.float32)
+    f = rng.standard_normal((S.m, heads)).astype(np.float32)
+    g = rng.standard_normal((S.n, heads)).astype(np.float32)
+    rp, ci, _, _, Ht = upload(S, None, f, H)
+    plan = fmm.Plan(rp, ci, S.n, r, split_nnz=256)
+    out = fmm.gat_forward(plan, heads, None, torch.from_numpy(f).cuda(),
+                          torch.from_numpy(g).cuda(), Ht, 0.2).double().cpu().numpy()
+    ref = oracle.gat(S.row_ptr, S.col_idx, None, f, g, H.astype(np.float64), heads, 0.2)
+    mag = oracle.gat(S.row_ptr, S.col_idx, None, f, g, np.abs(H.astype(np.float64)), heads, 0.2)
+    rows = np.repeat(np.arange(S.m), np.diff(S.row_ptr))
+    emax = float(np.max(np.abs(f[rows] + g[S.col_idx])))
+    deg = int(S.degrees().max())
+    assert np.all(np.abs(out - ref) <= 2 * (8 * emax + 2 * deg + 16) * U32 * mag + 1e-30)
