@@ -1093,7 +1093,9 @@ def run_batched(args, rank, world, local_rank):
                                    "plans with the library defaults (variant, long-row split)"},
         "e2e": {"value": units_step * world / (e2e_ms / 1e3), "unit": UNIT,
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms},
-        "gpu_launches": 2 * K,
+        # one persistent launch per phase, and one that sums the partial rows of
+        # the R-MAT matrices' hub rows
+        "gpu_launches": 4 * K,
         "clocks": clk,
         "setup": {"generate_s": gen_s, "autotune_s": tune_s, "tuned_groups": len(tuned),
                   "tuned_codes": tuned},

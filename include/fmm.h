@@ -102,7 +102,10 @@ typedef struct fmm_plan_options {
                                  summed in a fixed order; 0 = default:
                                  nnz / (4 x the teams of lanes that run at
                                  once for the kernel variant), clamped to
-                                 [256, 8192]                                  */
+                                 [256, 8192].  With a split_nnz that no row
+                                 (column) exceeds the plan counts as unsplit,
+                                 but its passes still cut rows longer than
+                                 the default size                             */
     int32_t variant;          /* kernel variant of the vectorised row passes:
                                  0 = chosen by the plan; else V*100 + N*10 + U
                                  with V = vectors per lane (as a multiple of
@@ -323,7 +326,8 @@ int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
  *
  * fmm_batch_forward queues a memset of the batch's work counter and one
  * persistent kernel in which warps pop work units (consecutive rows of one
- * matrix, longest rows of all matrices first) until none are left;
+ * matrix, matrix by matrix) until none are left, and, if a matrix has rows
+ * longer than the default split size, a kernel that sums their partial rows;
  * fmm_batch_backward does the same for the adjoint passes (over S: dA, ds;
  * over S^T: dB).  Both can be captured in a CUDA graph.  Each item runs the
  * kernel variant its plan selects (fmm_plan_set_variant), if the batch

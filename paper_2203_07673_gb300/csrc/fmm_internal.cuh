@@ -38,10 +38,13 @@ struct Side {
                                       // length buckets (length_key), index order
                                       // within a bucket
     int32_t n_split = 0;              // rows split into chunks
+    bool split_asked = true;          // whether the rows in chunks are longer than
+                                      // the plan's split_nnz (see build_side)
     int32_t n_light = 0;              // rows - n_split
     int4 *chunks = nullptr;           // {row, begin, end, unused} per chunk
     int32_t n_chunks = 0;
     int4 *split = nullptr;            // {row, first chunk, chunk count, unused}
+    std::vector<int4> split_host;     // host copy of `split`
     int2 *runs = nullptr;             // {first row, end row}: runs of consecutive
                                       // light rows for the streaming pass
     int32_t n_runs = 0;

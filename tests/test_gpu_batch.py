@@ -154,3 +154,47 @@ def test_batch_rejects_split_rows_and_mixed_dtypes():
     assert relF(out.double().cpu().numpy(),
                 oracle.fusedmm(S.row_ptr, S.col_idx, None, A.double().cpu().numpy(),
                                B.double().cpu().numpy(), 40)) <= 1e-5
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("hub", [256, 257, 700, 5000])
+def test_batch_cuts_long_rows(hub, dtype):
+    """Rows and columns around and far above the default split size in a
+    batch: plans that count as unsplit, chunks summed in the batch's own
+    memory, one plan used by two items with different operands, each item
+    bitwise its per-matrix call and within the rounding bound of the oracle."""
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(hub)
+    r = 64
+    S = wl.random_csr(400, 300, rng, mean_deg=6, hubs=((0, hub), (399, hub), (7, 300)))
+    S.col_idx[::3] = 11   # a hub column
+    rp, ci = torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda()
+    plan = fmm.Plan(rp, ci, S.n, r, dtype, split_nnz=1 << 30, variant=112)
+    assert plan.info()["split_rows"] == 0 and plan.info()["split_cols"] == 0
+    items = []
+    for _ in range(2):
+        f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+        items.append(dict(plan=plan, vals=f(S.nnz).abs(), A=f(S.m, r).to(dtype),
+                          B=f(S.n, r).to(dtype), G=f(S.m, r),
+                          out=torch.full((S.m, r), np.nan, device="cuda"),
+                          dA=torch.full((S.m, r), np.nan, device="cuda"),
+                          dB=torch.full((S.n, r), np.nan, device="cuda"),
+                          ds=torch.full((S.nnz,), np.nan, device="cuda")))
+    batch = fmm.Batch(items)
+    batch.forward()
+    batch.backward()
+    deg = max(int(S.degrees().max()), int(np.bincount(S.col_idx, minlength=S.n).max()))
+    for it in items:
+        assert torch.equal(it["out"], fmm.fusedmm(plan, it["vals"], it["A"], it["B"]))
+        g = fmm.fusedmm_bwd(plan, it["vals"], it["A"], it["B"], it["G"])
+        for k, x in zip(("dA", "dB", "ds"), g):
+            assert torch.equal(it[k], x), k
+        a, b, s, gg = (it[k].double().cpu().numpy() for k in ("A", "B", "vals", "G"))
+        ref = [oracle.fusedmm(S.row_ptr, S.col_idx, s, a, b, S.n),
+               *oracle.fusedmm_grad(S.row_ptr, S.col_idx, s, a, b, gg, S.n)]
+        mag = [oracle.fusedmm(S.row_ptr, S.col_idx, s, abs(a), abs(b), S.n),
+               *oracle.fusedmm_grad(S.row_ptr, S.col_idx, s, abs(a), abs(b), abs(gg), S.n)]
+        for k, x, m in zip(("out", "dA", "dB", "ds"), ref, mag):
+            err = np.abs(it[k].double().cpu().numpy() - x)
+            assert np.all(err <= 2 * (2 * r + deg + 4) * U32 * m + 1e-30), k
+    batch.close()
