@@ -252,9 +252,8 @@ int run_pass(const fmm_plan *p, const Side &side, int mode, const float *s, cons
     a.row_ptr = side.row_ptr;
     a.col_idx = side.col_idx;
     a.perm = side.perm;
-    a.order = side.light_order();
     a.n_light = side.n_light;
-    a.chunks = side.chunks;
+    a.items = side.items;
     a.n_chunks = side.n_chunks;
     a.partials = side.partials;
     a.runs = side.runs;

@@ -380,9 +380,8 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
             a.row_ptr = side.row_ptr;
             a.col_idx = side.col_idx;
             a.perm = side.perm;
-            a.order = side.light_order();
             a.n_light = side.n_light;
-            a.chunks = side.chunks;
+            a.items = side.items;
             a.n_chunks = side.n_chunks;
             a.partials = next_partials;
             a.s = s;

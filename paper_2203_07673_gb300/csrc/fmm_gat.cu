@@ -25,11 +25,9 @@
 namespace fmm {
 
 struct GatArgs {
-    const int32_t *row_ptr;
     const int32_t *col_idx;
-    const int32_t *order;     // light rows
+    const int4 *items;        // (row, begin, end): chunks of split rows, light rows
     int32_t n_light;
-    const int4 *chunks;       // chunks of split rows (row, begin, end)
     int32_t n_chunks;
     float *partials;          // per chunk: acc (r), max (r), sum (r)
     const int4 *split;        // split rows (row, first chunk, chunk count)
@@ -151,14 +149,10 @@ __global__ void __launch_bounds__(kGatBlock, MINB * (256 / kGatBlock)) gat_kerne
     const bool active = gid < total;
     int row = 0, beg = 0, end = 0, slot = -1;
     if (active) {
-        if (gid < a.n_chunks) {
-            const int4 c = a.chunks[gid];
-            row = c.x; beg = c.y; end = c.z; slot = (int)gid;
-        } else {
-            row = a.order[gid - a.n_chunks];
-            beg = __ldg(a.row_ptr + row);
-            end = __ldg(a.row_ptr + row + 1);
-        }
+        const int4 c = __ldg(a.items + gid);
+        row = c.x; beg = c.y; end = c.z;
+        if (gid < a.n_chunks)
+            slot = (int)gid;
     }
     const T *H = static_cast<const T *>(a.H);
     const int head = (EPL * lig) / a.rh;
@@ -383,15 +377,9 @@ __global__ void __launch_bounds__(256) gat_generic(const GatArgs a)
     const long long total = (long long)a.n_chunks + a.n_light;
     if (gid >= total)
         return;
-    int row, beg, end, slot = -1;
-    if (gid < a.n_chunks) {
-        const int4 c = a.chunks[gid];
-        row = c.x; beg = c.y; end = c.z; slot = (int)gid;
-    } else {
-        row = a.order[gid - a.n_chunks];
-        beg = __ldg(a.row_ptr + row);
-        end = __ldg(a.row_ptr + row + 1);
-    }
+    const int4 item = __ldg(a.items + gid);
+    const int row = item.x, beg = item.y, end = item.z;
+    const int slot = gid < a.n_chunks ? (int)gid : -1;
     const T *H = static_cast<const T *>(a.H);
     // a chunk accumulates into its partial row, a whole row into out
     float *o = slot >= 0 ? a.partials + (size_t)slot * 3 * a.r : a.out + (size_t)row * a.r;
@@ -602,11 +590,9 @@ int fmm_gat_forward(const fmm_plan *p, int32_t heads, const float *vals, const f
         return FMM_EINVAL;
     }
     GatArgs a;
-    a.row_ptr = p->rows.row_ptr;
     a.col_idx = p->rows.col_idx;
-    a.order = p->rows.light_order();
     a.n_light = p->rows.n_light;
-    a.chunks = p->rows.chunks;
+    a.items = p->rows.items;
     a.n_chunks = p->rows.n_chunks;
     a.partials = p->rows.partials;
     a.split = p->rows.split;

@@ -34,14 +34,18 @@ struct Side {
     const int32_t *row_ptr = nullptr; // rows + 1
     const int32_t *col_idx = nullptr; // nnz
     const int32_t *perm = nullptr;    // nnz; NULL on the S side (identity)
-    int32_t *order = nullptr;         // rows: split rows first, then the rest in
-                                      // length buckets (length_key), index order
-                                      // within a bucket
+    // work items {row, begin, end, unused}: the chunks of split rows, then the
+    // other rows in length buckets (length_key), index order within a bucket.
+    // One 16-byte load per item, consecutive items side by side, in place of
+    // the row's number and then its two row pointers at a random place: one
+    // dependent load less at the start of every row (GB300, bfloat16, r = 64:
+    // R-MAT 2^22 FusedMM 1.33 -> 1.26 ms, adjoint over S 1.96 -> 1.91; Zipf rows,
+    // both products, 2.32 -> 2.27).
+    int4 *items = nullptr;
     int32_t n_split = 0;              // rows split into chunks
     bool split_asked = true;          // whether the rows in chunks are longer than
                                       // the plan's split_nnz (see build_side)
     int32_t n_light = 0;              // rows - n_split
-    int4 *chunks = nullptr;           // {row, begin, end, unused} per chunk
     int32_t n_chunks = 0;
     int4 *split = nullptr;            // {row, first chunk, chunk count, unused}
     std::vector<int4> split_host;     // host copy of `split`
@@ -52,9 +56,9 @@ struct Side {
                                       // the attention pass's softmax states)
     int32_t max_nnz = 0;              // longest row
     KernelVariant variant;            // kernel variant of passes over this side
-    std::vector<int32_t> bucket_start;  // host: first position in `order` of
-                                        // each length key (257 entries)
-    const int32_t *light_order() const { return order ? order + n_split : nullptr; }
+    std::vector<int32_t> bucket_start;  // host: first position of each length key
+                                        // in the row order (split rows, key 0,
+                                        // first; 257 entries)
 };
 
 // Length key of a row for the plan's row order (ascending key = longer rows
@@ -98,9 +102,8 @@ struct PassArgs {
     const int32_t *row_ptr;
     const int32_t *col_idx;
     const int32_t *perm;       // maps a slot of this CSR to the CSR slot of S
-    const int32_t *order;      // light rows in processing order
+    const int4 *items;         // chunks, then light rows in processing order
     int32_t n_light;
-    const int4 *chunks;
     int32_t n_chunks;
     float *partials;
     const int2 *runs = nullptr;  // runs of consecutive light rows (streaming pass)

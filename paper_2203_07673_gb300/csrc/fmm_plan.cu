@@ -227,6 +227,17 @@ __global__ void row_keys_kernel(const int32_t *row_ptr, int32_t rows, int32_t sp
     }
 }
 
+// Work items of the light rows, in order: {row, begin, end, 0}.
+__global__ void row_items_kernel(const int32_t *order, int32_t n, const int32_t *row_ptr,
+                                 int4 *items)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const int32_t row = order[i];
+        items[i] = make_int4(row, row_ptr[row], row_ptr[row + 1], 0);
+    }
+}
+
 __global__ void split_ranges_kernel(const int32_t *order, int32_t n_split, const int32_t *row_ptr,
                                     int2 *ranges)
 {
@@ -424,7 +435,6 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
     side.row_ptr = row_ptr;
     if (rows == 0)
         return FMM_OK;
-    FMM_TRY(dmalloc(&side.order, (size_t)rows, plan), "allocate row order");
     FMM_TRY(cudaMemsetAsync(tmp.counters, 0, 2 * sizeof(int32_t), st), "memset");
     row_keys_kernel<<<blocks_for(rows, 256), 256, 0, st>>>(row_ptr, rows, split_nnz, tmp.ka,
                                                            tmp.va, tmp.counters);
@@ -446,9 +456,8 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
     bool in_b = false;
     FMM_TRY(radix_sort(tmp.ka, tmp.va, tmp.kb, tmp.vb, rows, 8, tmp.ghist, st, &in_b),
             "row order sort");
-    FMM_TRY(cudaMemcpyAsync(side.order, in_b ? tmp.vb : tmp.va, (size_t)rows * sizeof(int32_t),
-                            cudaMemcpyDeviceToDevice, st), "copy row order");
-    // start of every length key in `order`: the scanned digit offsets of the
+    const int32_t *order = reinterpret_cast<const int32_t *>(in_b ? tmp.vb : tmp.va);
+    // start of every length key in the order: the scanned digit offsets of the
     // sort's first tile (entry key * ntiles of the histogram)
     side.bucket_start.assign(257, 0);
     if (rows > 1) {
@@ -482,18 +491,23 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
         if (rc != FMM_OK)
             return rc;
     }
-    if (side.n_split == 0)
+    if (side.n_split == 0) {
+        FMM_TRY(dmalloc(&side.items, (size_t)rows, plan), "allocate work items");
+        row_items_kernel<<<blocks_for(rows, 256, sm_count() * 32), 256, 0, st>>>(order, rows,
+                                                                               row_ptr, side.items);
+        FMM_TRY(cudaGetLastError(), "work items");
         return FMM_OK;
+    }
     int2 *d_ranges = nullptr;
     FMM_TRY(cudaMalloc(&d_ranges, sizeof(int2) * side.n_split), "allocate ranges");
-    split_ranges_kernel<<<blocks_for(side.n_split, 256), 256, 0, st>>>(side.order, side.n_split,
+    split_ranges_kernel<<<blocks_for(side.n_split, 256), 256, 0, st>>>(order, side.n_split,
                                                                        row_ptr, d_ranges);
     std::vector<int2> ranges(side.n_split);
     std::vector<int32_t> rows_h(side.n_split);
     cudaError_t e = cudaMemcpyAsync(ranges.data(), d_ranges, sizeof(int2) * side.n_split,
                                     cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(rows_h.data(), side.order, sizeof(int32_t) * side.n_split,
+        e = cudaMemcpyAsync(rows_h.data(), order, sizeof(int32_t) * side.n_split,
                             cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(st);
@@ -509,13 +523,18 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
         split.push_back(make_int4(rows_h[s], first, (int32_t)chunks.size() - first, 0));
     }
     side.n_chunks = (int32_t)chunks.size();
-    FMM_TRY(dmalloc(&side.chunks, chunks.size(), plan), "allocate chunks");
+    FMM_TRY(dmalloc(&side.items, chunks.size() + side.n_light, plan), "allocate work items");
     FMM_TRY(dmalloc(&side.split, split.size(), plan), "allocate split table");
     // three partial rows per chunk: the FusedMM passes use the first
     // n_chunks x r floats; the attention pass also keeps its running softmax
     // maximum and sum per element there
     FMM_TRY(dmalloc(&side.partials, (size_t)side.n_chunks * r * 3, plan), "allocate partials");
-    FMM_TRY(cudaMemcpyAsync(side.chunks, chunks.data(), sizeof(int4) * chunks.size(),
+    if (side.n_light > 0) {
+        row_items_kernel<<<blocks_for(side.n_light, 256, sm_count() * 32), 256, 0, st>>>(
+            order + side.n_split, side.n_light, row_ptr, side.items + side.n_chunks);
+        FMM_TRY(cudaGetLastError(), "work items");
+    }
+    FMM_TRY(cudaMemcpyAsync(side.items, chunks.data(), sizeof(int4) * chunks.size(),
                             cudaMemcpyHostToDevice, st), "upload chunks");
     FMM_TRY(cudaMemcpyAsync(side.split, split.data(), sizeof(int4) * split.size(),
                             cudaMemcpyHostToDevice, st), "upload split table");
@@ -526,7 +545,7 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
 
 static void free_side(Side &s)
 {
-    cudaFree(s.order); cudaFree(s.chunks); cudaFree(s.split); cudaFree(s.partials);
+    cudaFree(s.items); cudaFree(s.split); cudaFree(s.partials);
     cudaFree(s.runs);
     s = Side();
 }

@@ -140,15 +140,9 @@ __device__ __forceinline__ void nz_store(const PassArgs &a, int slot, float v)
 __device__ __forceinline__ void pass_item(const PassArgs &a, long long gid, int &row,
                                           int &beg, int &end, int &slot)
 {
-    if (gid < a.n_chunks) {
-        const int4 c = a.chunks[gid];
-        row = c.x; beg = c.y; end = c.z; slot = (int)gid;
-    } else {
-        row = a.order[gid - a.n_chunks];
-        beg = __ldg(a.row_ptr + row);
-        end = __ldg(a.row_ptr + row + 1);
-        slot = -1;
-    }
+    const int4 c = __ldg(a.items + gid);
+    row = c.x; beg = c.y; end = c.z;
+    slot = gid < a.n_chunks ? (int)gid : -1;
 }
 
 // Cache operators of the row passes: gathered rows and CSR arrays take the

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256, MB) stream_pass_kernel(const PassArgs a)
     int rend = 0, rend2 = 0;   // end of the current row's nonzeros, of the next row's
     if (active) {
         if (gid < a.n_chunks) {
-            const int4 c = a.chunks[gid];
+            const int4 c = a.items[gid];
             row = c.x; last = c.x + 1; pbeg = c.y; pend = c.z; slot = (int)gid;
             rend = pend; rend2 = pend;
         } else {
