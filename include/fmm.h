@@ -415,10 +415,10 @@ int fmm_gat_project(int32_t rows, int32_t heads, int32_t rh, const float *X, con
  * (NULL = all ones), A (m x r), B (n x r) and out_m (m x r, float32) are as
  * for fmm_plan_create and fmm_fusedmm.  The only scratch is a fixed
  * file-scope device array of 34,603,264 bytes per device (held by every
- * device that loads the library's module until exit): rows longer than
- * ch = max(512, ceil(2 nnz / min(65536, 8388608 / r))) nonzeros are split
- * into chunks whose partial rows live there.  r > 65536 returns
- * FMM_EOVERFLOW.  The array is shared by all calls: calls that overlap on the
+ * device that loads the library's module until exit): the order of the rows
+ * by length, and the partial rows of rows longer than ch nonzeros, which are
+ * split into chunks of ch, at least 128 and more where the array has no room
+ * for that many partial rows.  r > 65536 returns FMM_EOVERFLOW.  The array is shared by all calls: calls that overlap on the
  * GPU race and give wrong results, so order them on one stream.  Every
  * call looks the array's address up (cudaGetSymbolAddress, which allocates
  * nothing) on the current device, so the call still finds it after

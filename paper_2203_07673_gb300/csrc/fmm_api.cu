@@ -66,7 +66,7 @@ int flex_lanes(int32_t r)
 // that divides a row and the alignment of the operands (float32 operands
 // beside bfloat16 rows are read in the same pieces, so an element count of
 // vb / e must keep them aligned as well).
-static int flex_vector_bytes(const PassArgs &a, int dtype)
+int flex_vector_bytes(const PassArgs &a, int dtype)
 {
     const uintptr_t e = dtype == FMM_BF16 ? 2 : 4;
     const uintptr_t rows = reinterpret_cast<uintptr_t>(a.L) | reinterpret_cast<uintptr_t>(a.Y) |
@@ -77,6 +77,19 @@ static int flex_vector_bytes(const PassArgs &a, int dtype)
            ((rows & (vb - 1)) || (f32 & (std::min<uintptr_t>(16, vb / e * 4) - 1))))
         vb /= 2;
     return vb;
+}
+
+// Lane groups per row of the flexible pass: doubled while the launch leaves
+// lanes idle (1024 resident per SM) and every group still has a batch of two
+// nonzeros.
+int flex_groups(const PassArgs &a)
+{
+    const long long items = (long long)a.n_chunks + a.n_light;
+    const long long fill = (long long)sm_count() * 32 * 32;
+    int ng = 1;
+    while (ng < 32 && items * flex_lanes(a.r) * ng * 2 <= fill && items * 4 * ng <= a.nnz)
+        ng *= 2;
+    return ng;
 }
 
 bool variant_known(int code)
@@ -177,15 +190,8 @@ cudaError_t launch_pass(int mode, int dtype, const KernelVariant &v, const PassA
         // a ring layout this width does not have: the team kernel below
     }
     if (!vec && a.r <= kFlexMaxR) {
-        // any other width or alignment: the flexible pass.  Lane groups per
-        // row: doubled while the launch leaves lanes idle (1024 resident per
-        // SM) and every group still has a batch of two nonzeros
-        const long long items = (long long)a.n_chunks + a.n_light;
-        const long long fill = (long long)sm_count() * 32 * 32;   // resident lanes
-        int ng = 1;
-        while (ng < 32 && items * flex_lanes(a.r) * ng * 2 <= fill && items * 4 * ng <= a.nnz)
-            ng *= 2;
-        const int vb = flex_vector_bytes(a, dtype);
+        // any other width or alignment: the flexible pass
+        const int vb = flex_vector_bytes(a, dtype), ng = flex_groups(a);
         return dtype == FMM_BF16 ? launch_flex_bf16(mode, a, vb, ng, st)
                                  : launch_flex_f32(mode, a, vb, ng, st);
     }
@@ -285,7 +291,8 @@ int run_pass(const fmm_plan *p, const Side &side, int mode, const float *s, cons
     if (e == cudaSuccess)
         e = launch_pass(mode, p->dtype, side.variant, a, st);
     if (e == cudaSuccess && mode != M_SDDMM)
-        e = launch_combine(side, out, p->r, accumulate, st);
+        e = launch_combine(side.split, side.n_split, nullptr, side.partials, out, p->r, accumulate,
+                           st);
     if (e != cudaSuccess) {
         set_error("kernel launch", e);
         return FMM_ECUDA;

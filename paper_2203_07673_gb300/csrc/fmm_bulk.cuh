@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256, MB) bulk_pass_kernel(const PassArgs a)
         const bool active = gid < total;
         int row = 0, beg = 0, end = 0, slot = -1;
         if (active)
-            pass_item(a, gid, row, beg, end, slot);
+            pass_item<false>(a, gid, row, beg, end, slot);
 
         float2 l2[E2], acc2[E2];
 #pragma unroll

@@ -155,8 +155,8 @@ __device__ __forceinline__ float ordered_sum(const float (&d)[EPV], int lig)
 
 // Accumulates into acc the nonzeros beg + first, beg + first + step, ... of
 // [beg, end): the share of one group of g lanes (lig = lane within it).
-// Every lane of the warp must call it.
-template <int MODE, typename T, int VB, int E>
+// Every lane of the warp must call it.  ORD: in the generic kernel's order.
+template <int MODE, typename T, int VB, int E, bool ORD, bool CHECK>
 __device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, int end, int first,
                                            int step, int g, int lig, int nvec, float (&acc)[E])
 {
@@ -203,7 +203,7 @@ __device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, 
             jn[u] = -1; sin_[u] = 0; svn[u] = 0.f;
             if (q + u * step < n) {
                 const int pp = beg + (int)(q + u * step);
-                jn[u] = __ldg(a.col_idx + pp);
+                jn[u] = pass_col<CHECK>(a, pp);
                 sin_[u] = (a.perm && (NZ || !a.s_direct)) ? __ldg(a.perm + pp) : pp;
                 svn[u] = a.s ? __ldg(a.s + (a.s_direct ? pp : sin_[u])) : 1.f;
             }
@@ -250,7 +250,7 @@ __device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, 
             continue;
         }
         float d[ND];
-        if constexpr (flex_ordered<MODE, T>()) {
+        if constexpr (ORD) {
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 float de[EPV] = {};
@@ -314,7 +314,7 @@ __device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, 
 // spills).
 constexpr int kFlexBlock = 64;
 
-template <int MODE, typename T, int VB, int E>
+template <int MODE, typename T, int VB, int E, bool ORD = flex_ordered<MODE, T>(), bool CHECK = false>
 __global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 12 : MODE == M_BWD_ROW ? 14 : 16))
     flex_pass_kernel(const PassArgs a, const FlexShape sh)
 {
@@ -324,12 +324,12 @@ __global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 1
     const int lig = lane & (sh.g - 1);
     const int grp = (lane & (team - 1)) / sh.g;
     const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / team;
-    const bool active = gid < (long long)a.n_chunks + a.n_light;
+    bool active = gid < (long long)a.n_chunks + a.n_light;
     int row = 0, beg = 0, end = 0, slot = -1;
     if (active)
-        pass_item(a, gid, row, beg, end, slot);
+        active = pass_item<CHECK>(a, gid, row, beg, end, slot);
     float acc[E];
-    flex_range<MODE, T, VB, E>(a, row, beg, end, grp, sh.ng, sh.g, lig, sh.nvec, acc);
+    flex_range<MODE, T, VB, E, ORD, CHECK>(a, row, beg, end, grp, sh.ng, sh.g, lig, sh.nvec, acc);
     if constexpr (MODE != M_SDDMM) {
         for (int off = sh.g; off < team; off <<= 1) {
 #pragma unroll
@@ -350,18 +350,18 @@ __global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 1
     }
 }
 
-template <int MODE, typename T, int VB, int E>
+template <int MODE, typename T, int VB, int E, bool ORD, bool CHECK>
 cudaError_t launch_flex_shape(const PassArgs &a, int ng, cudaStream_t st)
 {
     constexpr int EPV = VB / (int)sizeof(T);
     FlexShape sh;
     sh.nvec = a.r / EPV;
-    sh.g = flex_ordered<MODE, T>() ? 32 / EPV : flex_lanes(a.r);
+    sh.g = ORD ? 32 / EPV : flex_lanes(a.r);
     sh.ng = 1;
-    while (!flex_ordered<MODE, T>() && sh.ng < ng && sh.g * sh.ng < 32) sh.ng *= 2;
+    while (!ORD && sh.ng < ng && sh.g * sh.ng < 32) sh.ng *= 2;
     const long long total = (long long)a.n_chunks + a.n_light;
     const long long blocks = (total * sh.g * sh.ng + kFlexBlock - 1) / kFlexBlock;
-    flex_pass_kernel<MODE, T, VB, E><<<(unsigned)blocks, kFlexBlock, 0, st>>>(a, sh);
+    flex_pass_kernel<MODE, T, VB, E, ORD, CHECK><<<(unsigned)blocks, kFlexBlock, 0, st>>>(a, sh);
     return cudaGetLastError();
 }
 
@@ -370,18 +370,18 @@ cudaError_t launch_flex_shape(const PassArgs &a, int ng, cudaStream_t st)
 // keep the generic kernel's order hold 32 elements of a row per vector step,
 // so a lane's E elements cover r <= 32 E / EPV: narrower vectors for wider
 // rows.
-template <int MODE, typename T>
+template <int MODE, typename T, bool ORD = flex_ordered<MODE, T>(), bool CHECK = false>
 cudaError_t dispatch_flex(const PassArgs &a, int vb, int ng, cudaStream_t st)
 {
     int e = a.r <= 256 ? 8 : 16;
-    if constexpr (flex_ordered<MODE, T>()) {
+    if constexpr (ORD) {
         while (vb > 4 && a.r > 32 * 16 / (vb / 4)) vb /= 2;
         e = a.r <= 32 * 8 / (vb / 4) ? 8 : 16;
     }
-#define FMM_FLEX(VB)                                                  \
-    if (vb == VB)                                                     \
-        return e == 8 ? launch_flex_shape<MODE, T, VB, 8>(a, ng, st)  \
-                      : launch_flex_shape<MODE, T, VB, 16>(a, ng, st);
+#define FMM_FLEX(VB)                                                              \
+    if (vb == VB)                                                                 \
+        return e == 8 ? launch_flex_shape<MODE, T, VB, 8, ORD, CHECK>(a, ng, st)  \
+                      : launch_flex_shape<MODE, T, VB, 16, ORD, CHECK>(a, ng, st);
     FMM_FLEX(16)
     FMM_FLEX(8)
     FMM_FLEX(4)

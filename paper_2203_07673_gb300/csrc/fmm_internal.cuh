@@ -34,7 +34,7 @@ struct Side {
     const int32_t *row_ptr = nullptr; // rows + 1
     const int32_t *col_idx = nullptr; // nnz
     const int32_t *perm = nullptr;    // nnz; NULL on the S side (identity)
-    // work items {row, begin, end, unused}: the chunks of split rows, then the
+    // work items {row, begin, end, 1}: the chunks of split rows, then the
     // other rows in length buckets (length_key), index order within a bucket.
     // One 16-byte load per item, consecutive items side by side, in place of
     // the row's number and then its two row pointers at a random place: one
@@ -103,6 +103,8 @@ struct PassArgs {
     const int32_t *col_idx;
     const int32_t *perm;       // maps a slot of this CSR to the CSR slot of S
     const int4 *items;         // chunks, then light rows in processing order
+                               // {row, begin, end, w}; w = 0: nothing to do
+                               // (where a pass checks)
     int32_t n_light;
     int32_t n_chunks;
     float *partials;
@@ -122,6 +124,8 @@ struct PassArgs {
                                // bounded wait (NULL: not reported)
     int32_t accumulate = 0;    // 1: out += the pass's rows (else out =)
     int64_t nnz = 0;           // nonzeros of the pattern walked (launch rules)
+    int32_t cols = 0;          // its columns: where a pass checks, an index outside
+                               // [0, cols) counts as no nonzero
 };
 
 // Launches one row pass (main kernel; the combine kernel for split rows is
@@ -140,6 +144,8 @@ cudaError_t launch_flex_bf16(int mode, const PassArgs &a, int vb, int ng, cudaSt
 constexpr int32_t kFlexMaxR = 512;
 // Lanes of one group of the flexible pass for rows of r elements.
 int flex_lanes(int32_t r);
+int flex_vector_bytes(const PassArgs &a, int dtype);
+int flex_groups(const PassArgs &a);
 // Staged forward-role passes (fmm_staged.cuh): FusedMM, SDDMM and SpMM with a
 // cp.async ring of `stages` gathered rows per team; vector path only.
 cudaError_t launch_staged_f32(int mode, int vpl_mult, int stages, const PassArgs &a,
@@ -176,9 +182,12 @@ cudaError_t launch_values_t(const fmm_plan *p, const float *src, float *dst, cud
 // S^T slots per window of the windowed permutation (32 MB of float32 values:
 // a window's staging values stay in L2 while its slots are filled).
 constexpr int64_t kPermuteWindow = int64_t(1) << 23;
-// Sums the partial rows of every split row, in chunk order, into out (added
-// to out's rows when accumulate is set).
-cudaError_t launch_combine(const Side &side, float *out, int32_t r, bool accumulate,
+// Sums the partial rows of every entry {row, first chunk, chunks, unused} of
+// split, in chunk order, into out (added to out's rows when accumulate is
+// set).  n_dev: NULL, or the number of entries on the device (n_split at
+// most).
+cudaError_t launch_combine(const int4 *split, int32_t n_split, const int32_t *n_dev,
+                           const float *partials, float *out, int32_t r, bool accumulate,
                            cudaStream_t st);
 
 bool fast_r(int32_t r);

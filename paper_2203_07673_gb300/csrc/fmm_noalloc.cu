@@ -10,18 +10,33 @@
 // directly.  Its only scratch memory -- the chunk list and partial rows of
 // long rows -- lives in the file-scope device array below, of fixed size.
 //
+// The passes are those a plan picks by default, compiled with the checks that
+// a pattern no plan has validated needs.  What a plan prepares for
+// them is prepared on every call: the work items of the rows in order of
+// length, which one kernel counts per length key and another places (the
+// order within a key is free: a row's result does not depend on it).  With
+// rows of any lengths side by side, a warp and its block wait for their
+// longest row, which costs far more: Zipf(1.2) rows, 200003 x 100003, 4.8M
+// nonzeros, r = 128, bfloat16 (GB300), 810 us with the rows in the caller's
+// order in blocks of 16 rows, 412 with lane groups sharing a row and chunks of
+// 128, 198 in order of length (counting and placing 17, the pass 173).
+//
 // Scratch:  g_noalloc_scratch, 34,603,264 bytes per device (every device that
 // loads this library's module holds it until the process exits):
-//   header   256 B       two counters, cleared at the start of every call
-//   chunks   64 Ki x 16 B  (row, begin, end) of each chunk of a long row
-//   split    64 Ki x 16 B  (row, first chunk, chunk count) of each long row
-//   partials 8 Mi floats   one partial output row per chunk
-// Rows longer than ch nonzeros are split into chunks of ch, where
-// ch = max(512, ceil(2 nnz / cap)) and cap = min(64 Ki, 8 Mi / r): every long
-// row has more than ch nonzeros, so its ceil(deg / ch) chunks number fewer
-// than 2 deg / ch, and all chunks together fewer than 2 nnz / ch <= cap.
-// The partial rows of a long row are summed in chunk order, so results are
-// deterministic.  r may be at most 65536 (FMM_EOVERFLOW otherwise).
+//   header    2304 B          counters: chunks, split rows, rows per length
+//                             key and rows placed per length key
+//   chunks    up to 64 Ki x 16 B  work item of each chunk of a long row
+//   split     as many x 16 B  (row, first chunk, chunk count) of each long row
+//   items     up to 1 Mi x 16 B  work items of a slab of rows
+//   partials  the rest        one partial output row per chunk
+// The header and the chunk slots in use are cleared at the start of a slab.
+// More than 2^20 rows go slab by slab.  Rows longer than ch nonzeros are split
+// into chunks of ch, where ch = max(128, ceil(2 nnz / cap)) and cap = the
+// partial rows there is room for, 64 Ki at most: every long row has more than
+// ch nonzeros, so its ceil(deg / ch) chunks number fewer than 2 deg / ch, and
+// all chunks together fewer than 2 nnz / ch <= cap.  The partial rows of a
+// long row are summed in chunk order, so results are deterministic.  r may be
+// at most 65536 (FMM_EOVERFLOW otherwise).
 //
 // Every call uses the same array: calls that overlap on the GPU (two streams,
 // or two host threads without ordering) race on it and give wrong results.
@@ -29,301 +44,187 @@
 // with cudaGetSymbolAddress on the current device (no allocation); the first
 // call on a device may load the library's module there, so make that first
 // call before any stream capture.
+#include <algorithm>
 #include <cstdio>
 
-#include "fmm_rows.cuh"
+#include "fmm_flex.cuh"
+#include "fmm_pipe.cuh"
+#include "fmm_staged.cuh"
 
 namespace fmm {
 namespace noalloc {
 
 constexpr int32_t MAX_CHUNKS = 1 << 16;
-constexpr int32_t MAX_SPLIT = 1 << 16;
-constexpr int64_t PARTIAL_FLOATS = int64_t(1) << 23;
+constexpr int32_t MAX_SLAB = 1 << 20;
 constexpr int32_t MAX_R = 1 << 16;
-constexpr int32_t MIN_CHUNK = 512;
-constexpr size_t HEADER_BYTES = 256;
-constexpr size_t CHUNKS_OFF = HEADER_BYTES;
-constexpr size_t SPLIT_OFF = CHUNKS_OFF + sizeof(int4) * MAX_CHUNKS;
-constexpr size_t PARTIALS_OFF = SPLIT_OFF + sizeof(int4) * MAX_SPLIT;
-constexpr size_t SCRATCH_BYTES = PARTIALS_OFF + sizeof(float) * PARTIAL_FLOATS;
+constexpr int32_t MIN_CHUNK = 128;
+constexpr size_t SCRATCH_BYTES = 34603264;
 
 struct Header {
     int32_t n_chunks;
     int32_t n_split;
+    int32_t pad[62];
+    int32_t rows[256];      // rows per length key
+    int32_t placed[256];    // of them, placed
 };
+constexpr size_t CHUNKS_OFF = sizeof(Header);
+static_assert(CHUNKS_OFF % 256 == 0, "alignment");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
 
 struct Args {
     const int32_t *row_ptr;
-    const int32_t *col_idx;
-    const float *s;
-    const void *A;
-    const void *B;
-    float *out;
-    int32_t m, n, r, ch;
-    int32_t cap;            // chunk slots usable at this r
+    int32_t first, rows;    // the slab's rows
+    int32_t ch;             // nonzeros per chunk
+    int32_t cap;            // chunk slots (and split entries)
+    int32_t r;
     int64_t nnz;
     Header *hdr;
-    int4 *chunks;
+    int4 *items;            // cap chunk slots, then the rows
     int4 *split;
-    float *partials;
 };
-
-// A chunk descriptor is used only if it lies inside this call's pattern
-// (slots not written by this call hold an earlier call's descriptors).
-__device__ __forceinline__ bool chunk_ok(const Args &a, const int4 c)
-{
-    return c.x >= 0 && c.x < a.m && c.y >= 0 && c.z >= c.y && (int64_t)c.z <= a.nnz;
-}
 
 // Row range of `row`, or an empty range if row_ptr is not consistent there
 // (memory safety only: results for malformed patterns are unspecified).
-__device__ __forceinline__ void row_range(const Args &a, int row, int &beg, int &end)
+__device__ __forceinline__ int2 row_range(const Args &a, int row)
 {
-    beg = __ldg(a.row_ptr + row);
-    end = __ldg(a.row_ptr + row + 1);
-    if (beg < 0 || end < beg || (int64_t)end > a.nnz) {
-        beg = 0;
-        end = 0;
-    }
+    const int beg = __ldg(a.row_ptr + row), end = __ldg(a.row_ptr + row + 1);
+    return beg < 0 || end < beg || (int64_t)end > a.nnz ? make_int2(0, 0) : make_int2(beg, end);
 }
 
-__global__ void setup_kernel(const Args a)
-{
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.m; i += stride) {
-        int beg, end;
-        row_range(a, (int)i, beg, end);
-        if (end - beg <= a.ch)
-            continue;
-        const int nc = (end - beg + a.ch - 1) / a.ch;
-        const int first = atomicAdd(&a.hdr->n_chunks, nc);
-        const int slot = atomicAdd(&a.hdr->n_split, 1);
-        if (slot >= MAX_SPLIT)
-            continue;   // only a malformed pattern gets here; combine stops at MAX_SPLIT
-        if ((int64_t)first + nc > a.cap) {
-            a.split[slot] = make_int4((int)i, 0, 0, 0);   // malformed pattern: row left zero
-            continue;
-        }
-        a.split[slot] = make_int4((int)i, first, nc, 0);
-        for (int c = 0; c < nc; ++c) {
-            const int b = beg + c * a.ch;
-            a.chunks[first + c] = make_int4((int)i, b, (int)min((int64_t)end, (int64_t)b + a.ch), 0);
-        }
-    }
-}
+constexpr int kBlock = 256;
+constexpr int kPerThread = 4;   // rows per thread of the two setup kernels
 
-// The FusedMMA accumulation of nonzeros [beg, end) of `row` into acc (one
-// group of G lanes; every lane of the warp must call it).
-template <typename T, int R, int U>
-__device__ __forceinline__ void fused_range(const Args &a, int row, int beg, int end, bool active,
-                                            int lig, float (&acc)[Shape<T, R>::E])
+// Counts the slab's rows per length key (key 0: long rows) and lists the
+// chunks of the long ones.
+__global__ void __launch_bounds__(kBlock) count_kernel(const Args a)
 {
-    using S = Shape<T, R>;
-    constexpr int G = S::G, E = S::E;
-    const T *A = static_cast<const T *>(a.A);
-    const T *B = static_cast<const T *>(a.B);
-    float lrow[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) { lrow[e] = 0.f; acc[e] = 0.f; }
-    if (active)
-        load_row<T, R, true>(A + (size_t)row * R, lig, lrow);
-    const int iters = active ? (end - beg + U - 1) / U : 0;
-    const int witers = (int)__reduce_max_sync(0xffffffffu, (unsigned)iters);
-    for (int it = 0; it < witers; ++it) {
-        const int p0 = beg + it * U;
-        int jj[U];
-        float sv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int p = p0 + u;
-            jj[u] = -1;
-            sv[u] = 0.f;
-            if (active && p < end) {
-                const int j = __ldg(a.col_idx + p);
-                if (j >= 0 && j < a.n) {
-                    jj[u] = j;
-                    sv[u] = a.s ? __ldg(a.s + p) : 1.f;
-                }
-            }
-        }
-        float y[U][E];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (jj[u] >= 0) {
-                load_row<T, R, false>(B + (size_t)jj[u] * R, lig, y[u]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < E; ++e) y[u][e] = 0.f;
-            }
-        }
-        float d[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            float t = 0.f;
-#pragma unroll
-            for (int e = 0; e < E; ++e) t = fmaf(lrow[e], y[u][e], t);
-            d[u] = t;
-        }
-        group_allreduce<G, U>(d);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (jj[u] < 0) continue;
-            const float c = sv[u] * d[u];
-#pragma unroll
-            for (int e = 0; e < E; ++e) acc[e] = fmaf(c, y[u][e], acc[e]);
-        }
-    }
-}
-
-template <typename T, int R, int U>
-__global__ void __launch_bounds__(256) rows_kernel(const Args a)
-{
-    constexpr int G = Shape<T, R>::G, E = Shape<T, R>::E;
-    const int lig = threadIdx.x & (G - 1);
-    const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    int row = 0, beg = 0, end = 0;
-    bool active = gid < a.m;
-    if (active) {
-        row = (int)gid;
-        row_range(a, row, beg, end);
-        if (end - beg > a.ch)
-            active = false;   // a long row: done by chunks_kernel
-    }
-    float acc[E];
-    fused_range<T, R, U>(a, row, beg, end, active, lig, acc);
-    if (active)
-        store_row_f32<T, R>(a.out + (size_t)row * R, lig, acc);
-}
-
-template <typename T, int R, int U>
-__global__ void __launch_bounds__(256) chunks_kernel(const Args a)
-{
-    constexpr int G = Shape<T, R>::G, E = Shape<T, R>::E;
-    const int lig = threadIdx.x & (G - 1);
-    const int n_chunks = min(a.hdr->n_chunks, a.cap);
-    const long long groups = (long long)gridDim.x * blockDim.x / G;
-    const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const long long rounds = (n_chunks + groups - 1) / groups;   // the same for every warp
-    for (long long rd = 0; rd < rounds; ++rd) {
-        const long long item = rd * groups + gid;
-        bool active = item < n_chunks;
-        int4 c = make_int4(0, 0, 0, 0);
-        if (active) {
-            c = a.chunks[item];
-            if (!chunk_ok(a, c)) {
-                active = false;
-                c = make_int4(0, 0, 0, 0);
-            }
-        }
-        float acc[E];
-        fused_range<T, R, U>(a, c.x, c.y, c.z, active, lig, acc);
-        if (active)
-            store_row_f32<T, R>(a.partials + (size_t)item * R, lig, acc);
-    }
-}
-
-// Any r, any alignment: one warp per row or chunk, the output row
-// accumulated in place (lane k owns columns k, k + 32, ...).
-template <typename T>
-__device__ void generic_range(const Args &a, int row, int beg, int end, float *dst)
-{
+    __shared__ int32_t cnt[256];
+    cnt[threadIdx.x] = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int r = a.r;
-    const T *Ai = static_cast<const T *>(a.A) + (size_t)row * r;
-    const T *B = static_cast<const T *>(a.B);
-    for (int k = lane; k < r; k += 32)
-        dst[k] = 0.f;
-    for (int p = beg; p < end; ++p) {
-        const int j = __ldg(a.col_idx + p);
-        if (j < 0 || j >= a.n)
-            continue;   // uniform across the warp
-        const float sv = a.s ? __ldg(a.s + p) : 1.f;
-        const T *Bj = B + (size_t)j * r;
-        float d = 0.f;
-        for (int k = lane; k < r; k += 32)
-            d = fmaf(widen<T>(Ai[k]), widen<T>(Bj[k]), d);
-        d = warp_allreduce(d);
-        const float c = sv * d;
-        for (int k = lane; k < r; k += 32)
-            dst[k] = fmaf(c, widen<T>(Bj[k]), dst[k]);
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) rows_generic(const Args a)
-{
-    const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= a.m)
-        return;
-    int beg, end;
-    row_range(a, (int)w, beg, end);
-    if (end - beg > a.ch)
-        return;
-    generic_range<T>(a, (int)w, beg, end, a.out + (size_t)w * a.r);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) chunks_generic(const Args a)
-{
-    const int n_chunks = min(a.hdr->n_chunks, a.cap);
-    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; item < n_chunks;
-         item += warps) {
-        const int4 c = a.chunks[item];
-        if (!chunk_ok(a, c))
+#pragma unroll
+    for (int t = 0; t < kPerThread; ++t) {
+        const int64_t i = (int64_t)blockIdx.x * (kBlock * kPerThread) + t * kBlock + threadIdx.x;
+        const int row = a.first + (int)i;
+        int2 p = make_int2(0, 0);
+        int nc = 0;   // chunks of this lane's row
+        if (i < a.rows) {
+            p = row_range(a, row);
+            const uint32_t key = length_key(p.y - p.x, a.ch);
+            atomicAdd(&cnt[key], 1);
+            if (key == 0)
+                nc = (int)(((int64_t)p.y - p.x + a.ch - 1) / a.ch);
+        }
+        // the warp takes its chunk slots and split entries at once
+        const unsigned is_long = __ballot_sync(0xffffffffu, nc > 0);
+        if (!is_long)
             continue;
-        generic_range<T>(a, c.x, c.y, c.z, a.partials + (size_t)item * a.r);
-    }
-}
-
-__global__ void combine_kernel(const Args a)
-{
-    const int n_split = min(a.hdr->n_split, MAX_SPLIT);
-    const int lane = threadIdx.x & 31;
-    const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_split;
-         w += warps) {
-        const int4 sp = a.split[w];
-        if (sp.x < 0 || sp.x >= a.m || sp.y < 0 || sp.z < 0 || (int64_t)sp.y + sp.z > a.cap)
-            continue;
-        for (int k = lane; k < a.r; k += 32) {
-            float acc = 0.f;
-            for (int c = 0; c < sp.z; ++c)
-                acc += a.partials[(size_t)(sp.y + c) * a.r + k];
-            a.out[(size_t)sp.x * a.r + k] = acc;
+        int upto = nc;   // chunks of lanes 0 ... lane
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, upto, off);
+            if (lane >= off) upto += o;
+        }
+        int first = 0, slot = 0;
+        if (lane == 31) {
+            first = atomicAdd(&a.hdr->n_chunks, upto);
+            slot = atomicAdd(&a.hdr->n_split, __popc(is_long));
+        }
+        first = __shfl_sync(0xffffffffu, first, 31) + upto - nc;
+        slot = __shfl_sync(0xffffffffu, slot, 31) + __popc(is_long & ((1u << lane) - 1u));
+        if (nc == 0 || slot >= a.cap)
+            continue;   // (a full table: only a malformed pattern)
+        const bool fits = first >= 0 && (int64_t)first + nc <= a.cap;
+        a.split[slot] = make_int4(row, fits ? first : 0, fits ? nc : 0, 0);
+        for (int c = 0; fits && c < nc; ++c) {
+            const int64_t q = p.x + (int64_t)c * a.ch;
+            a.items[first + c] = make_int4(row, (int)q, (int)min((int64_t)p.y, q + a.ch), 1);
         }
     }
+    __syncthreads();
+    if (cnt[threadIdx.x])
+        atomicAdd(&a.hdr->rows[threadIdx.x], cnt[threadIdx.x]);
 }
 
+// Places the slab's rows in order of their length key.  A block ranks its
+// rows per key in shared memory and takes its places of a key at once.
+__global__ void __launch_bounds__(kBlock) place_kernel(const Args a)
+{
+    __shared__ int32_t cnt[256], base[256];
+    const int tid = threadIdx.x;
+    cnt[tid] = 0;
+    const int mine = a.hdr->rows[tid];
+    base[tid] = mine;
+    __syncthreads();
+    for (int off = 1; off < 256; off <<= 1) {   // inclusive scan of the key counts
+        const int v = tid >= off ? base[tid - off] : 0;
+        __syncthreads();
+        base[tid] += v;
+        __syncthreads();
+    }
+    const int start = base[tid] - mine;   // first place of key tid
+    uint32_t key[kPerThread];
+    int rank[kPerThread], row[kPerThread];
+    int2 p[kPerThread];
+#pragma unroll
+    for (int t = 0; t < kPerThread; ++t) {
+        const int64_t i = (int64_t)blockIdx.x * (kBlock * kPerThread) + t * kBlock + tid;
+        row[t] = -1;
+        if (i < a.rows) {
+            row[t] = a.first + (int)i;
+            p[t] = row_range(a, row[t]);
+            key[t] = length_key(p[t].y - p[t].x, a.ch);
+            rank[t] = atomicAdd(&cnt[key[t]], 1);
+        }
+    }
+    __syncthreads();
+    base[tid] = start + (cnt[tid] ? atomicAdd(&a.hdr->placed[tid], cnt[tid]) : 0);
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kPerThread; ++t)
+        if (row[t] >= 0)   // a long row keeps its place, without work
+            a.items[a.cap + base[key[t]] + rank[t]] =
+                key[t] == 0 ? make_int4(0, 0, 0, 0) : make_int4(row[t], p[t].x, p[t].y, 1);
+}
+
+// The pass over the work items: for vectorised widths the layouts of
+// default_variant (the register ring for bfloat16 rows of r = 64 and 128, the
+// staged pass for float32 rows of r = 128, else the team kernel with 8
+// elements per lane), otherwise the flexible or the generic pass.
 template <typename T, int R>
-void launch_vec(const Args &a, cudaStream_t st)
+cudaError_t launch_width(const PassArgs &p, cudaStream_t st)
 {
-    constexpr int G = Shape<T, R>::G;
-    constexpr int U = Shape<T, R>::E <= 4 ? 8 : 4;
-    const long long blocks = ((long long)a.m * G + 255) / 256;
-    if (blocks > 0)
-        rows_kernel<T, R, U><<<(unsigned)blocks, 256, 0, st>>>(a);
-    chunks_kernel<T, R, U><<<sm_count() * 8, 256, 0, st>>>(a);
+    constexpr int B = base_vpl<T, R>();
+    constexpr int V = sizeof(T) == 4 && R * 4 / 16 <= 32 ? 2 * B : B;   // 8 elements per lane
+    if constexpr (sizeof(T) == 2 && (R == 64 || R == 128)) {
+        if ((reinterpret_cast<uintptr_t>(p.Y) & 31u) == 0)
+            return launch_pipe<M_FUSED, T, R, 2 * B, 1, 2, 2, 1, true>(p, st);
+    }
+    if constexpr (sizeof(T) == 4 && R == 128)
+        return launch_staged<M_FUSED, T, R, V, 4, true>(p, st);
+    else
+        return launch_team<M_FUSED, T, R, V, 1, 2, true>(p, st);
 }
 
 template <typename T>
-void launch_typed(const Args &a, bool vec, cudaStream_t st)
+cudaError_t launch_checked(const PassArgs &p, int dtype, cudaStream_t st)
 {
-    if (vec) {
-        switch (a.r) {
-        case 32: launch_vec<T, 32>(a, st); return;
-        case 64: launch_vec<T, 64>(a, st); return;
-        case 128: launch_vec<T, 128>(a, st); return;
-        case 256: launch_vec<T, 256>(a, st); return;
+    const int vb = flex_vector_bytes(p, dtype);
+    if (vb == 16) {
+        switch (p.r) {
+        case 32: return launch_width<T, 32>(p, st);
+        case 64: return launch_width<T, 64>(p, st);
+        case 128: return launch_width<T, 128>(p, st);
+        case 256: return launch_width<T, 256>(p, st);
         default: break;
         }
     }
-    const long long blocks = ((long long)a.m + 7) / 8;
-    if (blocks > 0)
-        rows_generic<T><<<(unsigned)blocks, 256, 0, st>>>(a);
-    chunks_generic<T><<<sm_count() * 8, 256, 0, st>>>(a);
+    if (p.r <= kFlexMaxR)
+        return dispatch_flex<M_FUSED, T, false, true>(p, vb, flex_groups(p), st);
+    const long long total = (long long)p.n_chunks + p.n_light;
+    row_pass_generic<M_FUSED, T, true><<<(unsigned)((total + 7) / 8), 256, 0, st>>>(p);
+    return cudaGetLastError();
 }
 
 // The array's device address, looked up on every call with the current
@@ -340,8 +241,6 @@ int scratch_base(unsigned char **base)
     *base = static_cast<unsigned char *>(p);
     return FMM_OK;
 }
-
-bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace noalloc
 }  // namespace fmm
@@ -372,37 +271,58 @@ extern "C" int fmm_fusedmm_noalloc(const fmm_csr *S, int32_t r, int32_t dtype, c
     rc = scratch_base(&base);
     if (rc)
         return rc;
-    const int64_t cap = std::min<int64_t>(MAX_CHUNKS, PARTIAL_FLOATS / r);
+    // chunk slots: as many as there is room for beside the items of a slab
+    // (a split entry, an item and a partial row each), at most MAX_CHUNKS
+    const int64_t slab = std::min<int64_t>(S->m, MAX_SLAB);
+    const int64_t room = (int64_t)(SCRATCH_BYTES - CHUNKS_OFF) - 16 * slab - 256;
+    const int64_t cap = std::min<int64_t>(MAX_CHUNKS, room / (2 * (int64_t)sizeof(int4) + 4 * (int64_t)r));
     const int64_t ch = std::max<int64_t>(MIN_CHUNK, (2 * S->nnz + cap - 1) / cap);
     Args a;
     a.row_ptr = S->row_ptr;
-    a.col_idx = S->col_idx;
-    a.s = vals;
-    a.A = A;
-    a.B = B;
-    a.out = out_m;
-    a.m = S->m;
-    a.n = S->n;
-    a.r = r;
     a.ch = (int32_t)std::min<int64_t>(ch, INT32_MAX);
-    a.cap = (int32_t)cap;
+    // slots that this pattern can use
+    a.cap = (int32_t)std::min<int64_t>(cap, 2 * S->nnz / a.ch);
+    a.r = r;
     a.nnz = S->nnz;
     a.hdr = reinterpret_cast<Header *>(base);
-    a.chunks = reinterpret_cast<int4 *>(base + CHUNKS_OFF);
-    a.split = reinterpret_cast<int4 *>(base + SPLIT_OFF);
-    a.partials = reinterpret_cast<float *>(base + PARTIALS_OFF);
+    a.items = reinterpret_cast<int4 *>(base + CHUNKS_OFF);
+    a.split = a.items + a.cap + slab;
+    float *partials = reinterpret_cast<float *>(a.split + a.cap);
+    partials += (-(reinterpret_cast<uintptr_t>(partials) / 4)) & 63;   // 256-byte aligned
+    PassArgs p{};
+    p.row_ptr = S->row_ptr;
+    p.col_idx = S->col_idx;
+    p.items = a.items;
+    p.n_chunks = a.cap;
+    p.partials = partials;
+    p.s = vals;
+    p.s_direct = 1;
+    p.L = A;
+    p.Y = B;
+    p.out = out_m;
+    p.r = r;
+    p.nnz = S->nnz;
+    p.cols = S->n;
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(base, 0, HEADER_BYTES, st);
-    if (e == cudaSuccess) {
-        const long long blocks = std::min<long long>(((long long)S->m + 255) / 256, (long long)sm_count() * 16);
-        setup_kernel<<<(unsigned)blocks, 256, 0, st>>>(a);
-        const bool vec = fast_r(r) && aligned16(A) && aligned16(B) && aligned16(out_m);
-        if (dtype == FMM_BF16)
-            launch_typed<bf16_t>(a, vec, st);
-        else
-            launch_typed<float>(a, vec, st);
-        combine_kernel<<<sm_count() * 4, 256, 0, st>>>(a);
-        e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    for (int64_t first = 0; first < S->m && e == cudaSuccess; first += slab) {
+        a.first = (int32_t)first;
+        a.rows = (int32_t)std::min<int64_t>(slab, S->m - first);
+        p.n_light = a.rows;
+        const unsigned blocks = (unsigned)((a.rows + kBlock * kPerThread - 1) / (kBlock * kPerThread));
+        e = cudaMemsetAsync(base, 0, CHUNKS_OFF + sizeof(int4) * (size_t)a.cap, st);
+        if (e != cudaSuccess)
+            break;
+        count_kernel<<<blocks, kBlock, 0, st>>>(a);
+        place_kernel<<<blocks, kBlock, 0, st>>>(a);
+        e = dtype == FMM_BF16 ? launch_checked<bf16_t>(p, dtype, st)
+                              : launch_checked<float>(p, dtype, st);
+        if (e == cudaSuccess && a.cap > 0) {
+            // a long row has two chunks at least
+            e = launch_combine(a.split, a.cap / 2 + 1, &a.hdr->n_split, partials, out_m, r, false, st);
+        }
+        if (e == cudaSuccess)
+            e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
         set_error("fmm_fusedmm_noalloc launch", e);

@@ -87,7 +87,7 @@ constexpr int kPipeBlock = 32;
 // as 256 / kPipeBlock blocks each (a register cap of 65536 / (256 MB) per
 // thread): the register ring trades rows in flight per team against teams
 // per SM.
-template <int MODE, typename T, int R, int VPL, int U, int RING, int MB, int REFILL>
+template <int MODE, typename T, int R, int VPL, int U, int RING, int MB, int REFILL, bool CHECK = false>
 __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass_kernel(const PassArgs a)
 {
     static_assert(MODE >= M_FUSED && MODE <= M_BWD_COL, "role");
@@ -115,12 +115,12 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
     auto widx = [lig](int v) { return WIDE ? lig * VPL + v : v * G + lig; };
     const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
     const long long total = (long long)a.n_chunks + a.n_light;
-    const bool active = gid < total;
+    bool active = gid < total;
     const Loader ld;
 
     int row = 0, beg = 0, end = 0, slot = -1;
     if (active)
-        pass_item(a, gid, row, beg, end, slot);
+        active = pass_item<CHECK>(a, gid, row, beg, end, slot);
     const T *L = static_cast<const T *>(a.L);
     const T *Y = static_cast<const T *>(a.Y);
 
@@ -177,10 +177,12 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
             j[e] = -1; s[e] = 0.f; si[e] = -1;
             if (q < n) {
                 const int p = beg + q;
-                j[e] = ld.idx(a.col_idx + p);
+                j[e] = pass_col<CHECK>(a, p);
                 const int sp = (a.perm && (NZ || !a.s_direct)) ? ld.idx(a.perm + p) : p;
                 si[e] = sp;
                 s[e] = a.s ? ld.val(a.s + (a.s_direct ? p : sp)) : 1.f;
+                if (CHECK && j[e] < 0)
+                    s[e] = 0.f;   // its row reads as zeros
             }
         }
     };
@@ -408,13 +410,13 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
     }
 }
 
-template <int MODE, typename T, int R, int VPL, int U, int RING, int MB, int REFILL>
+template <int MODE, typename T, int R, int VPL, int U, int RING, int MB, int REFILL, bool CHECK = false>
 cudaError_t launch_pipe(const PassArgs &a, cudaStream_t st)
 {
     constexpr int G = TeamShape<T, R, VPL, 1>::G;
     const long long total = (long long)a.n_chunks + a.n_light;
     const long long blocks = (total * G + kPipeBlock - 1) / kPipeBlock;
-    pipe_pass_kernel<MODE, T, R, VPL, U, RING, MB, REFILL><<<(unsigned)blocks, kPipeBlock, 0, st>>>(a);
+    pipe_pass_kernel<MODE, T, R, VPL, U, RING, MB, REFILL, CHECK><<<(unsigned)blocks, kPipeBlock, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -227,14 +227,14 @@ __global__ void row_keys_kernel(const int32_t *row_ptr, int32_t rows, int32_t sp
     }
 }
 
-// Work items of the light rows, in order: {row, begin, end, 0}.
+// Work items of the light rows, in order: {row, begin, end, 1}.
 __global__ void row_items_kernel(const int32_t *order, int32_t n, const int32_t *row_ptr,
                                  int4 *items)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const int32_t row = order[i];
-        items[i] = make_int4(row, row_ptr[row], row_ptr[row + 1], 0);
+        items[i] = make_int4(row, row_ptr[row], row_ptr[row + 1], 1);
     }
 }
 
@@ -519,7 +519,7 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
         const int32_t first = (int32_t)chunks.size();
         for (int64_t c = beg; c < end; c += split_nnz)
             chunks.push_back(make_int4(rows_h[s], (int32_t)c,
-                                       (int32_t)std::min<int64_t>(end, c + split_nnz), 0));
+                                       (int32_t)std::min<int64_t>(end, c + split_nnz), 1));
         split.push_back(make_int4(rows_h[s], first, (int32_t)chunks.size() - first, 0));
     }
     side.n_chunks = (int32_t)chunks.size();
@@ -878,12 +878,14 @@ constexpr int kCombineLoads = 16;
 
 template <int VEC>
 __global__ void __launch_bounds__(128) combine_kernel(const int4 *split, int32_t n_split,
-                                                      int32_t tiles, const float *partials,
-                                                      float *out, int32_t r, int32_t accumulate)
+                                                      const int32_t *n_dev, int32_t tiles,
+                                                      const float *partials, float *out, int32_t r,
+                                                      int32_t accumulate)
 {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= (int64_t)n_split * tiles)
+    const int32_t n = n_dev ? min(*n_dev, n_split) : n_split;
+    if (w >= (int64_t)n * tiles)
         return;
     const int4 sp = split[w / tiles];
     const int k = ((int)(w % tiles) * 32 + lane) * VEC;
@@ -918,17 +920,18 @@ __global__ void __launch_bounds__(128) combine_kernel(const int4 *split, int32_t
     for (int v = 0; v < VEC; ++v) o[v] = accumulate ? o[v] + acc[v] : acc[v];
 }
 
-cudaError_t launch_combine(const Side &side, float *out, int32_t r, bool accumulate,
+cudaError_t launch_combine(const int4 *split, int32_t n_split, const int32_t *n_dev,
+                           const float *partials, float *out, int32_t r, bool accumulate,
                            cudaStream_t st)
 {
-    if (side.n_split == 0 || !out)
+    if (n_split == 0 || !out)
         return cudaSuccess;
     // partial rows start 16-byte aligned when r is a multiple of 4
     const int vec = r % 4 == 0 ? 4 : 1;
     const int32_t tiles = (r + 32 * vec - 1) / (32 * vec);
-    const unsigned blocks = (unsigned)(((int64_t)side.n_split * tiles + 3) / 4);
+    const unsigned blocks = (unsigned)(((int64_t)n_split * tiles + 3) / 4);
     auto *kernel = vec == 4 ? combine_kernel<4> : combine_kernel<1>;
-    kernel<<<blocks, 128, 0, st>>>(side.split, side.n_split, tiles, side.partials, out, r,
+    kernel<<<blocks, 128, 0, st>>>(split, n_split, n_dev, tiles, partials, out, r,
                                    accumulate ? 1 : 0);
     return cudaGetLastError();
 }

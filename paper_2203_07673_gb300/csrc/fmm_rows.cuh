@@ -137,12 +137,27 @@ __device__ __forceinline__ void nz_store(const PassArgs &a, int slot, float v)
 
 // Work item of group `gid`: chunks of split rows first, then light rows in
 // plan order.  slot >= 0 marks a chunk (its partial row goes to partials).
-__device__ __forceinline__ void pass_item(const PassArgs &a, long long gid, int &row,
+// CHECK (patterns that no plan has validated): false for an item without
+// work.  Compiled in only there: the test of a column index alone took the
+// register-ring pass from 2.27 to 2.83 ms on the Zipf rows, both products.
+template <bool CHECK>
+__device__ __forceinline__ bool pass_item(const PassArgs &a, long long gid, int &row,
                                           int &beg, int &end, int &slot)
 {
     const int4 c = __ldg(a.items + gid);
     row = c.x; beg = c.y; end = c.z;
     slot = gid < a.n_chunks ? (int)gid : -1;
+    return !CHECK || c.w != 0;
+}
+
+// Column index of slot p; CHECK: -1 if it is out of range.
+template <bool CHECK>
+__device__ __forceinline__ int pass_col(const PassArgs &a, int p)
+{
+    const int j = __ldg(a.col_idx + p);
+    if constexpr (CHECK)
+        return (unsigned)j < (unsigned)a.cols ? j : -1;
+    return j;
 }
 
 // Cache operators of the row passes: gathered rows and CSR arrays take the
@@ -252,7 +267,7 @@ __device__ __forceinline__ void team_store_f32(const Loader &ld, float *row, int
 //
 // team_pass_body does the work of team `gid` (every lane of the warp must
 // call it; lanes whose team is not active only join the shuffles).
-template <int MODE, typename T, int R, int VPL, int NG, int U>
+template <int MODE, typename T, int R, int VPL, int NG, int U, bool CHECK = false>
 __device__ __forceinline__ void team_pass_body(const PassArgs &a, long long gid, bool active)
 {
     using TS = TeamShape<T, R, VPL, NG>;
@@ -270,7 +285,7 @@ __device__ __forceinline__ void team_pass_body(const PassArgs &a, long long gid,
 
     int row = 0, beg = 0, end = 0, slot = -1;
     if (active)
-        pass_item(a, gid, row, beg, end, slot);
+        active = pass_item<CHECK>(a, gid, row, beg, end, slot);
 
     const T *L = static_cast<const T *>(a.L);
     const T *Y = static_cast<const T *>(a.Y);
@@ -399,7 +414,7 @@ __device__ __forceinline__ void team_pass_body(const PassArgs &a, long long gid,
             int myj = -1, mysi = 0;
             float mys = 0.f;
             if (q < end) {
-                myj = ld.idx(a.col_idx + q);
+                myj = pass_col<CHECK>(a, q);
                 // the slot in S order is needed for per-nonzero outputs and
                 // for values not yet in this CSR's order
                 mysi = (a.perm && (NZ || !a.s_direct)) ? ld.idx(a.perm + q) : q;
@@ -434,7 +449,7 @@ __device__ __forceinline__ void team_pass_body(const PassArgs &a, long long gid,
             for (int u = 0; u < U; ++u) {
                 const int p = p0 + u * NG;
                 if (p < end) {
-                    jj[u] = ld.idx(a.col_idx + p);
+                    jj[u] = pass_col<CHECK>(a, p);
                     sidx[u] = (a.perm && (NZ || !a.s_direct)) ? ld.idx(a.perm + p) : p;
                     sv[u] = a.s ? ld.val(a.s + (a.s_direct ? p : sidx[u])) : 1.f;
                 } else {
@@ -487,7 +502,7 @@ constexpr int team_min_blocks()
 // meaning: 256 / kTeamBlock blocks per 256 threads.
 constexpr int kTeamBlock = 64;
 
-template <int MODE, typename T, int R, int VPL, int NG, int U>
+template <int MODE, typename T, int R, int VPL, int NG, int U, bool CHECK = false>
 __global__ void __launch_bounds__(kTeamBlock,
                                   (256 / kTeamBlock) * (team_min_blocks<MODE, T, R, VPL, NG, U>()))
     team_pass_kernel(const PassArgs a)
@@ -495,7 +510,7 @@ __global__ void __launch_bounds__(kTeamBlock,
     constexpr int TEAM = TeamShape<T, R, VPL, NG>::TEAM;
     const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / TEAM;
     const long long total = (long long)a.n_chunks + a.n_light;
-    team_pass_body<MODE, T, R, VPL, NG, U>(a, gid, gid < total);
+    team_pass_body<MODE, T, R, VPL, NG, U, CHECK>(a, gid, gid < total);
 }
 
 template <typename T> __device__ __forceinline__ float widen(T x);
@@ -517,7 +532,7 @@ __device__ __forceinline__ float warp_allreduce(float v)
 // any alignment: one warp per row or chunk,
 // scalar loads strided by lane, the output row accumulated in place (each
 // lane owns the columns k = lane + 32 t, so no two lanes touch one word).
-template <int MODE, typename T>
+template <int MODE, typename T, bool CHECK = false>
 __global__ void __launch_bounds__(256) row_pass_generic(const PassArgs a)
 {
     constexpr bool ACC = MODE != M_SDDMM;
@@ -527,7 +542,8 @@ __global__ void __launch_bounds__(256) row_pass_generic(const PassArgs a)
     if (gid >= total)
         return;   // uniform per warp
     int row, beg, end, slot;
-    pass_item(a, gid, row, beg, end, slot);
+    if (!pass_item<CHECK>(a, gid, row, beg, end, slot))
+        return;
     const int r = a.r;
     const T *L = static_cast<const T *>(a.L);
     const T *Y = static_cast<const T *>(a.Y);
@@ -541,7 +557,9 @@ __global__ void __launch_bounds__(256) row_pass_generic(const PassArgs a)
             dst[k] = 0.f;
     const T *Li = L ? L + (size_t)row * r : nullptr;
     for (int p = beg; p < end; ++p) {
-        const int j = __ldg(a.col_idx + p);
+        const int j = pass_col<CHECK>(a, p);
+        if (CHECK && j < 0)
+            continue;   // uniform across the warp
         const int sidx = a.perm ? __ldg(a.perm + p) : p;
         const float sv = a.s ? __ldg(a.s + (a.s_direct ? p : sidx)) : 1.f;
         const T *Yj = Y + (size_t)j * r;
@@ -595,13 +613,13 @@ struct Variant {
     int vpl, ng, u;
 };
 
-template <int MODE, typename T, int R, int VPL, int NG, int U>
+template <int MODE, typename T, int R, int VPL, int NG, int U, bool CHECK = false>
 cudaError_t launch_team(const PassArgs &a, cudaStream_t st)
 {
     constexpr int TEAM = TeamShape<T, R, VPL, NG>::TEAM;
     const long long total = (long long)a.n_chunks + a.n_light;
     const long long blocks = (total * TEAM + kTeamBlock - 1) / kTeamBlock;
-    team_pass_kernel<MODE, T, R, VPL, NG, U><<<(unsigned)blocks, kTeamBlock, 0, st>>>(a);
+    team_pass_kernel<MODE, T, R, VPL, NG, U, CHECK><<<(unsigned)blocks, kTeamBlock, 0, st>>>(a);
     return cudaGetLastError();
 }
 

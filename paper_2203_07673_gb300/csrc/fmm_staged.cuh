@@ -55,7 +55,7 @@ __device__ __forceinline__ void stage_read(const uint4 *ring, int st, int tid, f
     }
 }
 
-template <int MODE, typename T, int R, int VPL, int D>
+template <int MODE, typename T, int R, int VPL, int D, bool CHECK = false>
 __global__ void __launch_bounds__(256) staged_pass_kernel(const PassArgs a)
 {
     static_assert(MODE == M_FUSED || MODE == M_SDDMM || MODE == M_SPMM, "forward roles");
@@ -75,12 +75,12 @@ __global__ void __launch_bounds__(256) staged_pass_kernel(const PassArgs a)
     const int tbase = lane & ~(G - 1);
     const long long gid = ((long long)blockIdx.x * blockDim.x + tid) / G;
     const long long total = (long long)a.n_chunks + a.n_light;
-    const bool active = gid < total;
+    bool active = gid < total;
     const Loader ld;
 
     int row = 0, beg = 0, end = 0, slot = -1;
     if (active)
-        pass_item(a, gid, row, beg, end, slot);
+        active = pass_item<CHECK>(a, gid, row, beg, end, slot);
     const T *L = static_cast<const T *>(a.L);
     const T *Y = static_cast<const T *>(a.Y);
     float lrow[E], acc[E];
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256) staged_pass_kernel(const PassArgs a)
             j[e] = -1; s[e] = 0.f; si[e] = 0;
             if (q < n) {
                 const int p = beg + q;
-                j[e] = ld.idx(a.col_idx + p);
+                j[e] = pass_col<CHECK>(a, p);
                 // the slot in S order: for per-nonzero outputs, and for
                 // values not yet in this CSR's order
                 const int sp = (a.perm && (NZ || !a.s_direct)) ? ld.idx(a.perm + p) : p;
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(256) staged_pass_kernel(const PassArgs a)
     }
 }
 
-template <int MODE, typename T, int R, int VPL, int D>
+template <int MODE, typename T, int R, int VPL, int D, bool CHECK = false>
 cudaError_t launch_staged(const PassArgs &a, cudaStream_t st)
 {
     constexpr int G = TeamShape<T, R, VPL, 1>::G;
@@ -208,7 +208,7 @@ cudaError_t launch_staged(const PassArgs &a, cudaStream_t st)
             return e;
         const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
         if (!bit || !(done.load() & bit)) {
-            e = cudaFuncSetAttribute(staged_pass_kernel<MODE, T, R, VPL, D>,
+            e = cudaFuncSetAttribute(staged_pass_kernel<MODE, T, R, VPL, D, CHECK>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess)
                 return e;
@@ -217,7 +217,7 @@ cudaError_t launch_staged(const PassArgs &a, cudaStream_t st)
     }
     const long long total = (long long)a.n_chunks + a.n_light;
     const long long blocks = (total * G + 255) / 256;
-    staged_pass_kernel<MODE, T, R, VPL, D><<<(unsigned)blocks, 256, smem, st>>>(a);
+    staged_pass_kernel<MODE, T, R, VPL, D, CHECK><<<(unsigned)blocks, 256, smem, st>>>(a);
     return cudaGetLastError();
 }
 
