@@ -176,8 +176,29 @@ cudaError_t launch_pipe_bf16(int mode, int vpl_mult, int u, int ring, int mb, in
 // dst[q] = src[perm[q]] for q < nnz (values of S into the order of S^T).
 cudaError_t launch_permute(const float *src, const int32_t *perm, float *dst, int64_t nnz,
                            cudaStream_t st);
-// Values of S in the order of S^T for a plan: the windowed two-pass
-// permutation where the plan has it, else launch_permute.
+// The permutation through shared memory (fmm_values.cu): tiles of W values on
+// both sides.
+struct ValueTiles {
+    int32_t W = 0, tiles = 0;     // 0: the plan has none
+    uint16_t *pos1 = nullptr;     // nnz: place of each value of S in its tile's runs
+    uint16_t *pos2 = nullptr;     // nnz: slot of each staged value in its S^T tile
+    uint32_t *first = nullptr;    // tiles x W / 32: a bit at the first value of a run
+    uint16_t *before = nullptr;   // tiles x W / 32: runs that start before these 32
+    int32_t *run = nullptr;       // tiles x tiles: by run, staging place - tile place
+    float *stage = nullptr;       // nnz
+};
+constexpr int32_t kTileValuesMax = 49152;   // 192 KB of shared memory
+constexpr int32_t kTilesMax = 512 * 11;
+// Tile size for a pattern, 0 = not through shared memory.
+int32_t values_tile(int64_t nnz);
+// Fills v's tables (allocated by the caller) from perm (S^T slot -> S slot);
+// inv: scratch, nnz words.
+cudaError_t build_value_tiles(ValueTiles &v, const int32_t *perm, int64_t nnz, uint32_t *inv,
+                              cudaStream_t st);
+cudaError_t launch_value_tiles(const ValueTiles &v, const float *src, float *dst, int64_t nnz,
+                               cudaStream_t st);
+// Values of S in the order of S^T for a plan: through shared memory or the
+// windowed two-pass permutation where the plan has it, else launch_permute.
 cudaError_t launch_values_t(const fmm_plan *p, const float *src, float *dst, cudaStream_t st);
 // S^T slots per window of the windowed permutation (32 MB of float32 values:
 // a window's staging values stay in L2 while its slots are filled).
@@ -240,6 +261,7 @@ struct fmm_plan {
     // windowed value permutation (plans with more than 2 windows of
     // nonzeros): S-order slot p -> its place in the window staging array,
     // S^T slot q -> where its value waits there, and the staging array
+    fmm::ValueTiles tiles;
     int32_t *win_pos1 = nullptr;
     int32_t *win_pos2 = nullptr;
     float *win_tmp = nullptr;

@@ -605,6 +605,12 @@ void destroy_plan(fmm_plan *p)
     cudaFree(p->perm_t);
     cudaFree(p->vals_t);
     cudaFree(p->vals_static);
+    cudaFree(p->tiles.pos1);
+    cudaFree(p->tiles.pos2);
+    cudaFree(p->tiles.first);
+    cudaFree(p->tiles.before);
+    cudaFree(p->tiles.run);
+    cudaFree(p->tiles.stage);
     cudaFree(p->win_pos1);
     cudaFree(p->win_pos2);
     cudaFree(p->win_tmp);
@@ -683,7 +689,19 @@ int create_plan(const fmm_csr *S, int32_t r, int32_t dtype, const fmm_plan_optio
             PLAN_TRY(cudaGetLastError(), "transpose rows");
         }
         PLAN_TRY(dmalloc(&p->vals_t, (size_t)S->nnz, p), "allocate S^T values");
-        if (S->nnz > 2 * kPermuteWindow) {
+        if (const int32_t W = values_tile(S->nnz); W > 0 && S->nnz > 0) {
+            ValueTiles &v = p->tiles;
+            const int64_t tiles = (S->nnz + W - 1) / W;
+            PLAN_TRY(dmalloc(&v.pos1, (size_t)S->nnz, p), "allocate value places");
+            PLAN_TRY(dmalloc(&v.pos2, (size_t)S->nnz, p), "allocate value places");
+            PLAN_TRY(dmalloc(&v.first, (size_t)tiles * (W / 32), p), "allocate value runs");
+            PLAN_TRY(dmalloc(&v.before, (size_t)tiles * (W / 32), p), "allocate value runs");
+            PLAN_TRY(dmalloc(&v.run, (size_t)(tiles * tiles), p), "allocate value runs");
+            PLAN_TRY(dmalloc(&v.stage, (size_t)S->nnz, p), "allocate staged values");
+            v.W = W;
+            v.tiles = (int32_t)tiles;
+            PLAN_TRY(build_value_tiles(v, p->perm_t, S->nnz, tmp.ka, st), "value tiles");
+        } else if (S->nnz > 2 * kPermuteWindow) {
             // the windowed value permutation (launch_values_t)
             const int64_t P = kPermuteWindow;
             const int64_t W = (S->nnz + P - 1) / P;
@@ -856,6 +874,8 @@ cudaError_t launch_values_t(const fmm_plan *p, const float *src, float *dst, cud
 {
     if (p->nnz == 0 || !src)
         return cudaSuccess;
+    if (p->tiles.W)
+        return launch_value_tiles(p->tiles, src, dst, p->nnz, st);
     if (!p->win_pos1)
         return launch_permute(src, p->perm_t, dst, p->nnz, st);
     const int64_t per_block = kPermuteBlock * kPermutePerThread;
