@@ -280,6 +280,17 @@ int fmm_fusedmm_t_bwd(const fmm_plan *plan, const float *vals, const void *A,
                       float *ds, fmm_stream stream);
 
 /*
+ * The adjoints with dA (m x r) and dB (n x r) in the plan's dtype: bfloat16
+ * plans get the float32 results rounded once (nearest even) as they are
+ * stored, without a pass over float32 gradients.  ds stays float32.
+ * bfloat16 plans of r > 512 return FMM_EUNSUPPORTED.
+ */
+int fmm_fusedmm_bwd_typed(const fmm_plan *plan, const float *vals, const void *A, const void *B,
+                          const float *G, void *dA, void *dB, float *ds, fmm_stream stream);
+int fmm_fusedmm_t_bwd_typed(const fmm_plan *plan, const float *vals, const void *A, const void *B,
+                            const float *Gn, void *dA, void *dB, float *ds, fmm_stream stream);
+
+/*
  * Accumulating forms, the "+=" of the distributed algorithms (Algorithm 1:
  * each phase adds the contribution of one column block of S to the rows it
  * owns): out_m += FusedMMA, out_n += FusedMMB, dA += and dB += the adjoint

@@ -35,7 +35,10 @@ class FusedMMFunction(torch.autograd.Function):
                 vals is not None and ctx.needs_input_grad[1])
         if not any(need):
             return None, None, None, None, None
-        fn = fmm.fusedmm_t_bwd if ctx.transpose else fmm.fusedmm_bwd
+        if ctx.plan.r <= 512:   # gradients rounded to A's dtype as they are stored
+            fn = fmm.fusedmm_t_bwd_typed if ctx.transpose else fmm.fusedmm_bwd_typed
+        else:
+            fn = fmm.fusedmm_t_bwd if ctx.transpose else fmm.fusedmm_bwd
         dA, dB, ds = fn(ctx.plan, vals, A, B, G, need)
         if dA is not None and dA.dtype != A.dtype:
             dA = dA.to(A.dtype)

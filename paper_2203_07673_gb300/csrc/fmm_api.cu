@@ -70,7 +70,7 @@ int flex_vector_bytes(const PassArgs &a, int dtype)
 {
     const uintptr_t e = dtype == FMM_BF16 ? 2 : 4;
     const uintptr_t rows = reinterpret_cast<uintptr_t>(a.L) | reinterpret_cast<uintptr_t>(a.Y) |
-                           ((uintptr_t)a.r * e);
+                           reinterpret_cast<uintptr_t>(a.out16) | ((uintptr_t)a.r * e);
     const uintptr_t f32 = reinterpret_cast<uintptr_t>(a.H) | reinterpret_cast<uintptr_t>(a.out);
     int vb = 16;
     while (vb > (int)e &&
@@ -159,7 +159,7 @@ cudaError_t launch_pass(int mode, int dtype, const KernelVariant &v, const PassA
                         cudaStream_t st)
 {
     const bool vec = fast_r(a.r) && aligned16(a.L) && aligned16(a.Y) && aligned16(a.H) &&
-                     aligned16(a.out) && aligned16(a.partials);
+                     aligned16(a.out) && aligned16(a.out16) && aligned16(a.partials);
     const bool fwd = mode == M_FUSED || mode == M_SDDMM || mode == M_SPMM;
     if (v.stages > 0 && vec && fwd) {
         return dtype == FMM_BF16 ? launch_staged_bf16(mode, v.vpl_mult, v.stages, a, st)
@@ -252,7 +252,7 @@ int need_t(const fmm_plan *p)
 
 int run_pass(const fmm_plan *p, const Side &side, int mode, const float *s, const void *L,
              const void *Y, const float *H, float *out, float *nzout, cudaStream_t st,
-             bool accumulate = false)
+             bool accumulate = false, uint16_t *out16 = nullptr)
 {
     PassArgs a;
     a.row_ptr = side.row_ptr;
@@ -270,6 +270,7 @@ int run_pass(const fmm_plan *p, const Side &side, int mode, const float *s, cons
     a.Y = Y;
     a.H = H;
     a.out = out;
+    a.out16 = out16;
     a.nzout = nzout;
     a.r = p->r;
     a.err = p->err;
@@ -291,8 +292,8 @@ int run_pass(const fmm_plan *p, const Side &side, int mode, const float *s, cons
     if (e == cudaSuccess)
         e = launch_pass(mode, p->dtype, side.variant, a, st);
     if (e == cudaSuccess && mode != M_SDDMM)
-        e = launch_combine(side.split, side.n_split, nullptr, side.partials, out, p->r, accumulate,
-                           st);
+        e = launch_combine(side.split, side.n_split, nullptr, side.partials, out, out16, p->r,
+                           accumulate, st);
     if (e != cudaSuccess) {
         set_error("kernel launch", e);
         return FMM_ECUDA;
@@ -496,9 +497,10 @@ static int fusedmm_b(const fmm_plan *p, const float *vals, const void *A, const 
                     (cudaStream_t)stream, acc);
 }
 
+// rows16: dA and dB are bfloat16 (void * below).
 static int fusedmm_a_bwd(const fmm_plan *p, const float *vals, const void *A, const void *B,
-                         const float *G, float *dA, float *dB, float *ds, fmm_stream stream,
-                         bool acc)
+                         const float *G, void *dA, void *dB, float *ds, fmm_stream stream,
+                         bool acc, bool rows16)
 {
     CHECK(check_plan(p));
     CHECK(need(A, p->m, "A"));
@@ -508,9 +510,11 @@ static int fusedmm_a_bwd(const fmm_plan *p, const float *vals, const void *A, co
         CHECK(need_t(p));
     cudaStream_t st = (cudaStream_t)stream;
     if (dA || ds)
-        CHECK(run_pass(p, p->rows, M_BWD_ROW, vals, A, B, G, dA, ds, st, acc));
+        CHECK(run_pass(p, p->rows, M_BWD_ROW, vals, A, B, G, rows16 ? nullptr : (float *)dA, ds, st,
+                       acc, rows16 ? (uint16_t *)dA : nullptr));
     if (dB)
-        CHECK(run_pass(p, p->cols, M_BWD_COL, vals, B, A, G, dB, nullptr, st, acc));
+        CHECK(run_pass(p, p->cols, M_BWD_COL, vals, B, A, G, rows16 ? nullptr : (float *)dB, nullptr,
+                       st, acc, rows16 ? (uint16_t *)dB : nullptr));
     return FMM_OK;
 }
 
@@ -529,7 +533,7 @@ int fmm_fusedmm_t(const fmm_plan *p, const float *vals, const void *A, const voi
 int fmm_fusedmm_bwd(const fmm_plan *p, const float *vals, const void *A, const void *B,
                     const float *G, float *dA, float *dB, float *ds, fmm_stream stream)
 {
-    return fusedmm_a_bwd(p, vals, A, B, G, dA, dB, ds, stream, false);
+    return fusedmm_a_bwd(p, vals, A, B, G, dA, dB, ds, stream, false, false);
 }
 
 int fmm_fusedmm_acc(const fmm_plan *p, const float *vals, const void *A, const void *B,
@@ -547,11 +551,12 @@ int fmm_fusedmm_t_acc(const fmm_plan *p, const float *vals, const void *A, const
 int fmm_fusedmm_bwd_acc(const fmm_plan *p, const float *vals, const void *A, const void *B,
                         const float *G, float *dA, float *dB, float *ds, fmm_stream stream)
 {
-    return fusedmm_a_bwd(p, vals, A, B, G, dA, dB, ds, stream, true);
+    return fusedmm_a_bwd(p, vals, A, B, G, dA, dB, ds, stream, true, false);
 }
 
-int fmm_fusedmm_t_bwd(const fmm_plan *p, const float *vals, const void *A, const void *B,
-                      const float *Gn, float *dA, float *dB, float *ds, fmm_stream stream)
+static int fusedmm_b_bwd(const fmm_plan *p, const float *vals, const void *A, const void *B,
+                         const float *Gn, void *dA, void *dB, float *ds, fmm_stream stream,
+                         bool rows16)
 {
     CHECK(check_plan(p));
     CHECK(need(A, p->m, "A"));
@@ -561,10 +566,44 @@ int fmm_fusedmm_t_bwd(const fmm_plan *p, const float *vals, const void *A, const
         CHECK(need_t(p));
     cudaStream_t st = (cudaStream_t)stream;
     if (dB || ds)
-        CHECK(run_pass(p, p->cols, M_BWD_ROW, vals, B, A, Gn, dB, ds, st));
+        CHECK(run_pass(p, p->cols, M_BWD_ROW, vals, B, A, Gn, rows16 ? nullptr : (float *)dB, ds, st,
+                       false, rows16 ? (uint16_t *)dB : nullptr));
     if (dA)
-        CHECK(run_pass(p, p->rows, M_BWD_COL, vals, A, B, Gn, dA, nullptr, st));
+        CHECK(run_pass(p, p->rows, M_BWD_COL, vals, A, B, Gn, rows16 ? nullptr : (float *)dA, nullptr,
+                       st, false, rows16 ? (uint16_t *)dA : nullptr));
     return FMM_OK;
+}
+
+int fmm_fusedmm_t_bwd(const fmm_plan *p, const float *vals, const void *A, const void *B,
+                      const float *Gn, float *dA, float *dB, float *ds, fmm_stream stream)
+{
+    return fusedmm_b_bwd(p, vals, A, B, Gn, dA, dB, ds, stream, false);
+}
+
+// The generic pass (r above kFlexMaxR) accumulates its rows in place, in
+// float32, so it has no bfloat16 form.
+static int need_rows16(const fmm_plan *p)
+{
+    CHECK(check_plan(p));
+    if (p->dtype == FMM_BF16 && p->r > kFlexMaxR) {
+        set_error_msg("gradients in bfloat16 need r <= 512");
+        return FMM_EUNSUPPORTED;
+    }
+    return FMM_OK;
+}
+
+int fmm_fusedmm_bwd_typed(const fmm_plan *p, const float *vals, const void *A, const void *B,
+                          const float *G, void *dA, void *dB, float *ds, fmm_stream stream)
+{
+    CHECK(need_rows16(p));
+    return fusedmm_a_bwd(p, vals, A, B, G, dA, dB, ds, stream, false, p->dtype == FMM_BF16);
+}
+
+int fmm_fusedmm_t_bwd_typed(const fmm_plan *p, const float *vals, const void *A, const void *B,
+                            const float *Gn, void *dA, void *dB, float *ds, fmm_stream stream)
+{
+    CHECK(need_rows16(p));
+    return fusedmm_b_bwd(p, vals, A, B, Gn, dA, dB, ds, stream, p->dtype == FMM_BF16);
 }
 
 int fmm_plan_status(fmm_plan *p, fmm_stream stream)

@@ -111,6 +111,21 @@ __device__ __forceinline__ void flex_store_f32(float *p, const float *f, bool ad
     }
 }
 
+// EPV floats as bfloat16 to an address aligned to 2 EPV bytes.
+template <int EPV>
+__device__ __forceinline__ void flex_store_bf16(uint16_t *p, const float *f)
+{
+    if constexpr (EPV == 8) {
+        store_bf16x8(p, f);
+    } else if constexpr (EPV == 4) {
+        __stcs(reinterpret_cast<uint2 *>(p), make_uint2(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3])));
+    } else if constexpr (EPV == 2) {
+        __stcs(reinterpret_cast<uint32_t *>(p), pack_bf16x2(f[0], f[1]));
+    } else {
+        *p = (uint16_t)pack_bf16x2(f[0], 0.f);
+    }
+}
+
 // Whether a role adds in the order of the generic kernel: float32 FusedMM and
 // SpMM, whose results an iteration may amplify (the conjugate gradients of
 // ALS past their convergence), are the same bits as the generic kernel's.
@@ -340,6 +355,16 @@ __global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 1
             return;
         float *dst = slot >= 0 ? a.partials + (size_t)slot * a.r
                                : (a.out ? a.out + (size_t)row * a.r : nullptr);
+        if constexpr (sizeof(T) == 2 && (MODE == M_BWD_ROW || MODE == M_BWD_COL)) {
+            if (a.out16 && slot < 0) {
+#pragma unroll
+                for (int v = 0; v < VPL; ++v)
+                    if (v * sh.g + lig < sh.nvec)
+                        flex_store_bf16<EPV>(a.out16 + (size_t)row * a.r + (v * sh.g + lig) * EPV,
+                                             &acc[v * EPV]);
+                return;
+            }
+        }
         if (!dst)
             return;
 #pragma unroll

@@ -118,6 +118,8 @@ struct PassArgs {
     const void *Y;             // gathered rows (dtype of the plan)
     const float *H;            // float32 gradient rows (local or gathered)
     float *out;                // rows x r (NULL: not stored)
+    uint16_t *out16 = nullptr; // bfloat16 rows x r in place of out (adjoint roles of
+                               // bfloat16 plans; float32 results rounded once)
     float *nzout;              // per-nonzero output in S order (NULL: none)
     int32_t r;
     int32_t *err = nullptr;    // device word set to 1 by a pass that gave up a
@@ -205,11 +207,11 @@ cudaError_t launch_values_t(const fmm_plan *p, const float *src, float *dst, cud
 constexpr int64_t kPermuteWindow = int64_t(1) << 23;
 // Sums the partial rows of every entry {row, first chunk, chunks, unused} of
 // split, in chunk order, into out (added to out's rows when accumulate is
-// set).  n_dev: NULL, or the number of entries on the device (n_split at
-// most).
+// set), or as bfloat16 into out16.  n_dev: NULL, or the number of entries on
+// the device (n_split at most).
 cudaError_t launch_combine(const int4 *split, int32_t n_split, const int32_t *n_dev,
-                           const float *partials, float *out, int32_t r, bool accumulate,
-                           cudaStream_t st);
+                           const float *partials, float *out, uint16_t *out16, int32_t r,
+                           bool accumulate, cudaStream_t st);
 
 bool fast_r(int32_t r);
 // Streaming multiprocessors of the current device (queried once per device;

@@ -319,7 +319,8 @@ extern "C" int fmm_fusedmm_noalloc(const fmm_csr *S, int32_t r, int32_t dtype, c
                               : launch_checked<float>(p, dtype, st);
         if (e == cudaSuccess && a.cap > 0) {
             // a long row has two chunks at least
-            e = launch_combine(a.split, a.cap / 2 + 1, &a.hdr->n_split, partials, out_m, r, false, st);
+            e = launch_combine(a.split, a.cap / 2 + 1, &a.hdr->n_split, partials, out_m, nullptr, r,
+                               false, st);
         }
         if (e == cudaSuccess)
             e = cudaGetLastError();

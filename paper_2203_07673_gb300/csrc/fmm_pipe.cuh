@@ -394,6 +394,15 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
         if (active) {
             float *dst = slot >= 0 ? a.partials + (size_t)slot * R
                                    : (a.out ? a.out + (size_t)row * R : nullptr);
+            if constexpr (TWO && sizeof(T) == 2) {
+                if (a.out16 && slot < 0) {
+#pragma unroll
+                    for (int v = 0; v < VPL; ++v)
+                        store_bf16x8(a.out16 + (size_t)row * R + widx(v) * 8,
+                                     reinterpret_cast<const float *>(&acc2[v * W2]));
+                    dst = nullptr;
+                }
+            }
             if (dst) {
 #pragma unroll
                 for (int v = 0; v < VPL; ++v) {

@@ -13,6 +13,8 @@
 #include <cstdio>
 #include <vector>
 
+#include <cuda_bf16.h>
+
 #include "fmm_internal.cuh"
 
 namespace fmm {
@@ -899,7 +901,8 @@ constexpr int kCombineLoads = 16;
 template <int VEC>
 __global__ void __launch_bounds__(128) combine_kernel(const int4 *split, int32_t n_split,
                                                       const int32_t *n_dev, int32_t tiles,
-                                                      const float *partials, float *out, int32_t r,
+                                                      const float *partials, float *out,
+                                                      uint16_t *out16, int32_t r,
                                                       int32_t accumulate)
 {
     const int lane = threadIdx.x & 31;
@@ -935,23 +938,29 @@ __global__ void __launch_bounds__(128) combine_kernel(const int4 *split, int32_t
         }
     }
     // element by element: out needs no alignment
+    if (out16) {
+        uint16_t *o = out16 + (size_t)sp.x * r + k;
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) o[v] = __bfloat16_as_ushort(__float2bfloat16_rn(acc[v]));
+        return;
+    }
     float *o = out + (size_t)sp.x * r + k;
 #pragma unroll
     for (int v = 0; v < VEC; ++v) o[v] = accumulate ? o[v] + acc[v] : acc[v];
 }
 
 cudaError_t launch_combine(const int4 *split, int32_t n_split, const int32_t *n_dev,
-                           const float *partials, float *out, int32_t r, bool accumulate,
-                           cudaStream_t st)
+                           const float *partials, float *out, uint16_t *out16, int32_t r,
+                           bool accumulate, cudaStream_t st)
 {
-    if (n_split == 0 || !out)
+    if (n_split == 0 || (!out && !out16))
         return cudaSuccess;
     // partial rows start 16-byte aligned when r is a multiple of 4
     const int vec = r % 4 == 0 ? 4 : 1;
     const int32_t tiles = (r + 32 * vec - 1) / (32 * vec);
     const unsigned blocks = (unsigned)(((int64_t)n_split * tiles + 3) / 4);
     auto *kernel = vec == 4 ? combine_kernel<4> : combine_kernel<1>;
-    kernel<<<blocks, 128, 0, st>>>(split, n_split, n_dev, tiles, partials, out, r,
+    kernel<<<blocks, 128, 0, st>>>(split, n_split, n_dev, tiles, partials, out, out16, r,
                                    accumulate ? 1 : 0);
     return cudaGetLastError();
 }

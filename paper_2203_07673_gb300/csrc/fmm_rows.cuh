@@ -258,6 +258,22 @@ __device__ __forceinline__ void team_store_f32(const Loader &ld, float *row, int
     }
 }
 
+// Two floats as a word of bfloat16 (a in the low half), nearest even.
+__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b)
+{
+    uint32_t w;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(b), "f"(a));
+    return w;
+}
+
+// Eight floats as a 16-byte word of bfloat16, streaming.
+__device__ __forceinline__ void store_bf16x8(uint16_t *p, const float *f)
+{
+    __stcs(reinterpret_cast<uint4 *>(p),
+           make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]),
+                      pack_bf16x2(f[6], f[7])));
+}
+
 // One row pass.  A team of NG x G lanes owns one work item (a light row, or
 // a chunk of a split row); per batch each group handles U nonzeros, so a
 // batch covers NG * U consecutive nonzeros (nonzero base + u * NG + g goes to
@@ -471,6 +487,14 @@ __device__ __forceinline__ void team_pass_body(const PassArgs &a, long long gid,
         if (active && grp == 0) {
             float *dst = slot >= 0 ? a.partials + (size_t)slot * R
                                    : (a.out ? a.out + (size_t)row * R : nullptr);
+            if constexpr (TWO && sizeof(T) == 2) {
+                if (a.out16 && slot < 0) {
+#pragma unroll
+                    for (int v = 0; v < VPL; ++v)
+                        store_bf16x8(a.out16 + (size_t)row * R + (v * G + lig) * 8, acc + 8 * v);
+                    dst = nullptr;
+                }
+            }
             if (dst)
                 team_store_f32<T, VPL, G>(ld, dst, lig, acc, a.accumulate && slot < 0);
         }

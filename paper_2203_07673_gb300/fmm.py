@@ -38,6 +38,8 @@ _SIGNATURES = {
     "fmm_fusedmm_t": ([_P, _P, _P, _P, _P, _P], ctypes.c_int),
     "fmm_fusedmm_bwd": ([_P, _P, _P, _P, _P, _P, _P, _P, _P], ctypes.c_int),
     "fmm_fusedmm_t_bwd": ([_P, _P, _P, _P, _P, _P, _P, _P, _P], ctypes.c_int),
+    "fmm_fusedmm_bwd_typed": ([_P, _P, _P, _P, _P, _P, _P, _P, _P], ctypes.c_int),
+    "fmm_fusedmm_t_bwd_typed": ([_P, _P, _P, _P, _P, _P, _P, _P, _P], ctypes.c_int),
     "fmm_fusedmm_acc": ([_P, _P, _P, _P, _P, _P], ctypes.c_int),
     "fmm_sddmm_acc": ([_P, _P, _P, _P, _P, _P], ctypes.c_int),
     "fmm_spmm_acc": ([_P, _P, _P, _P, _P], ctypes.c_int),
@@ -308,6 +310,29 @@ def fusedmm_bwd(plan: Plan, vals, A, B, G, need=(True, True, True), stream=None,
                                plan._f32(ds, (plan.nnz,), "ds"), _stream(stream))
     _check(rc, "fmm_fusedmm_bwd")
     return dA, dB, ds
+
+
+def _bwd_typed(name, plan: Plan, rows, vals, A, B, G, need, stream):
+    dA = torch.empty((plan.m, plan.r), dtype=plan.dtype, device=plan.device) if need[0] else None
+    dB = torch.empty((plan.n, plan.r), dtype=plan.dtype, device=plan.device) if need[1] else None
+    ds = torch.empty((plan.nnz,), dtype=torch.float32, device=plan.device) if need[2] else None
+    rc = getattr(lib(), name)(plan.handle, plan._f32(vals, (plan.nnz,), "vals"),
+                              plan._dense(A, plan.m, "A"), plan._dense(B, plan.n, "B"),
+                              plan._f32(G, (rows, plan.r), "G"), plan._dense(dA, plan.m, "dA"),
+                              plan._dense(dB, plan.n, "dB"), plan._f32(ds, (plan.nnz,), "ds"),
+                              _stream(stream))
+    _check(rc, name)
+    return dA, dB, ds
+
+
+def fusedmm_bwd_typed(plan: Plan, vals, A, B, G, need=(True, True, True), stream=None):
+    """fmm_fusedmm_bwd_typed: as fusedmm_bwd with dA and dB in the plan's dtype."""
+    return _bwd_typed("fmm_fusedmm_bwd_typed", plan, plan.m, vals, A, B, G, need, stream)
+
+
+def fusedmm_t_bwd_typed(plan: Plan, vals, A, B, Gn, need=(True, True, True), stream=None):
+    """fmm_fusedmm_t_bwd_typed: as fusedmm_t_bwd with dA and dB in the plan's dtype."""
+    return _bwd_typed("fmm_fusedmm_t_bwd_typed", plan, plan.n, vals, A, B, Gn, need, stream)
 
 
 def sddmm_acc(plan: Plan, vals, A, B, v, stream=None):

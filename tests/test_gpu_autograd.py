@@ -75,3 +75,34 @@ def test_autograd_partial_requirements():
     assert At.grad is None and Bt.grad is not None
     ref = oracle.fusedmm_grad(S.row_ptr, S.col_idx, None, A, B, np.ones((100, 32)), S.n)[1]
     assert relF(Bt.grad.double().cpu().numpy(), ref) <= 1e-5
+
+
+@pytest.mark.parametrize("transpose", [False, True], ids=["A", "B"])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("r", [32, 64, 256, 6, 7, 20, 512])
+def test_gradients_in_the_plan_dtype(r, dtype, transpose):
+    """fmm_fusedmm_bwd_typed and fmm_fusedmm_t_bwd_typed: the float32 gradients
+    rounded once, bit for bit, rows in chunks and rows without nonzeros among
+    them, each output alone too; bfloat16 of r > 512 is refused."""
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(r)
+    S = wl.random_csr(400, 300, rng, mean_deg=6, empty_frac=0.1, hubs=((9, 900), (11, 3000)))
+    S.col_idx[::4] = 7
+    f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+    rp, ci = torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda()
+    plan = fmm.Plan(rp, ci, S.n, r, dtype)
+    vals, A, B, G = f(S.nnz), f(S.m, r).to(dtype), f(S.n, r).to(dtype), f(S.n if transpose else S.m, r)
+    plain = fmm.fusedmm_t_bwd if transpose else fmm.fusedmm_bwd
+    typed = fmm.fusedmm_t_bwd_typed if transpose else fmm.fusedmm_bwd_typed
+    want = plain(plan, vals, A, B, G)
+    for need in ((True, True, True), (True, False, False), (False, True, False)):
+        for x, w, n in zip(typed(plan, vals, A, B, G, need), want, need):
+            if n:
+                assert torch.equal(x, w.to(x.dtype))
+            else:
+                assert x is None
+    if dtype == torch.bfloat16:
+        wide = fmm.Plan(rp, ci, S.n, 513, dtype)
+        with pytest.raises(fmm.FmmError):
+            typed(wide, vals, f(S.m, 513).to(dtype), f(S.n, 513).to(dtype),
+                  f(S.n if transpose else S.m, 513))
