@@ -49,4 +49,10 @@ class FusedMMFunction(torch.autograd.Function):
 
 def fusedmm(plan, vals, A, B, transpose: bool = False):
     """Differentiable FusedMMA (or FusedMMB with transpose=True)."""
+    if plan.fast is not None:
+        # the same function in native code (csrc/torch_calls.cpp), for ordinary
+        # tensors outside of modes and transforms
+        out = fmm._calls.autograd(plan.fast, plan, vals, A, B, transpose)
+        if out is not NotImplemented:
+            return out
     return FusedMMFunction.apply(plan, vals, A, B, transpose)

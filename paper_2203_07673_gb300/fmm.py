@@ -5,10 +5,16 @@ shapes, passes raw device pointers and the current CUDA stream to the C entry
 point of the same name, and raises ``FmmError`` on a nonzero status.  All
 computation happens in the library's CUDA kernels; there is no CPU path.  If
 the library cannot be loaded, every call raises.
+
+The most frequent calls go through a native module first
+(csrc/torch_calls.cpp), which does the same marshalling for ordinary tensors on
+the current stream and returns NotImplemented for anything else.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 import threading
 
@@ -16,6 +22,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "_build", "libfmm.so")
+CALLS_PATH = os.path.join(_PKG, "_build", "fmm_calls.so")
 
 FMM_OK, FMM_EINVAL, FMM_EUNSUPPORTED, FMM_EOVERFLOW, FMM_ECUDA, FMM_ENOMEM, FMM_ETIMEOUT = \
     0, -1, -2, -3, -4, -5, -6
@@ -92,11 +99,22 @@ class _Info(ctypes.Structure):
 
 _lock = threading.Lock()
 _lib = None
+_calls = None   # the native call path, once the library is loaded (if it is built)
+
+
+def _load_calls():
+    if not os.path.exists(CALLS_PATH):
+        return None
+    loader = importlib.machinery.ExtensionFileLoader("fmm_calls", CALLS_PATH)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("fmm_calls", loader))
+    loader.exec_module(mod)
+    mod.set_check(_check)
+    return mod
 
 
 def lib() -> ctypes.CDLL:
     """The loaded libfmm (raises if it is not built or cannot be loaded)."""
-    global _lib
+    global _lib, _calls
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -109,6 +127,8 @@ def lib() -> ctypes.CDLL:
                 fn.argtypes = args
                 fn.restype = res
             _lib = handle
+            if _calls is None:
+                _calls = _load_calls()
     return _lib
 
 
@@ -168,6 +188,7 @@ class Plan:
         if dtype not in _DT:
             raise TypeError(f"unsupported dtype {dtype}")
         self.handle = None
+        self.fast = None   # the plan as the native call path holds it
         self.device = row_ptr.device
         _ptr(row_ptr, "row_ptr", torch.int32)
         _ptr(col_idx, "col_idx", torch.int32, device=self.device)
@@ -186,6 +207,9 @@ class Plan:
                                        _stream(stream), ctypes.byref(out))
         _check(rc, "fmm_plan_create")
         self.handle = out.value
+        if _calls is not None:
+            self.fast = _calls.plan(self.handle, self.m, self.n, self.r, self.nnz,
+                                    dtype == torch.bfloat16, self.device.index or 0)
 
     def set_variant(self, variant: int = 0, variant_t: int = 0):
         """fmm_plan_set_variant (0 leaves a side unchanged)."""
@@ -212,6 +236,9 @@ class Plan:
 
     def close(self):
         if self.handle is not None:
+            if self.fast is not None:
+                _calls.close(self.fast)
+                self.fast = None
             lib().fmm_plan_destroy(self.handle)
             self.handle = None
 
@@ -247,6 +274,10 @@ def _out(out, shape, plan):
 
 
 def sddmm(plan: Plan, vals, A, B, out=None, stream=None):
+    if stream is None and plan.fast is not None:
+        done = _calls.sddmm(plan.fast, vals, A, B, out)
+        if done is not NotImplemented:
+            return done
     out = _out(out, (plan.nnz,), plan)
     rc = lib().fmm_sddmm(plan.handle, plan._f32(vals, (plan.nnz,), "vals"),
                          plan._dense(A, plan.m, "A"), plan._dense(B, plan.n, "B"),
@@ -256,6 +287,10 @@ def sddmm(plan: Plan, vals, A, B, out=None, stream=None):
 
 
 def spmm(plan: Plan, v, B, out=None, stream=None):
+    if stream is None and plan.fast is not None:
+        done = _calls.spmm(plan.fast, v, B, out)
+        if done is not NotImplemented:
+            return done
     out = _out(out, (plan.m, plan.r), plan)
     rc = lib().fmm_spmm(plan.handle, plan._f32(v, (plan.nnz,), "v"),
                         plan._dense(B, plan.n, "B"), plan._f32(out, (plan.m, plan.r), "out"),
@@ -265,6 +300,10 @@ def spmm(plan: Plan, v, B, out=None, stream=None):
 
 
 def spmm_t(plan: Plan, v, A, out=None, stream=None):
+    if stream is None and plan.fast is not None:
+        done = _calls.spmm_t(plan.fast, v, A, out)
+        if done is not NotImplemented:
+            return done
     out = _out(out, (plan.n, plan.r), plan)
     rc = lib().fmm_spmm_t(plan.handle, plan._f32(v, (plan.nnz,), "v"),
                           plan._dense(A, plan.m, "A"), plan._f32(out, (plan.n, plan.r), "out"),
@@ -274,6 +313,10 @@ def spmm_t(plan: Plan, v, A, out=None, stream=None):
 
 
 def fusedmm(plan: Plan, vals, A, B, out=None, stream=None):
+    if stream is None and plan.fast is not None:
+        done = _calls.fusedmm(plan.fast, vals, A, B, out)
+        if done is not NotImplemented:
+            return done
     out = _out(out, (plan.m, plan.r), plan)
     rc = lib().fmm_fusedmm(plan.handle, plan._f32(vals, (plan.nnz,), "vals"),
                            plan._dense(A, plan.m, "A"), plan._dense(B, plan.n, "B"),
@@ -283,6 +326,10 @@ def fusedmm(plan: Plan, vals, A, B, out=None, stream=None):
 
 
 def fusedmm_t(plan: Plan, vals, A, B, out=None, stream=None):
+    if stream is None and plan.fast is not None:
+        done = _calls.fusedmm_t(plan.fast, vals, A, B, out)
+        if done is not NotImplemented:
+            return done
     out = _out(out, (plan.n, plan.r), plan)
     rc = lib().fmm_fusedmm_t(plan.handle, plan._f32(vals, (plan.nnz,), "vals"),
                              plan._dense(A, plan.m, "A"), plan._dense(B, plan.n, "B"),
@@ -520,6 +567,9 @@ def cg_init(lam, b, mx, x, res, p, rs, stream=None):
 
 def cg_update(lam, x, res, p, q, rs, stream=None):
     """fmm_cg_update on float32 row blocks (rows x r)."""
+    if stream is None and _calls is not None and _calls.cg_update(
+            float(lam), x, res, p, q, rs) is not NotImplemented:
+        return
     rows, r = x.shape
     rc = lib().fmm_cg_update(rows, r, float(lam), _rows_f32(x, rows, r, "x"),
                              _rows_f32(res, rows, r, "res"), _rows_f32(p, rows, r, "p"),
