@@ -119,8 +119,8 @@ typedef struct fmm_plan_options {
                                  and SpMM stage the next D - 1 gathered rows
                                  of each row in shared memory (cp.async);
                                  or F*10000 + M*1000 + P*100 + U*10 + V
-                                 (22212, 23212, 22412, 32212, 24221, 34221,
-                                 23421, 23241): FusedMM, SDDMM and SpMM keep
+                                 (22212, 23212, 22412, 32212, 32412, 24221,
+                                 34221, 23421, 23241): FusedMM, SDDMM and SpMM keep
                                  the gathered rows of the next P - 1 (F = 2)
                                  or P (F = 3) batches of U nonzeros in
                                  flight in registers, with M resident
@@ -147,9 +147,11 @@ typedef struct fmm_plan_options {
                                  kinds need the gathered operand 32-byte
                                  aligned.  A layout a width does not have
                                  falls back to that team layout.
-                                 Default: 32212 for bfloat16 rows of r = 64
-                                 and 128, 1042 for float32 rows of r = 128,
-                                 else that team layout                       */
+                                 Default: 32212 for bfloat16 rows (32412 for
+                                 r = 128), 1042 for float32 rows of r = 128,
+                                 else that team layout; SDDMM, SpMM and the
+                                 adjoints of a plan left to its default may
+                                 run another layout                          */
 } fmm_plan_options;
 
 typedef struct fmm_plan fmm_plan;   /* opaque */
@@ -316,8 +318,9 @@ int fmm_spmm_t_acc(const fmm_plan *plan, const float *v, const void *A, float *o
 /*
  * Kernel variant of a plan's row passes (the codes of
  * fmm_plan_options.variant; 0 leaves a side unchanged).  variant applies to
- * passes over S, variant_t to passes over S^T.  Used by the autotuner; calls
- * already queued are not affected.
+ * passes over S, variant_t to passes over S^T.  The code of a plan's default
+ * gives the default back, with its own choice per operation.  Used by the
+ * autotuner; calls already queued are not affected.
  */
 int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
 

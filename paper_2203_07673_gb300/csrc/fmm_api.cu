@@ -51,7 +51,7 @@ static bool aligned32(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // S^T by the team kernel.
 static const int kVariantCodes[] = {114, 118, 222, 224, 441, 442, 214, 124, 112, 122, 212, 221,
                                     1041, 1042, 1081, 1082,
-                                    22212, 23212, 22412, 32212, 24221, 34221, 23421, 23241,
+                                    22212, 23212, 22412, 32212, 32412, 24221, 34221, 23421, 23241,
                                     44042, 43082, 44041, 44081, 52212, 52412, 54211};
 
 int flex_lanes(int32_t r)
@@ -155,9 +155,10 @@ int encode_variant(const KernelVariant &v)
     return v.vpl_mult * 100 + v.ng * 10 + v.u;
 }
 
-cudaError_t launch_pass(int mode, int dtype, const KernelVariant &v, const PassArgs &a,
+cudaError_t launch_pass(int mode, int dtype, const KernelVariant &given, const PassArgs &a,
                         cudaStream_t st)
 {
+    const KernelVariant v = given.own ? role_variant(mode, a.r, dtype) : given;
     const bool vec = fast_r(a.r) && aligned16(a.L) && aligned16(a.Y) && aligned16(a.H) &&
                      aligned16(a.out) && aligned16(a.out16) && aligned16(a.partials);
     const bool fwd = mode == M_FUSED || mode == M_SDDMM || mode == M_SPMM;
@@ -179,9 +180,11 @@ cudaError_t launch_pass(int mode, int dtype, const KernelVariant &v, const PassA
         if (e != cudaErrorNotSupported)
             return e;
     }
-    // the register-ring pass loads gathered rows 32 bytes at a time; of the
-    // adjoint roles it has the pass over S
-    if (v.ring > 0 && vec && (fwd || mode == M_BWD_ROW) && aligned32(a.Y)) {
+    // the register-ring pass loads gathered rows (bfloat16 rows' gradient rows
+    // too) 32 bytes at a time; of the adjoint roles it has the pass over S, and
+    // the pass over S^T as the plan's own choice
+    if (v.ring > 0 && vec && aligned32(a.Y) &&
+        (fwd || mode == M_BWD_ROW || (v.own && aligned32(a.H)))) {
         const cudaError_t e = dtype == FMM_BF16
                                   ? launch_pipe_bf16(mode, v.vpl_mult, v.u, v.ring, v.mb, v.refill, a, st)
                                   : launch_pipe_f32(mode, v.vpl_mult, v.u, v.ring, v.mb, v.refill, a, st);

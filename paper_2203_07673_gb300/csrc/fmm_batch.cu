@@ -89,7 +89,7 @@ __device__ __forceinline__ void run_unit(const PassArgs &a, int begin, int count
     const int lane = threadIdx.x & 31;
     for (int t0 = 0; t0 < count; t0 += TPW) {
         const int t = t0 + lane / TEAM;
-        team_pass_body<MODE, T, R, VPL, NG, U>(a, (long long)begin + t, t < count);
+        team_pass_body<MODE, T, R, VPL, NG, U, false, false>(a, (long long)begin + t, t < count);
     }
 }
 
@@ -293,10 +293,13 @@ int fmm_plan_set_variant(fmm_plan *p, int32_t variant, int32_t variant_t)
         set_error_msg("invalid plan or variant code");
         return FMM_EINVAL;
     }
+    // the code of the plan's own choice gives that choice back
+    const KernelVariant own = default_variant(p->r, p->dtype, 0.0);
+    const int own_code = encode_variant(own);
     if (variant)
-        p->rows.variant = decode_variant(variant);
+        p->rows.variant = variant == own_code ? own : decode_variant(variant);
     if (variant_t)
-        p->cols.variant = decode_variant(variant_t);
+        p->cols.variant = variant_t == own_code ? own : decode_variant(variant_t);
     return FMM_OK;
 }
 

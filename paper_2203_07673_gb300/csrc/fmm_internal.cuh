@@ -22,6 +22,8 @@ struct KernelVariant {
     int refill = 0;   // pipelined pass: 1 = refill a slot as soon as it is read
     int depth = 0;    // > 0: the bulk-staged pass (fmm_bulk.cuh), this many row
                       // slots in shared memory per team (forward roles)
+    bool own = false; // the plan's own choice for its width (not asked for): every
+                      // role then runs what role_variant gives
     int stream = 0;   // 1: the streaming pass (fmm_stream.cuh): a team walks a run
                       // of consecutive rows as one stream of nonzeros, with the
                       // register ring of the pipelined pass (ring, mb; refill)
@@ -223,6 +225,8 @@ int encode_variant(const KernelVariant &v);
 // Default kernel variant of a pass over rows of width r (dtype, average
 // nonzeros per row).
 KernelVariant default_variant(int32_t r, int32_t dtype, double avg_nnz);
+// The same per role (default_variant is that of FusedMM).
+KernelVariant role_variant(int mode, int32_t r, int32_t dtype);
 // The team kernel's layout for a width (one group per row, 8 elements per
 // lane, 2 nonzeros per batch): the default of the batch kernels.
 KernelVariant team_default_variant(int32_t r, int32_t dtype);

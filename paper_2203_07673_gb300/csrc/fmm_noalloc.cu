@@ -189,17 +189,17 @@ __global__ void __launch_bounds__(kBlock) place_kernel(const Args a)
 }
 
 // The pass over the work items: for vectorised widths the layouts of
-// default_variant (the register ring for bfloat16 rows of r = 64 and 128, the
-// staged pass for float32 rows of r = 128, else the team kernel with 8
-// elements per lane), otherwise the flexible or the generic pass.
+// default_variant (the register ring for bfloat16 rows, the staged pass for
+// float32 rows of r = 128, else the team kernel with 8 elements per lane),
+// otherwise the flexible or the generic pass.
 template <typename T, int R>
 cudaError_t launch_width(const PassArgs &p, cudaStream_t st)
 {
     constexpr int B = base_vpl<T, R>();
     constexpr int V = sizeof(T) == 4 && R * 4 / 16 <= 32 ? 2 * B : B;   // 8 elements per lane
-    if constexpr (sizeof(T) == 2 && (R == 64 || R == 128)) {
+    if constexpr (sizeof(T) == 2) {
         if ((reinterpret_cast<uintptr_t>(p.Y) & 31u) == 0)
-            return launch_pipe<M_FUSED, T, R, 2 * B, 1, 2, 2, 1, true>(p, st);
+            return launch_pipe<M_FUSED, T, R, 2 * B, 1, R == 128 ? 4 : 2, 2, 1, true>(p, st);
     }
     if constexpr (sizeof(T) == 4 && R == 128)
         return launch_staged<M_FUSED, T, R, V, 4, true>(p, st);

@@ -37,11 +37,10 @@
 //
 // Roles: FusedMM, SDDMM, SpMM, and the two adjoint passes: over S (two
 // dot products of the gathered row, against the local row and the local
-// float32 gradient row; ds written) and over S^T (the gathered row and its
-// float32 gradient row both in the ring).  The pass over S is instantiated
-// for the default layout only (code 32212): on R-MAT 2^22 with bfloat16 rows
-// of r = 64 the backward took 5.205 ms with it against 5.289 ms with the
-// team kernel; the pass over S^T (5.47 ms with it) is not instantiated.  One
+// float32 gradient row; ds kept per lane and stored a block at a time, as the
+// SDDMM values) and over S^T (the gathered row and its float32 gradient row
+// both in the ring, the latter by 32-byte loads).  Which layout a role runs by
+// default, and both sides of each choice, stand at role_variant.  One
 // team of G lanes per row or chunk of a split row.
 #pragma once
 
@@ -59,6 +58,14 @@ __device__ __forceinline__ void load32(const void *p, uint4 &w0, uint4 &w1)
     asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(w0.x), "=r"(w0.y), "=r"(w0.z), "=r"(w0.w), "=r"(w1.x), "=r"(w1.y),
                    "=r"(w1.z), "=r"(w1.w)
+                 : "l"(p));
+}
+
+__device__ __forceinline__ void load32f(const float *p, float4 &w0, float4 &w1)
+{
+    asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(w0.x), "=f"(w0.y), "=f"(w0.z), "=f"(w0.w), "=f"(w1.x), "=f"(w1.y),
+                   "=f"(w1.z), "=f"(w1.w)
                  : "l"(p));
 }
 
@@ -165,7 +172,7 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
     // the end of the row j = -1 and s = 0
     int jc[K], jn[K], ic[K], in_[K];
     float sc[K], sn[K];
-    // per-nonzero outputs (SDDMM): the lane holding a nonzero's index entry
+    // per-nonzero outputs (v, ds): the lane holding a nonzero's index entry
     // keeps its value and stores the block's values at once
     float held[K];
 #pragma unroll
@@ -222,15 +229,26 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
         for (int u = 0; u < U; ++u) {
             const int t = bb * U + u;
             const int jj = __shfl_sync(0xffffffffu, j[t / G], tbase + (t % G));
+            if constexpr (EPV == 8) {   // 32 bytes per word of bfloat16
 #pragma unroll
-            for (int v = 0; v < VPL; ++v)
-#pragma unroll
-                for (int q = 0; q < EPV / 4; ++q) {
-                    dst[u][v * (EPV / 4) + q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int v = 0; v < VPL; ++v) {
+                    dst[u][2 * v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    dst[u][2 * v + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (jj >= 0)
-                        dst[u][v * (EPV / 4) + q] =
-                            ld.f4(a.H + (size_t)jj * R + widx(v) * EPV + 4 * q, true);
+                        load32f(a.H + (size_t)jj * R + widx(v) * EPV, dst[u][2 * v],
+                                dst[u][2 * v + 1]);
                 }
+            } else {
+#pragma unroll
+                for (int v = 0; v < VPL; ++v)
+#pragma unroll
+                    for (int q = 0; q < EPV / 4; ++q) {
+                        dst[u][v * (EPV / 4) + q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (jj >= 0)
+                            dst[u][v * (EPV / 4) + q] =
+                                ld.f4(a.H + (size_t)jj * R + widx(v) * EPV + 4 * q, true);
+                    }
+            }
         }
     };
     auto issue_all = [&](int slot_, const int (&j)[K], int bb) {
@@ -258,13 +276,10 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
             }
             // use batch bb
             float sv[U];
-            int sidx[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int t = bb * U + u;
                 sv[u] = __shfl_sync(0xffffffffu, sc[t / G], tbase + (t % G));
-                sidx[u] = (NZ && MODE != M_SDDMM) ? __shfl_sync(0xffffffffu, ic[t / G], tbase + (t % G))
-                                                  : 0;
             }
             float2 y2[U][E2];
             float2 g2[GATHER_H ? U : 1][GATHER_H ? E2 : 1];
@@ -356,8 +371,9 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
                     // ds = <A_i, B_j> <G_i, B_j>;  dA_i += s <G_i, B_j> B_j
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        if (a.nzout && sidx[u] >= 0 && lig == (u % G))
-                            a.nzout[sidx[u]] = d[u] * d[U + u];
+                        const int t = bb * U + u;
+                        if (lig == t % G)
+                            held[t / G] = d[u] * d[U + u];
                         const float c = sv[u] * d[U + u];
                         const float2 c2 = make_float2(c, c);
 #pragma unroll
@@ -376,10 +392,10 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
                 }
             }
         }
-        if constexpr (MODE == M_SDDMM) {
+        if constexpr (NZ) {
 #pragma unroll
             for (int e = 0; e < K; ++e)
-                if (ic[e] >= 0)
+                if (ic[e] >= 0 && (MODE == M_SDDMM || a.nzout))
                     nz_store<MODE>(a, ic[e], held[e]);
         }
         // the next block becomes current; fetch the one after it
@@ -459,6 +475,20 @@ cudaError_t dispatch_pipe(int mode, int vpl, int u, int ring, int mb, int refill
     FMM_PIPE_MODES(2 * B, 1, 2, 3, 0)
     FMM_PIPE_MODES(2 * B, 1, 4, 2, 0)
     FMM_PIPE_MODES(2 * B, 1, 2, 2, 1) FMM_PIPE(M_BWD_ROW, 2 * B, 1, 2, 2, 1)
+    // 32412, and what role_variant picks beside the codes
+    FMM_PIPE_MODES(2 * B, 1, 4, 2, 1) FMM_PIPE(M_BWD_ROW, 2 * B, 1, 4, 2, 1)
+    if constexpr (sizeof(T) == 2 && R == 64) {
+        FMM_PIPE(M_BWD_COL, B, 1, 4, 2, 1)
+    }
+    if constexpr (sizeof(T) == 2 && R >= 128) {
+        FMM_PIPE(M_BWD_COL, 2 * B, 1, 2, 2, 1)
+    }
+    if constexpr (sizeof(T) == 4 && R == 128) {
+        FMM_PIPE(M_SDDMM, 2 * B, 2, 2, 3, 1)
+    }
+    if constexpr (sizeof(T) == 4 && R == 256) {
+        FMM_PIPE(M_SDDMM, 2 * B, 2, 2, 2, 1)
+    }
     FMM_PIPE_MODES(B, 2, 2, 4, 0)
     FMM_PIPE_MODES(B, 2, 2, 4, 1)
     FMM_PIPE_MODES(B, 2, 4, 3, 0)

@@ -756,24 +756,29 @@ KernelVariant team_default_variant(int32_t r, int32_t dtype)
     return v;
 }
 
+// The register-ring pass: vpl x the minimum vectors per lane, a ring of
+// `ring` batches of one nonzero, refilled, 2 x 256 threads per SM.
+static KernelVariant ring_variant(int vpl, int ring)
+{
+    KernelVariant v;
+    v.vpl_mult = vpl;
+    v.ng = 1;
+    v.u = 1;
+    v.ring = ring;
+    v.mb = 2;
+    v.refill = 1;
+    return v;
+}
+
 KernelVariant default_variant(int32_t r, int32_t dtype, double avg_nnz)
 {
     (void)avg_nnz;
     KernelVariant v = team_default_variant(r, dtype);
-    // bfloat16 rows of r = 64 and 128: the register-ring pass with 16
-    // elements per lane, one nonzero per batch and the slot refilled as soon
-    // as it is read (code 32212).  Measured on GB300 (FusedMMA / FusedMMB
-    // pass, ms): Zipf rows 2^21 x 2^19 1.71 / 1.54 -> 1.36 / 1.06, R-MAT 2^22
-    // 1.65 -> 1.41, Erdos-Renyi 2^20 at r = 128 1.55 / 1.74 -> 1.41 / 1.53.
-    // Of the backward roles, the pass over S runs the same ring pass, the pass
-    // over S^T the team kernel's default layout.
-    if (dtype == FMM_BF16 && (r == 64 || r == 128)) {
-        v.vpl_mult = 2;
-        v.u = 1;
-        v.ring = 2;
-        v.mb = 2;
-        v.refill = 1;
-    }
+    // bfloat16 rows: the register-ring pass with 16 elements per lane, one
+    // nonzero per batch and the slot refilled as soon as it is read (code 32212;
+    // r = 128 with a ring of 4, 32412)
+    if (dtype == FMM_BF16 && fast_r(r))
+        v = ring_variant(2, r == 128 ? 4 : 2);
     // float32 rows of r = 128 (512 bytes): the staged pass with a ring of 4
     // gathered rows per team, 3-4 % faster on Erdos-Renyi rows at the DRAM
     // roofline (it needs no register spill); where gathers mostly hit L2 the
@@ -781,6 +786,52 @@ KernelVariant default_variant(int32_t r, int32_t dtype, double avg_nnz)
     // gains, and the team kernel stays
     if (dtype == FMM_F32 && r == 128)
         v.stages = 4;
+    v.own = true;
+    return v;
+}
+
+// Measured on GB300 (ms; R-MAT, then Zipf rows at r = 32 and 64 or
+// Erdos-Renyi at r = 128 and 256; the team kernel with 8 elements per lane ->
+// the ring pass, where that is the choice):
+//   bfloat16             r = 32         r = 64         r = 128       r = 256
+//   FusedMM            .207 .438 ->   1.65 1.71 ->      1.55 ->    .416 .222 ->
+//                      .197 .385      1.26 1.29       .604 .068    .319 .148
+//   adjoint over S     .291 .638 ->   1.08 1.11 ->    .892 .100 -> .667 .354 ->
+//     (ring of 4; from a ring of 2    .833 .875       .753 .088    .417 .192
+//      at r = 64, 128) .246 .571
+//   adjoint over S^T       team       2.79 1.23 ->    1.35 .198 -> .764 .472 ->
+//     (r = 64: 8 elements per lane,   2.69 1.15       1.26 .198    .636 .460
+//      ring of 4; above: 16, 2)
+//   SDDMM                  team         ring            ring       .351 .177 ->
+//                                                                  .248 .111
+//   SpMM                   team         ring            ring       .224 .113 ->
+//                                                                  .220 .107
+// (SDDMM and SpMM of r = 32 by the ring: .165 -> .185, .156 -> .178.)  Float32
+// rows: SDDMM of r = 128 by a ring of 2 batches of 2 (.778 .099 with the staged
+// pass -> .754 .081) and of r = 256 (.394 .218 -> .381 .193), adjoint over S of
+// r = 256 (.623 .345 -> .537 .313); the other roles lose with a ring (FusedMM
+// also has to keep its order of sums, see fmm_flex.cuh).
+KernelVariant role_variant(int mode, int32_t r, int32_t dtype)
+{
+    KernelVariant v = default_variant(r, dtype, 0.0);
+    if (!fast_r(r))
+        return v;
+    if (dtype == FMM_BF16) {
+        if (mode == M_BWD_ROW)
+            v = ring_variant(2, 4);
+        else if (mode == M_BWD_COL)
+            v = r == 32 ? team_default_variant(r, dtype)
+                        : r == 64 ? ring_variant(1, 4) : ring_variant(2, 2);
+        else if (mode != M_FUSED)
+            v = r == 32 ? team_default_variant(r, dtype) : ring_variant(2, 2);
+    } else if (mode == M_SDDMM && r >= 128) {
+        v = ring_variant(2, 2);
+        v.u = 2;
+        v.mb = r == 128 ? 3 : 2;
+    } else if (mode == M_BWD_ROW && r == 256) {
+        v = ring_variant(2, 2);
+    }
+    v.own = true;
     return v;
 }
 

@@ -53,6 +53,18 @@ __device__ __forceinline__ void unpack_bf16x8(const uint4 q, float *f)
     f[6] = __uint_as_float(q.w << 16); f[7] = __uint_as_float(q.w & 0xffff0000u);
 }
 
+// The 16 bytes q of a row of T as floats.
+template <typename T>
+__device__ __forceinline__ void unpack16(const uint4 q, float *f)
+{
+    if constexpr (sizeof(T) == 2) {
+        unpack_bf16x8(q, f);
+    } else {
+        f[0] = __uint_as_float(q.x); f[1] = __uint_as_float(q.y);
+        f[2] = __uint_as_float(q.z); f[3] = __uint_as_float(q.w);
+    }
+}
+
 // Row loads and stores with fixed cache operators: STREAM = read once
 // (ld.global.cs), else the read-only path.
 template <typename T, int R, bool STREAM>
@@ -283,7 +295,9 @@ __device__ __forceinline__ void store_bf16x8(uint16_t *p, const float *f)
 //
 // team_pass_body does the work of team `gid` (every lane of the warp must
 // call it; lanes whose team is not active only join the shuffles).
-template <int MODE, typename T, int R, int VPL, int NG, int U, bool CHECK = false>
+// RAW: the gathers of the pass over S^T all before any is widened (15 more
+// registers, which the batch kernel has not).
+template <int MODE, typename T, int R, int VPL, int NG, int U, bool CHECK = false, bool RAW = true>
 __device__ __forceinline__ void team_pass_body(const PassArgs &a, long long gid, bool active)
 {
     using TS = TeamShape<T, R, VPL, NG>;
@@ -332,17 +346,56 @@ __device__ __forceinline__ void team_pass_body(const PassArgs &a, long long gid,
     auto batch = [&](const int (&jj)[U], const int (&sidx)[U], const float (&sv)[U], int first) {
         float y[U][E];
         float h[MODE == M_BWD_COL ? U : 1][E];
+        if constexpr (MODE == M_BWD_COL && RAW) {
+            // two rows per nonzero: the raw words of all of them first, unpacked
+            // together (with each row widened beside its loads the pass waited
+            // between them: GB300, R-MAT 2^22, r = 64, bfloat16, 2.84 -> 2.74 ms;
+            // the roles with one row per nonzero gain nothing)
+            constexpr int Q = TS::EPV / 4;   // float4 per vector of T
+            uint4 yw[U][VPL];
+            float4 hw[U][VPL * Q];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (jj[u] >= 0) {
-                team_load<T, VPL, G>(ld, Y + (size_t)jj[u] * R, lig, y[u], true);
-                if constexpr (MODE == M_BWD_COL)
-                    team_load_f32<T, VPL, G>(ld, a.H + (size_t)jj[u] * R, lig, h[u], true);
-            } else {
+            for (int u = 0; u < U; ++u) {
+                const uint4 *yp = reinterpret_cast<const uint4 *>(Y + (size_t)jj[u] * R) + lig;
+                const float4 *hp =
+                    reinterpret_cast<const float4 *>(a.H + (size_t)jj[u] * R) + lig * Q;
 #pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    y[u][e] = 0.f;
-                    if constexpr (MODE == M_BWD_COL) h[u][e] = 0.f;
+                for (int v = 0; v < VPL; ++v) {
+                    yw[u][v] = make_uint4(0u, 0u, 0u, 0u);
+                    if (jj[u] >= 0)
+                        yw[u][v] = __ldg(yp + v * G);
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) {
+                        hw[u][v * Q + q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (jj[u] >= 0)
+                            hw[u][v * Q + q] = __ldg(hp + v * G * Q + q);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+#pragma unroll
+                for (int v = 0; v < VPL; ++v)
+                    unpack16<T>(yw[u][v], &y[u][v * TS::EPV]);
+#pragma unroll
+                for (int q = 0; q < E / 4; ++q) {
+                    h[u][4 * q] = hw[u][q].x; h[u][4 * q + 1] = hw[u][q].y;
+                    h[u][4 * q + 2] = hw[u][q].z; h[u][4 * q + 3] = hw[u][q].w;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (jj[u] >= 0) {
+                    team_load<T, VPL, G>(ld, Y + (size_t)jj[u] * R, lig, y[u], true);
+                    if constexpr (MODE == M_BWD_COL)
+                        team_load_f32<T, VPL, G>(ld, a.H + (size_t)jj[u] * R, lig, h[u], true);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        y[u][e] = 0.f;
+                        if constexpr (MODE == M_BWD_COL) h[u][e] = 0.f;
+                    }
                 }
             }
         }
