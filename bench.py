@@ -1053,6 +1053,7 @@ def run_batched(args, rank, world, local_rank):
 
     nnz = [it["ci"].numel() for it in items]
     rs = [it["plan"].r for it in items]
+    ring = [it["plan"].info()["variant"] >= 20000 for it in items]
     units_step = float(sum(z * r for z, r in zip(nnz, rs)))
     value = whole_job_value(units_step, K, world, elapsed_ms)
     fwd_bytes = sum(gather_model_bytes(it["plan"].m, z, r, 2, True) for it, z, r in zip(items, nnz, rs))
@@ -1071,8 +1072,8 @@ def run_batched(args, rank, world, local_rank):
         "config": {"workload": wl.WORKLOADS[5], "matrices": len(items), "rows": int(sum(
             it["plan"].m for it in items)), "nnz": int(sum(nnz)), "r_mix": {
             str(r): rs.count(r) for r in (32, 64, 128)},
-            "step": "batched FusedMMA forward + backward (dA, dB, ds), one persistent launch "
-                    "each, replayed from CUDA graphs; units = sum nnz*r per step",
+            "step": "batched FusedMMA forward + backward (dA, dB, ds), persistent launches "
+                    "replayed from CUDA graphs; units = sum nnz*r per step",
             "l2": "not flushed: the batch's operands total several GB",
             "parallelism": f"replicas x{args.gpus}", "scale_rows": args.scale},
         "roofline": {"bound": "hbm", "kernel": dom_name, "achieved": achieved, "peak": peak,
@@ -1093,9 +1094,10 @@ def run_batched(args, rank, world, local_rank):
                                    "plans with the library defaults (variant, long-row split)"},
         "e2e": {"value": units_step * world / (e2e_ms / 1e3), "unit": UNIT,
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms},
-        # one persistent launch per phase, and one that sums the partial rows of
-        # the R-MAT matrices' hub rows
-        "gpu_launches": 4 * K,
+        # persistent launches (the register-ring layouts of untuned plans: one in
+        # the forward and two in the backward phase; tuned codes: one each), and
+        # per phase one that sums the partial rows of the R-MAT matrices' hub rows
+        "gpu_launches": K * (2 + 3 * any(ring) + 2 * (not all(ring))),
         "clocks": clk,
         "setup": {"generate_s": gen_s, "autotune_s": tune_s, "tuned_groups": len(tuned),
                   "tuned_codes": tuned},

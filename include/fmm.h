@@ -338,16 +338,18 @@ int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
  * forward-only batch.  The batch stores the pointers: they must stay valid
  * and the buffers at those addresses are read and written by every launch.
  *
- * fmm_batch_forward queues a memset of the batch's work counter and one
+ * fmm_batch_forward queues a memset of the batch's work counters and a
  * persistent kernel in which warps pop work units (consecutive rows of one
  * matrix, matrix by matrix) until none are left, and, if a matrix has rows
  * longer than the default split size, a kernel that sums their partial rows;
  * fmm_batch_backward does the same for the adjoint passes (over S: dA, ds;
- * over S^T: dB).  Both can be captured in a CUDA graph.  Each item runs the
- * kernel variant its plan selects (fmm_plan_set_variant), if the batch
- * kernels have it for that width and role (codes 112, 114, 122, 212, 214,
- * 221, with at most 32 floats live per lane in the forward phase and 48 in
- * the backward phase), else the width's default with
+ * over S^T: dB), a kernel each.  Items whose plans ask for different kinds of
+ * kernels make two launches of one.  Both can be captured in a CUDA graph.
+ * Each item runs the kernel variant its plan selects (fmm_plan_set_variant),
+ * if the batch kernels have it for that width and role (codes 112, 114, 122,
+ * 212, 214, 221, with at most 32 floats live per lane in the forward phase and
+ * 48 in the backward phase; bfloat16 plans left to their default run its
+ * register-ring layouts), else the width's default team layout with
  * fewer nonzeros per batch.  Results equal the per-item calls with the same variants
  * bit for bit.  Calls on one batch must be ordered (one stream).
  */

@@ -25,12 +25,13 @@
 // ends evenly.  64 matrices, rows log-uniform in [1e3, 2e5], r of 32, 64 and
 // 128, bfloat16 (GB300): forward 4.08 -> 1.97 ms, backward 7.71 -> 6.09, with
 // the rows above the default size cut into chunks; uncut, the hub row of the
-// largest matrix alone took the 4.08 ms.
+// largest matrix alone took the 4.08 ms.  With the register-ring layouts, the
+// pass arguments in shared memory and smaller units 1.36 and 5.21 ms.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
 
-#include "fmm_rows.cuh"
+#include "fmm_pipe.cuh"
 
 namespace fmm {
 
@@ -38,9 +39,6 @@ struct BatchItemDev {
     PassArgs fwd;       // over S: FusedMMA
     PassArgs bwd_row;   // over S: dA (and ds)
     PassArgs bwd_col;   // over S^T: dB
-    int32_t code_fwd;   // (r << 16) | variant code of each role
-    int32_t code_row;
-    int32_t code_col;
 };
 
 // 128 columns (or fewer) of one split row: the sum of `chunks` partial rows,
@@ -135,29 +133,121 @@ __device__ __forceinline__ void run_code(int code, const PassArgs &a, int begin,
 #undef FMM_BATCH_CASE
 }
 
+// Items of bfloat16 plans left to their own choice: the layouts of
+// role_variant, in a kernel of their own (128 registers a thread, which the
+// team codes above would only pay for).
+template <int MODE, int R, int VPL, int RING>
+__device__ __forceinline__ void run_ring_unit(const PassArgs &a, int begin, int count)
+{
+    constexpr int G = TeamShape<bf16_t, R, VPL, 1>::G, TPW = 32 / G;
+    const int lane = threadIdx.x & 31;
+    for (int t0 = 0; t0 < count; t0 += TPW) {
+        const int t = t0 + lane / G;
+        pipe_pass_body<MODE, bf16_t, R, VPL, 1, RING, 1, false>(a, (long long)begin + t, t < count);
+    }
+}
+
+constexpr int kRingCode = 9;   // in place of a team code
+
+// Vectors per lane of the ring layouts of role_variant (0: the team kernel).
+template <int MODE>
+constexpr int ring_vpl(int r)
+{
+    return MODE != M_BWD_COL ? 2 : r == 32 ? 0 : r == 64 ? 1 : 2;
+}
+template <int MODE>
+constexpr int ring_depth(int r)
+{
+    return MODE == M_FUSED ? (r == 128 ? 4 : 2) : MODE == M_BWD_ROW ? 4 : r == 64 ? 4 : 2;
+}
+
+template <int MODE>
+__device__ __forceinline__ void run_ring(int r, const PassArgs &a, int begin, int count)
+{
+    switch (r) {
+    case 32:
+        if constexpr (ring_vpl<MODE>(32) == 0)
+            run_unit<MODE, bf16_t, 32, 1, 1, 2>(a, begin, count);
+        else
+            run_ring_unit<MODE, 32, ring_vpl<MODE>(32), ring_depth<MODE>(32)>(a, begin, count);
+        return;
+    case 64: run_ring_unit<MODE, 64, ring_vpl<MODE>(64), ring_depth<MODE>(64)>(a, begin, count); return;
+    case 128: run_ring_unit<MODE, 128, ring_vpl<MODE>(128), ring_depth<MODE>(128)>(a, begin, count); return;
+    case 256: run_ring_unit<MODE, 256, ring_vpl<MODE>(256), ring_depth<MODE>(256)>(a, begin, count); return;
+    }
+}
+
+// Hands the units of a list to the calling warp until none are left.  The next
+// unit's number is fetched while the current unit is worked on, and the pass
+// of the current matrix is kept in shared memory (one PassArgs per warp),
+// where it costs no registers: read from global memory by the row, it cost the
+// forward phase of the 64-matrix batch 1.72 ms in place of 1.41.
+template <typename Work>
+__device__ __forceinline__ void for_units(const BatchItemDev *items, const int4 *units, int n_units,
+                                          int *counter, unsigned char *shared, Work work)
+{
+    static_assert(sizeof(PassArgs) % 8 == 0, "copied in 8-byte words");
+    constexpr int WORDS = sizeof(PassArgs) / 8;
+    const PassArgs &pass = *reinterpret_cast<const PassArgs *>(shared);
+    const int lane = threadIdx.x & 31;
+    int next = 0, item = -1;
+    if (lane == 0)
+        next = atomicAdd(counter, 1);
+    for (;;) {
+        const int u = __shfl_sync(0xffffffffu, next, 0);
+        if (u >= n_units)
+            break;
+        if (lane == 0)
+            next = atomicAdd(counter, 1);
+        const int4 unit = __ldg(units + u);
+        const int kind = unit.y & 3, code = unit.y >> 2;
+        if (unit.x * 4 + kind != item) {   // uniform in the warp
+            item = unit.x * 4 + kind;
+            const BatchItemDev &it = items[unit.x];
+            const PassArgs &role = kind == U_FWD ? it.fwd : kind == U_BWD_ROW ? it.bwd_row : it.bwd_col;
+            const uint2 *from = reinterpret_cast<const uint2 *>(&role);
+            __syncwarp();
+            for (int w = lane; w < WORDS; w += 32) reinterpret_cast<uint2 *>(shared)[w] = from[w];
+            __syncwarp();
+        }
+        work(kind, code, pass, unit.z, unit.w);
+    }
+}
+
+// The ring layouts have a kernel per role: one for the whole backward phase
+// spilled at its 128 registers (6.2 ms in place of 1.86 + 3.6).
+template <int MODE>
+__global__ void __launch_bounds__(32, 16) ring_batch_kernel(const BatchItemDev *items,
+                                                            const int4 *units, int n_units,
+                                                            int *counter)
+{
+    __shared__ __align__(16) unsigned char shared[sizeof(PassArgs)];
+    for_units(items, units, n_units, counter, shared,
+              [](int, int, const PassArgs &a, int begin, int count) {
+                  run_ring<MODE>(a.r, a, begin, count);
+              });
+}
+
+// The team layouts one per phase: a kernel per role was slower (48 float32
+// matrices of 1e3 to 9e3 rows, a step 1.08 -> 1.36 ms; the rows of one matrix
+// are then gathered by both passes close together, and one launch fewer ends
+// unevenly).
 template <typename T, int PHASE>
 __global__ void __launch_bounds__(256) batch_kernel(const BatchItemDev *items, const int4 *units,
                                                     int n_units, int *counter)
 {
-    const int lane = threadIdx.x & 31;
-    for (;;) {
-        int u = 0;
-        if (lane == 0)
-            u = atomicAdd(counter, 1);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= n_units)
-            break;
-        const int4 unit = units[u];
-        const BatchItemDev &it = items[unit.x];
-        if constexpr (PHASE == 0) {
-            run_code<M_FUSED, T>(it.code_fwd, it.fwd, unit.z, unit.w);
-        } else {
-            if (unit.y == U_BWD_ROW)
-                run_code<M_BWD_ROW, T>(it.code_row, it.bwd_row, unit.z, unit.w);
-            else
-                run_code<M_BWD_COL, T>(it.code_col, it.bwd_col, unit.z, unit.w);
-        }
-    }
+    __shared__ __align__(16) unsigned char shared[8][(sizeof(PassArgs) + 15) / 16 * 16];
+    for_units(items, units, n_units, counter, shared[threadIdx.x >> 5],
+              [](int kind, int code, const PassArgs &a, int begin, int count) {
+                  if constexpr (PHASE == 0) {
+                      run_code<M_FUSED, T>(code, a, begin, count);
+                  } else {
+                      if (kind == U_BWD_ROW)
+                          run_code<M_BWD_ROW, T>(code, a, begin, count);
+                      else
+                          run_code<M_BWD_COL, T>(code, a, begin, count);
+                  }
+              });
 }
 
 template <typename T>
@@ -180,22 +270,27 @@ inline bool batch_listed(int code)
 
 using namespace fmm;
 
+constexpr int LISTS = 5;   // of work units: a kernel and a counter each
+
 struct fmm_batch {
     int32_t count = 0, dtype = 0, device = 0;
     bool has_bwd = false;
     BatchItemDev *d_items = nullptr;
-    int4 *d_units_fwd = nullptr, *d_units_bwd = nullptr;
-    int32_t n_fwd = 0, n_bwd = 0;
+    // units {item, 4 ((r << 16) | code) + kind, first work item, count} by list:
+    // the team kernels' by phase, then the ring kernels' by kind
+    int4 *d_units[LISTS] = {};
+    int32_t n_units[LISTS] = {};
     int *d_counters = nullptr;
     float *d_partials = nullptr;            // partial rows of chunks, every pass its own
     BatchSum *d_sums_fwd = nullptr, *d_sums_bwd = nullptr;
     int32_t n_sums_fwd = 0, n_sums_bwd = 0;
-    int grid_fwd = 0, grid_bwd = 0;
+    int grid[LISTS] = {};
 };
 
 namespace {
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+bool aligned32(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 
 // The variant a batch runs for a pass: the plan's, if the batch kernels
 // have it for this width and role, else the width's default.
@@ -222,8 +317,12 @@ int batch_code(int dtype, int mode, int r, const KernelVariant &v)
 }
 
 // Teams per warp of a variant code at width r.
-int teams_per_warp(int dtype, int r, int code)
+int teams_per_warp(int dtype, int r, int code, int mode)
 {
+    if (code == kRingCode) {
+        const int vpl = mode == M_BWD_COL ? ring_vpl<M_BWD_COL>(r) : ring_vpl<M_FUSED>(r);
+        return 32 / (r / 8 / std::max(1, vpl));
+    }
     const int vecs = r * (dtype == FMM_BF16 ? 2 : 4) / 16;
     const int base = vecs > 32 ? vecs / 32 : 1;
     const int V = (code / 100) * base, N = (code / 10) % 10;
@@ -231,12 +330,16 @@ int teams_per_warp(int dtype, int r, int code)
 }
 
 // Units of one pass: consecutive chunks, or consecutive rows within one
-// length bucket, about 512 nonzeros of work each (from the bucket's shortest
-// row length), a multiple of the warp's team count.
-void make_units(std::vector<int4> &out, const Side &side, int item, int kind, int tpw)
+// length bucket, about unit_nnz nonzeros of work each (from the bucket's
+// shortest row length), a multiple of the warp's team count.  Small units end
+// a launch evenly (48 float32 matrices of 1e3 to 9e3 rows, forward + backward:
+// units of 512 nonzeros 1120 us, 128: 770, 32: 631; the 64-matrix batch 6.89
+// ms, 6.57, 6.59), but a list of them is a table of 16 bytes each, so
+// fmm_batch_create aims at 2^19 units per role.
+void make_units(std::vector<int4> &out, const Side &side, int item, int code, int tpw, int unit_nnz)
 {
     for (int c = 0; c < side.n_chunks; c += tpw)
-        out.push_back(make_int4(item, kind, c, std::min(tpw, side.n_chunks - c)));
+        out.push_back(make_int4(item, code, c, std::min(tpw, side.n_chunks - c)));
     for (int key = 1; key < 256; ++key) {   // key 0: the split rows
         const int b0 = side.bucket_start[key], b1 = side.bucket_start[key + 1];
         if (b1 <= b0)
@@ -244,14 +347,14 @@ void make_units(std::vector<int4> &out, const Side &side, int item, int kind, in
         int per = tpw;
         if (key >= 136 && key < 255) {
             const int lo = length_key_min((uint32_t)key);
-            per = std::max(tpw, std::min(256, 512 / std::max(lo, 1)));
+            per = std::max(tpw, std::min(256, unit_nnz / std::max(lo, 1)));
             per = (per + tpw - 1) / tpw * tpw;
         } else if (key == 255) {
             per = 256;                        // empty rows: zero fills
         }
         const int shift = side.n_chunks - side.n_split;   // row position -> work item
         for (int t = b0; t < b1; t += per)
-            out.push_back(make_int4(item, kind, shift + t, std::min(per, b1 - t)));
+            out.push_back(make_int4(item, code, shift + t, std::min(per, b1 - t)));
     }
 }
 
@@ -268,12 +371,12 @@ void make_sums(std::vector<BatchSum> &out, const Side &side, const float *partia
                            std::min(128, r - k), r});
 }
 
-int grid_for(const void *kernel)
+int grid_for(const void *kernel, int threads)
 {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0);
     return std::max(1, sms * std::max(1, per));
 }
 
@@ -365,6 +468,9 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
         return e == cudaErrorMemoryAllocation ? FMM_ENOMEM : FMM_ECUDA;
     }
     float *next_partials = b->d_partials;
+    int64_t total_nnz = 0;
+    for (int i = 0; i < count; ++i) total_nnz += items[i].plan->nnz;
+    const int unit_nnz = (int)std::min<int64_t>(512, std::max<int64_t>(32, total_nnz >> 19));
     // matrices in the order of their work, most first
     std::vector<int> order(count);
     for (int i = 0; i < count; ++i) order[i] = i;
@@ -372,7 +478,7 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
         return items[x].plan->nnz * items[x].plan->r > items[y].plan->nnz * items[y].plan->r;
     });
     std::vector<BatchItemDev> host(count);
-    std::vector<int4> units_f, units_b;
+    std::vector<int4> units[LISTS];
     std::vector<BatchSum> sums_f, sums_b;
     for (int i : order) {
         const fmm_batch_item &it = items[i];
@@ -402,29 +508,37 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
         fill(d.bwd_row, p->rows, it.vals, it.A, it.B, it.G, it.dA, it.ds);
         PassArgs empty{};
         d.bwd_col = empty;
-        const int cf = batch_code(dtype, M_FUSED, p->r, p->rows.variant);
-        d.code_fwd = (p->r << 16) | cf;
-        make_units(units_f, p->rows, i, U_FWD, teams_per_warp(dtype, p->r, cf));
-        d.code_row = d.code_col = 0;
+        // the ring kernel loads gathered rows 32 bytes at a time
+        auto code_of = [&](int mode, const KernelVariant &v, const void *Y, const void *H) {
+            return v.own && dtype == FMM_BF16 && aligned32(Y) && aligned32(H)
+                       ? kRingCode
+                       : batch_code(dtype, mode, p->r, v);
+        };
+        auto list = [&](int kind, int code) -> std::vector<int4> & {
+            return units[code == kRingCode ? 2 + kind : kind != U_FWD];
+        };
+        const int cf = code_of(M_FUSED, p->rows.variant, it.B, nullptr);
+        const int rcode = p->r << 16;
+        make_units(list(U_FWD, cf), p->rows, i, 4 * (rcode | cf) + U_FWD, teams_per_warp(dtype, p->r, cf, M_FUSED),
+                   unit_nnz);
         if (bwd) {
-            const int cr = batch_code(dtype, M_BWD_ROW, p->r, p->rows.variant);
-            d.code_row = (p->r << 16) | cr;
+            const int cr = code_of(M_BWD_ROW, p->rows.variant, it.B, nullptr);
             make_sums(sums_b, p->rows, next_partials, it.dA, p->r);
             next_partials += (size_t)p->rows.n_chunks * p->r;
             if (it.dA || it.ds)
-                make_units(units_b, p->rows, i, U_BWD_ROW, teams_per_warp(dtype, p->r, cr));
+                make_units(list(U_BWD_ROW, cr), p->rows, i, 4 * (rcode | cr) + U_BWD_ROW,
+                           teams_per_warp(dtype, p->r, cr, M_BWD_ROW), unit_nnz);
             if (it.dB) {
                 fill(d.bwd_col, p->cols, it.vals, it.B, it.A, it.G, it.dB, nullptr);
                 make_sums(sums_b, p->cols, next_partials, it.dB, p->r);
                 next_partials += (size_t)p->cols.n_chunks * p->r;
-                const int cc = batch_code(dtype, M_BWD_COL, p->r, p->cols.variant);
-                d.code_col = (p->r << 16) | cc;
-                make_units(units_b, p->cols, i, U_BWD_COL, teams_per_warp(dtype, p->r, cc));
+                const int cc = code_of(M_BWD_COL, p->cols.variant, it.A, it.G);
+                make_units(list(U_BWD_COL, cc), p->cols, i, 4 * (rcode | cc) + U_BWD_COL,
+                           teams_per_warp(dtype, p->r, cc, M_BWD_COL), unit_nnz);
             }
         }
     }
-    b->n_fwd = (int32_t)units_f.size();
-    b->n_bwd = (int32_t)units_b.size();
+    for (int k = 0; k < LISTS; ++k) b->n_units[k] = (int32_t)units[k].size();
     b->n_sums_fwd = (int32_t)sums_f.size();
     b->n_sums_bwd = (int32_t)sums_b.size();
     cudaStream_t st = (cudaStream_t)stream;
@@ -437,11 +551,10 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
             e = cudaMemcpyAsync(*dst, v.data(), one * v.size(), cudaMemcpyHostToDevice, st);
     };
     upload(&b->d_items, host);
-    upload(&b->d_units_fwd, units_f);
-    upload(&b->d_units_bwd, units_b);
+    for (int k = 0; k < LISTS; ++k) upload(&b->d_units[k], units[k]);
     upload(&b->d_sums_fwd, sums_f);
     upload(&b->d_sums_bwd, sums_b);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, LISTS * sizeof(int));
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -450,13 +563,51 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
         return e == cudaErrorMemoryAllocation ? FMM_ENOMEM : FMM_ECUDA;
     }
     if (dtype == FMM_BF16) {
-        b->grid_fwd = grid_for((const void *)batch_kernel<bf16_t, 0>);
-        b->grid_bwd = grid_for((const void *)batch_kernel<bf16_t, 1>);
+        b->grid[0] = grid_for((const void *)batch_kernel<bf16_t, 0>, 256);
+        b->grid[1] = grid_for((const void *)batch_kernel<bf16_t, 1>, 256);
+        b->grid[2] = grid_for((const void *)ring_batch_kernel<M_FUSED>, 32);
+        b->grid[3] = grid_for((const void *)ring_batch_kernel<M_BWD_ROW>, 32);
+        b->grid[4] = grid_for((const void *)ring_batch_kernel<M_BWD_COL>, 32);
     } else {
-        b->grid_fwd = grid_for((const void *)batch_kernel<float, 0>);
-        b->grid_bwd = grid_for((const void *)batch_kernel<float, 1>);
+        b->grid[0] = grid_for((const void *)batch_kernel<float, 0>, 256);
+        b->grid[1] = grid_for((const void *)batch_kernel<float, 1>, 256);
     }
     *batch = b;
+    return FMM_OK;
+}
+
+// One phase: the units of the ring kernels, those of the team kernel, and the
+// sums of the split rows.
+static int run_phase(const fmm_batch *b, int phase, fmm_stream stream, const char *name)
+{
+    cudaStream_t st = (cudaStream_t)stream;
+    cudaError_t e = cudaMemsetAsync(b->d_counters, 0, LISTS * sizeof(int), st);
+    auto run = [&](auto *kernel, int list, int threads) {
+        if (e != cudaSuccess || b->n_units[list] == 0)
+            return;
+        kernel<<<b->grid[list], threads, 0, st>>>(b->d_items, b->d_units[list], b->n_units[list],
+                                                  b->d_counters + list);
+        e = cudaGetLastError();
+    };
+    const bool bf16 = b->dtype == FMM_BF16;
+    if (phase == 0) {
+        run(ring_batch_kernel<M_FUSED>, 2, 32);
+        run(bf16 ? batch_kernel<bf16_t, 0> : batch_kernel<float, 0>, 0, 256);
+    } else {
+        run(ring_batch_kernel<M_BWD_ROW>, 3, 32);
+        run(ring_batch_kernel<M_BWD_COL>, 4, 32);
+        run(bf16 ? batch_kernel<bf16_t, 1> : batch_kernel<float, 1>, 1, 256);
+    }
+    const int n_sums = phase ? b->n_sums_bwd : b->n_sums_fwd;
+    if (e == cudaSuccess && n_sums > 0) {
+        batch_sum_kernel<<<(n_sums + 3) / 4, 128, 0, st>>>(phase ? b->d_sums_bwd : b->d_sums_fwd,
+                                                          n_sums);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) {
+        set_error(name, e);
+        return FMM_ECUDA;
+    }
     return FMM_OK;
 }
 
@@ -466,24 +617,7 @@ int fmm_batch_forward(const fmm_batch *b, fmm_stream stream)
         set_error_msg("batch is NULL");
         return FMM_EINVAL;
     }
-    cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(b->d_counters, 0, sizeof(int), st);
-    if (e == cudaSuccess && b->n_fwd > 0) {
-        if (b->dtype == FMM_BF16)
-            batch_kernel<bf16_t, 0><<<b->grid_fwd, 256, 0, st>>>(b->d_items, b->d_units_fwd,
-                                                                 b->n_fwd, b->d_counters);
-        else
-            batch_kernel<float, 0><<<b->grid_fwd, 256, 0, st>>>(b->d_items, b->d_units_fwd,
-                                                                b->n_fwd, b->d_counters);
-        if (b->n_sums_fwd > 0)
-            batch_sum_kernel<<<(b->n_sums_fwd + 3) / 4, 128, 0, st>>>(b->d_sums_fwd, b->n_sums_fwd);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) {
-        set_error("fmm_batch_forward", e);
-        return FMM_ECUDA;
-    }
-    return FMM_OK;
+    return run_phase(b, 0, stream, "fmm_batch_forward");
 }
 
 int fmm_batch_backward(const fmm_batch *b, fmm_stream stream)
@@ -496,24 +630,7 @@ int fmm_batch_backward(const fmm_batch *b, fmm_stream stream)
         set_error_msg("batch built without G and gradient outputs (or without S^T)");
         return FMM_EUNSUPPORTED;
     }
-    cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(b->d_counters + 1, 0, sizeof(int), st);
-    if (e == cudaSuccess && b->n_bwd > 0) {
-        if (b->dtype == FMM_BF16)
-            batch_kernel<bf16_t, 1><<<b->grid_bwd, 256, 0, st>>>(b->d_items, b->d_units_bwd,
-                                                                 b->n_bwd, b->d_counters + 1);
-        else
-            batch_kernel<float, 1><<<b->grid_bwd, 256, 0, st>>>(b->d_items, b->d_units_bwd,
-                                                                b->n_bwd, b->d_counters + 1);
-        if (b->n_sums_bwd > 0)
-            batch_sum_kernel<<<(b->n_sums_bwd + 3) / 4, 128, 0, st>>>(b->d_sums_bwd, b->n_sums_bwd);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) {
-        set_error("fmm_batch_backward", e);
-        return FMM_ECUDA;
-    }
-    return FMM_OK;
+    return run_phase(b, 1, stream, "fmm_batch_backward");
 }
 
 int fmm_batch_destroy(fmm_batch *b)
@@ -522,8 +639,7 @@ int fmm_batch_destroy(fmm_batch *b)
         return FMM_OK;
     cudaDeviceSynchronize();
     cudaFree(b->d_items);
-    cudaFree(b->d_units_fwd);
-    cudaFree(b->d_units_bwd);
+    for (int4 *u : b->d_units) cudaFree(u);
     cudaFree(b->d_counters);
     cudaFree(b->d_partials);
     cudaFree(b->d_sums_fwd);

@@ -94,8 +94,11 @@ constexpr int kPipeBlock = 32;
 // as 256 / kPipeBlock blocks each (a register cap of 65536 / (256 MB) per
 // thread): the register ring trades rows in flight per team against teams
 // per SM.
-template <int MODE, typename T, int R, int VPL, int U, int RING, int MB, int REFILL, bool CHECK = false>
-__global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass_kernel(const PassArgs a)
+//
+// pipe_pass_body does the work of team `gid` (every lane of the warp must call
+// it; lanes whose team is not active only join the shuffles).
+template <int MODE, typename T, int R, int VPL, int U, int RING, int REFILL, bool CHECK>
+__device__ __forceinline__ void pipe_pass_body(const PassArgs &a, long long gid, bool active)
 {
     static_assert(MODE >= M_FUSED && MODE <= M_BWD_COL, "role");
     using TS = TeamShape<T, R, VPL, 1>;
@@ -120,9 +123,6 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
     const int tbase = lane & ~(G - 1);
     // the row word that word v of this lane holds
     auto widx = [lig](int v) { return WIDE ? lig * VPL + v : v * G + lig; };
-    const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const long long total = (long long)a.n_chunks + a.n_light;
-    bool active = gid < total;
     const Loader ld;
 
     int row = 0, beg = 0, end = 0, slot = -1;
@@ -433,6 +433,15 @@ __global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass
             }
         }
     }
+}
+
+template <int MODE, typename T, int R, int VPL, int U, int RING, int MB, int REFILL, bool CHECK = false>
+__global__ void __launch_bounds__(kPipeBlock, MB * (256 / kPipeBlock)) pipe_pass_kernel(const PassArgs a)
+{
+    constexpr int G = TeamShape<T, R, VPL, 1>::G;
+    const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const long long total = (long long)a.n_chunks + a.n_light;
+    pipe_pass_body<MODE, T, R, VPL, U, RING, REFILL, CHECK>(a, gid, gid < total);
 }
 
 template <int MODE, typename T, int R, int VPL, int U, int RING, int MB, int REFILL, bool CHECK = false>

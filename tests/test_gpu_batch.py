@@ -198,3 +198,53 @@ def test_batch_cuts_long_rows(hub, dtype):
             err = np.abs(it[k].double().cpu().numpy() - x)
             assert np.all(err <= 2 * (2 * r + deg + 4) * U32 * m + 1e-30), k
     batch.close()
+
+
+@pytest.mark.parametrize("offset", [0, 8])
+@pytest.mark.parametrize("r", [32, 64, 128, 256])
+def test_batch_of_default_bfloat16_plans(r, offset):
+    """bfloat16 plans left to their own choice run the register-ring layouts in
+    the batch: bitwise the per-matrix calls where every operand is 32-byte
+    aligned; operands 16 bytes further on (offset 8) take the team kernel.
+    Either way within the rounding bound of the oracle; forward and backward
+    twice, a matrix without nonzeros and one of a single row among them."""
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(r + offset)
+    items, host = [], []
+    for m, n, deg in ((300, 250, 9.0), (1, 40, 30.0), (50, 60, 0.0), (700, 90, 3.0)):
+        S = wl.random_csr(m, n, rng, mean_deg=deg, hubs=((0, 400),) if m == 700 else ())
+        f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+
+        def rows(k):
+            buf = torch.empty(k * r + offset, dtype=torch.bfloat16, device="cuda")
+            buf[offset:] = f(k * r).bfloat16()
+            return buf[offset:].view(k, r)
+        plan = fmm.Plan(torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda(), n, r,
+                        torch.bfloat16, split_nnz=1 << 30)
+        items.append(dict(plan=plan, vals=f(S.nnz), A=rows(m), B=rows(n), G=f(m, r),
+                          out=torch.empty(m, r, device="cuda"), dA=torch.empty(m, r, device="cuda"),
+                          dB=torch.empty(n, r, device="cuda"), ds=torch.empty(S.nnz, device="cuda")))
+        host.append(S)
+    batch = fmm.Batch(items)
+    for _ in range(2):
+        for it in items:
+            for k in ("out", "dA", "dB", "ds"):
+                it[k].fill_(float("nan"))
+        batch.forward()
+        batch.backward()
+    for it, S in zip(items, host):
+        p = it["plan"]
+        want = (fmm.fusedmm(p, it["vals"], it["A"], it["B"]),
+                *fmm.fusedmm_bwd(p, it["vals"], it["A"], it["B"], it["G"]))
+        a, b, s, g = (it[k].double().cpu().numpy() for k in ("A", "B", "vals", "G"))
+        ref = [oracle.fusedmm(S.row_ptr, S.col_idx, s, a, b, S.n),
+               *oracle.fusedmm_grad(S.row_ptr, S.col_idx, s, a, b, g, S.n)]
+        mag = [oracle.fusedmm(S.row_ptr, S.col_idx, abs(s), abs(a), abs(b), S.n),
+               *oracle.fusedmm_grad(S.row_ptr, S.col_idx, abs(s), abs(a), abs(b), abs(g), S.n)]
+        deg = max(int(S.degrees().max()), int(np.bincount(S.col_idx, minlength=S.n).max()))
+        for k, w, x, m in zip(("out", "dA", "dB", "ds"), want, ref, mag):
+            if offset == 0:
+                assert torch.equal(it[k], w), k
+            err = np.abs(it[k].double().cpu().numpy() - x)
+            assert np.all(err <= 2 * (2 * r + deg + 4) * U32 * m + 1e-30), k
+    batch.close()
