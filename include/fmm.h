@@ -150,8 +150,9 @@ typedef struct fmm_plan_options {
                                  Default: 32212 for bfloat16 rows (32412 for
                                  r = 128), 1042 for float32 rows of r = 128,
                                  else that team layout; SDDMM, SpMM and the
-                                 adjoints of a plan left to its default may
-                                 run another layout                          */
+                                 adjoints of a plan left to its default, and
+                                 passes bound by their longest rows, may run
+                                 another layout                              */
 } fmm_plan_options;
 
 typedef struct fmm_plan fmm_plan;   /* opaque */
@@ -319,7 +320,7 @@ int fmm_spmm_t_acc(const fmm_plan *plan, const float *v, const void *A, float *o
  * Kernel variant of a plan's row passes (the codes of
  * fmm_plan_options.variant; 0 leaves a side unchanged).  variant applies to
  * passes over S, variant_t to passes over S^T.  The code of a plan's default
- * gives the default back, with its own choice per operation.  Used by the
+ * for both gives the default back, with its own choice per operation and size.  Used by the
  * autotuner; calls already queued are not affected.
  */
 int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
@@ -350,8 +351,8 @@ int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
  * 212, 214, 221, with at most 32 floats live per lane in the forward phase and
  * 48 in the backward phase; bfloat16 plans left to their default run its
  * register-ring layouts), else the width's default team layout with
- * fewer nonzeros per batch.  Results equal the per-item calls with the same variants
- * bit for bit.  Calls on one batch must be ordered (one stream).
+ * fewer nonzeros per batch.  Results equal the per-item calls of plans with the
+ * same variants set bit for bit.  Calls on one batch must be ordered (one stream).
  */
 typedef struct fmm_batch fmm_batch;   /* opaque */
 

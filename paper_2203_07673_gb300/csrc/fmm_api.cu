@@ -155,6 +155,49 @@ int encode_variant(const KernelVariant &v)
     return v.vpl_mult * 100 + v.ng * 10 + v.u;
 }
 
+// Work items that get a warp each (fmm_wide.cuh); 0: none, the pass runs the
+// variant.  Worth it where the longest item, on one lane group, takes longer
+// than the gathers of the whole pass at 10 TB/s: about 0.19 us per nonzero for
+// the team and staged passes, 0.10 for the register ring.  Then every item of
+// 48 nonzeros or more gets a warp, and every item of 8 or more where the items
+// are few enough for a warp each.  Measured on GB300 (us, variant -> wide):
+//   float32, R-MAT of 2^14 vertices, r = 32 / 64 / 128 / 256:
+//     FusedMM 59 -> 20 / 54 -> 21 / 72 -> 25 / 56 -> 49
+//     adjoint over S 69 -> 15 / 67 -> 21 / 67 -> 32 / 70 -> 60
+//     adjoint over S^T 60 -> 16 / 56 -> 26 / 57 -> 48 / 66 -> 84
+//     SDDMM 55 -> 12 / 48 -> 19 / 23 -> 26 / 34 -> 56
+//     SpMM 47 -> 17 / 40 -> 15 / 41 -> 17 / 39 -> 26
+//   bfloat16, r = 32 / 64 / 128: FusedMM 32 -> 14 / 29 -> 22 / 28 -> 30, adjoint
+//     over S 41 -> 15 / 39 -> 22 / 38 -> 32; r = 32: adjoint over S^T 60 -> 21,
+//     SDDMM 54 -> 12, SpMM 45 -> 12
+//   Erdos-Renyi rows of 32, float32, r = 32, FusedMM / adjoint over S^T: 4096
+//     rows 8.7 -> 6.0 / 15 -> 6.2, 16384 rows (the line) 11.0 -> 10.9 / 17 -> 16
+// Past the line the pass is its gathers, and the variant moves them better: a
+// Zipf pattern of 2^16 rows at r = 128 takes 106 and would take 122.  A row of
+// r = 256 occupies a warp with one group, so there the line lies higher, and
+// the roles that lose (above, and bfloat16 past the widths named) stay out.
+static int wide_items(int mode, int dtype, const PassArgs &a)
+{
+    if (!a.bucket_start)
+        return 0;
+    const bool bf16 = dtype == FMM_BF16;
+    const bool ok = bf16 ? a.r == 32 || (mode == M_FUSED && a.r == 64) ||
+                               (mode == M_BWD_ROW && a.r <= 128)
+                         : mode == M_SDDMM ? a.r <= 64 : mode != M_BWD_COL || a.r <= 128;
+    if (!ok)
+        return 0;
+    const bool ring = bf16 && (mode == M_FUSED || mode == M_BWD_ROW);
+    const double chain = (ring ? 0.10 : 0.19) * a.longest;
+    const int row_bytes = a.r * ((bf16 ? 2 : 4) + (mode == M_BWD_COL ? 4 : 0));
+    const double work = (double)a.nnz * row_bytes / 1e7;
+    const bool high = bf16 || a.r == 256 || (mode == M_BWD_ROW && a.r == 128);
+    if (chain <= (high ? 1.6 : 0.9) * work)
+        return 0;
+    const long long items = (long long)a.n_chunks + a.n_light;
+    const uint32_t key = length_key(items <= (long long)sm_count() * 48 ? 8 : 48, INT32_MAX);
+    return a.n_chunks + a.bucket_start[key + 1] - a.bucket_start[1];
+}
+
 cudaError_t launch_pass(int mode, int dtype, const KernelVariant &given, const PassArgs &a,
                         cudaStream_t st)
 {
@@ -162,6 +205,12 @@ cudaError_t launch_pass(int mode, int dtype, const KernelVariant &given, const P
     const bool vec = fast_r(a.r) && aligned16(a.L) && aligned16(a.Y) && aligned16(a.H) &&
                      aligned16(a.out) && aligned16(a.out16) && aligned16(a.partials);
     const bool fwd = mode == M_FUSED || mode == M_SDDMM || mode == M_SPMM;
+    if (given.own && vec) {
+        const int n_wide = wide_items(mode, dtype, a);
+        if (n_wide > 0)
+            return dtype == FMM_BF16 ? launch_wide_bf16(mode, a, n_wide, st)
+                                     : launch_wide_f32(mode, a, n_wide, st);
+    }
     if (v.stages > 0 && vec && fwd) {
         return dtype == FMM_BF16 ? launch_staged_bf16(mode, v.vpl_mult, v.stages, a, st)
                                  : launch_staged_f32(mode, v.vpl_mult, v.stages, a, st);
@@ -279,6 +328,8 @@ int run_pass(const fmm_plan *p, const Side &side, int mode, const float *s, cons
     a.err = p->err;
     a.accumulate = accumulate ? 1 : 0;
     a.nnz = p->nnz;
+    a.longest = side.longest;
+    a.bucket_start = side.bucket_start.empty() ? nullptr : side.bucket_start.data();
     cudaError_t e = cudaSuccess;
     if (side.perm && s) {
         if (s == p->static_src && p->vals_static) {

@@ -396,13 +396,13 @@ int fmm_plan_set_variant(fmm_plan *p, int32_t variant, int32_t variant_t)
         set_error_msg("invalid plan or variant code");
         return FMM_EINVAL;
     }
-    // the code of the plan's own choice gives that choice back
+    // the code of the plan's own choice on both sides gives that choice back
     const KernelVariant own = default_variant(p->r, p->dtype, 0.0);
-    const int own_code = encode_variant(own);
+    const bool back = variant == variant_t && variant == encode_variant(own);
     if (variant)
-        p->rows.variant = variant == own_code ? own : decode_variant(variant);
+        p->rows.variant = back ? own : decode_variant(variant);
     if (variant_t)
-        p->cols.variant = variant_t == own_code ? own : decode_variant(variant_t);
+        p->cols.variant = back ? own : decode_variant(variant_t);
     return FMM_OK;
 }
 

@@ -170,13 +170,13 @@ __device__ __forceinline__ float ordered_sum(const float (&d)[EPV], int lig)
 
 // Accumulates into acc the nonzeros beg + first, beg + first + step, ... of
 // [beg, end): the share of one group of g lanes (lig = lane within it).
-// Every lane of the warp must call it.  ORD: in the generic kernel's order.
-template <int MODE, typename T, int VB, int E, bool ORD, bool CHECK>
+// Every lane of the warp must call it.  U: nonzeros per batch; ORD: in the
+// generic kernel's order.
+template <int MODE, typename T, int VB, int E, int U, bool ORD, bool CHECK>
 __device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, int end, int first,
                                            int step, int g, int lig, int nvec, float (&acc)[E])
 {
     constexpr int EPV = VB / (int)sizeof(T), VPL = E / EPV;
-    constexpr int U = E <= 8 ? 2 : 1;
     constexpr bool HAS_L = MODE != M_SPMM;
     constexpr bool TWO = MODE == M_BWD_ROW || MODE == M_BWD_COL;
     constexpr bool NZ = MODE == M_SDDMM || MODE == M_BWD_ROW;
@@ -324,27 +324,21 @@ __device__ __forceinline__ void flex_range(const PassArgs &a, int row, int beg, 
     }
 }
 
-// Blocks of two warps, as the team kernel's; register caps of 64 per thread
-// in the forward roles, 72 in the pass over S, 80 in the pass over S^T (none
-// spills).
-constexpr int kFlexBlock = 64;
-
-template <int MODE, typename T, int VB, int E, bool ORD = flex_ordered<MODE, T>(), bool CHECK = false>
-__global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 12 : MODE == M_BWD_ROW ? 14 : 16))
-    flex_pass_kernel(const PassArgs a, const FlexShape sh)
+// Work item `item` by a team of sh.g x sh.ng lanes.
+template <int MODE, typename T, int VB, int E, int U, bool ORD, bool CHECK>
+__device__ __forceinline__ void flex_item(const PassArgs &a, long long item, bool active,
+                                          const FlexShape &sh)
 {
     constexpr int EPV = VB / (int)sizeof(T), VPL = E / EPV;
     const int team = sh.g * sh.ng;
     const int lane = threadIdx.x & 31;
     const int lig = lane & (sh.g - 1);
     const int grp = (lane & (team - 1)) / sh.g;
-    const long long gid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / team;
-    bool active = gid < (long long)a.n_chunks + a.n_light;
     int row = 0, beg = 0, end = 0, slot = -1;
     if (active)
-        active = pass_item<CHECK>(a, gid, row, beg, end, slot);
+        active = pass_item<CHECK>(a, item, row, beg, end, slot);
     float acc[E];
-    flex_range<MODE, T, VB, E, ORD, CHECK>(a, row, beg, end, grp, sh.ng, sh.g, lig, sh.nvec, acc);
+    flex_range<MODE, T, VB, E, U, ORD, CHECK>(a, row, beg, end, grp, sh.ng, sh.g, lig, sh.nvec, acc);
     if constexpr (MODE != M_SDDMM) {
         for (int off = sh.g; off < team; off <<= 1) {
 #pragma unroll
@@ -373,6 +367,21 @@ __global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 1
                 flex_store_f32<EPV>(dst + (v * sh.g + lig) * EPV, &acc[v * EPV],
                                     a.accumulate && slot < 0);
     }
+}
+
+// Blocks of two warps, as the team kernel's; register caps of 64 per thread
+// in the forward roles, 72 in the pass over S, 80 in the pass over S^T (none
+// spills).
+constexpr int kFlexBlock = 64;
+
+template <int MODE, typename T, int VB, int E, bool ORD = flex_ordered<MODE, T>(), bool CHECK = false>
+__global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 12 : MODE == M_BWD_ROW ? 14 : 16))
+    flex_pass_kernel(const PassArgs a, const FlexShape sh)
+{
+    const long long gid =
+        ((long long)blockIdx.x * blockDim.x + threadIdx.x) / (sh.g * sh.ng);
+    flex_item<MODE, T, VB, E, E <= 8 ? 2 : 1, ORD, CHECK>(
+        a, gid, gid < (long long)a.n_chunks + a.n_light, sh);
 }
 
 template <int MODE, typename T, int VB, int E, bool ORD, bool CHECK>

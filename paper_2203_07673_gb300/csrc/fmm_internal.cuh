@@ -57,6 +57,7 @@ struct Side {
     float *partials = nullptr;        // 3 x n_chunks x r floats: partial rows (and
                                       // the attention pass's softmax states)
     int32_t max_nnz = 0;              // longest row
+    int32_t longest = 0;              // longest work item (chunk or light row)
     KernelVariant variant;            // kernel variant of passes over this side
     std::vector<int32_t> bucket_start;  // host: first position of each length key
                                         // in the row order (split rows, key 0,
@@ -128,6 +129,8 @@ struct PassArgs {
                                // bounded wait (NULL: not reported)
     int32_t accumulate = 0;    // 1: out += the pass's rows (else out =)
     int64_t nnz = 0;           // nonzeros of the pattern walked (launch rules)
+    int32_t longest = 0;       // nonzeros of its longest work item
+    const int32_t *bucket_start = nullptr;  // host: Side::bucket_start (launch rules)
     int32_t cols = 0;          // its columns: where a pass checks, an index outside
                                // [0, cols) counts as no nonzero
 };
@@ -144,6 +147,10 @@ cudaError_t launch_pass_bf16(int mode, int vpl_mult, int ng, int u, bool vec, co
 // per row at most.
 cudaError_t launch_flex_f32(int mode, const PassArgs &a, int vb, int ng, cudaStream_t st);
 cudaError_t launch_flex_bf16(int mode, const PassArgs &a, int vb, int ng, cudaStream_t st);
+// Passes with a warp for each of the first n_wide work items (fmm_wide.cuh);
+// vectorised widths.
+cudaError_t launch_wide_f32(int mode, const PassArgs &a, int n_wide, cudaStream_t st);
+cudaError_t launch_wide_bf16(int mode, const PassArgs &a, int n_wide, cudaStream_t st);
 // Widest row of the flexible pass (32 lanes of 16 elements).
 constexpr int32_t kFlexMaxR = 512;
 // Lanes of one group of the flexible pass for rows of r elements.

@@ -483,6 +483,7 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
     side.n_split = counters[0];
     side.max_nnz = counters[1];
     side.n_light = rows - side.n_split;
+    side.longest = std::min(side.max_nnz, split_nnz);
     if (rows == 1) {
         const int key = (int)length_key(side.max_nnz, split_nnz);
         for (int k = 0; k <= key; ++k)
