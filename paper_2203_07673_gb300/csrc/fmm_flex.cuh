@@ -16,12 +16,18 @@
 // and values of the next batch are loaded while the current one is used
 // (every lane of a group reads the same word: one request per group).
 // 8 elements per lane up to r = 256, as the team kernel's default layout (the
-// light register footprint keeps more rows in flight), 16 up to 512.
+// light register footprint keeps more rows in flight), 12 up to 384, 16 up to
+// 512; the roles that keep an order (below) as few as cover the row, since a
+// vector step costs the same whether it holds elements or not (Erdos-Renyi,
+// 60000 rows of 16, r = 25, float32, FusedMM: 149 us with 8 steps, 55 with 1).
 //
 // Measured on GB300 against the generic kernel, which it replaces for r <=
-// 512 (float32, r = 100, 60013 x 41999, 1.2M nonzeros, a hub row of 1200):
-// FusedMM 337 -> 115 us (88 with the order of its sums left free), adjoint over
-// S 378 -> 120, over S^T 325 -> 106.
+// 512 (us, Erdos-Renyi as above / Zipf rows, 60000 of 24): float32, r = 100:
+// FusedMM 215 -> 43 / 399 -> 108, SDDMM 124 -> 43 / 247 -> 70, SpMM 136 -> 29 /
+// 304 -> 79, adjoint over S 249 -> 67 / 488 -> 115, over S^T 260 -> 81 /
+// 381 -> 112; r = 201: FusedMM 253 -> 97 / 516 -> 169, SDDMM 131 -> 91 /
+// 251 -> 157, SpMM 211 -> 77 / 524 -> 134; bfloat16, r = 201: FusedMM 243 -> 161 /
+// 504 -> 263, SDDMM 133 -> 120 / 232 -> 197, SpMM 183 -> 136 / 435 -> 229.
 #pragma once
 
 #include "fmm_rows.cuh"
@@ -370,32 +376,64 @@ __device__ __forceinline__ void flex_item(const PassArgs &a, long long item, boo
 }
 
 // Blocks of two warps, as the team kernel's; register caps of 64 per thread
-// in the forward roles, 72 in the pass over S, 80 in the pass over S^T (none
-// spills).
+// in the forward roles, 72 in the pass over S, 80 in the pass over S^T (the
+// narrow vectors of the adjoints spill up to 40 bytes).
 constexpr int kFlexBlock = 64;
 
-template <int MODE, typename T, int VB, int E, bool ORD = flex_ordered<MODE, T>(), bool CHECK = false>
-__global__ void __launch_bounds__(kFlexBlock, E > 8 ? 8 : (MODE == M_BWD_COL ? 12 : MODE == M_BWD_ROW ? 14 : 16))
-    flex_pass_kernel(const PassArgs a, const FlexShape sh)
+template <int MODE, int E>
+constexpr int flex_min_blocks()
 {
-    const long long gid =
-        ((long long)blockIdx.x * blockDim.x + threadIdx.x) / (sh.g * sh.ng);
-    flex_item<MODE, T, VB, E, E <= 8 ? 2 : 1, ORD, CHECK>(
-        a, gid, gid < (long long)a.n_chunks + a.n_light, sh);
+    return E > 12 ? 8 : E > 8 ? (MODE == M_BWD_COL ? 8 : 10)
+         : MODE == M_BWD_COL ? 12 : MODE == M_BWD_ROW ? 14 : 16;
 }
 
-template <int MODE, typename T, int VB, int E, bool ORD, bool CHECK>
+// Roles whose order is free give the first n_wide items (chunks and rows of 64
+// nonzeros or more; the items are in order of length) all lane groups of a
+// warp; the other items take sh (Zipf rows, 60000 of 24, bfloat16, r = 25:
+// FusedMM 160 -> 73 us, SpMM 180 -> 79: a chunk of 256 nonzeros on one group of
+// four lanes was the pass).  G > 0: the lanes of a group as a constant, so the
+// vectors of a row lie at constant offsets (Erdos-Renyi, 60000 rows of 16,
+// r = 201: float32 FusedMM 156 -> 97, SDDMM 153 -> 91, bfloat16 adjoint over S
+// 270 -> 204).
+template <int MODE, typename T, int VB, int E, int G, bool ORD, bool CHECK>
+__global__ void __launch_bounds__(kFlexBlock, flex_min_blocks<MODE, E>())
+    flex_pass_kernel(const PassArgs a, FlexShape sh, int n_wide, int wide_blocks)
+{
+    const long long total = (long long)a.n_chunks + a.n_light;
+    long long item = ((long long)blockIdx.x - wide_blocks) * blockDim.x + threadIdx.x;
+    if constexpr (G > 0)
+        sh.g = G;
+    if constexpr (ORD || G == 32)
+        sh.ng = 1;
+    if (!ORD && G < 32 && (int)blockIdx.x < wide_blocks) {
+        sh.ng = 32 / sh.g;
+        item = (long long)blockIdx.x * (kFlexBlock / 32) + (threadIdx.x >> 5);
+        if (item >= n_wide)
+            item = total;
+    } else {
+        item = n_wide + item / (sh.g * sh.ng);
+    }
+    flex_item<MODE, T, VB, E, (ORD && E <= 4 ? 4 : E <= 8 ? 2 : 1), ORD, CHECK>(a, item,
+                                                                               item < total, sh);
+}
+
+template <int MODE, typename T, int VB, int E, int G, bool ORD, bool CHECK>
 cudaError_t launch_flex_shape(const PassArgs &a, int ng, cudaStream_t st)
 {
-    constexpr int EPV = VB / (int)sizeof(T);
+    constexpr int EPV = VB / (int)sizeof(T), WB = kFlexBlock / 32;
     FlexShape sh;
     sh.nvec = a.r / EPV;
-    sh.g = ORD ? 32 / EPV : flex_lanes(a.r);
+    sh.g = G > 0 ? G : flex_lanes(a.r);
     sh.ng = 1;
     while (!ORD && sh.ng < ng && sh.g * sh.ng < 32) sh.ng *= 2;
-    const long long total = (long long)a.n_chunks + a.n_light;
-    const long long blocks = (total * sh.g * sh.ng + kFlexBlock - 1) / kFlexBlock;
-    flex_pass_kernel<MODE, T, VB, E, ORD, CHECK><<<(unsigned)blocks, kFlexBlock, 0, st>>>(a, sh);
+    int n_wide = 0;
+    if (!ORD && a.bucket_start && sh.g * sh.ng < 32)
+        n_wide = a.n_chunks + a.bucket_start[length_key(64, INT32_MAX) + 1] - a.bucket_start[1];
+    const int wide_blocks = (n_wide + WB - 1) / WB;
+    const long long rest = (long long)a.n_chunks + a.n_light - n_wide;
+    const long long blocks = wide_blocks + (rest * sh.g * sh.ng + kFlexBlock - 1) / kFlexBlock;
+    flex_pass_kernel<MODE, T, VB, E, G, ORD, CHECK>
+        <<<(unsigned)blocks, kFlexBlock, 0, st>>>(a, sh, n_wide, wide_blocks);
     return cudaGetLastError();
 }
 
@@ -407,15 +445,34 @@ cudaError_t launch_flex_shape(const PassArgs &a, int ng, cudaStream_t st)
 template <int MODE, typename T, bool ORD = flex_ordered<MODE, T>(), bool CHECK = false>
 cudaError_t dispatch_flex(const PassArgs &a, int vb, int ng, cudaStream_t st)
 {
-    int e = a.r <= 256 ? 8 : 16;
     if constexpr (ORD) {
         while (vb > 4 && a.r > 32 * 16 / (vb / 4)) vb /= 2;
-        e = a.r <= 32 * 8 / (vb / 4) ? 8 : 16;
+#define FMM_FLEX(VB, E)                                                           \
+    if (vb == VB && a.r <= 32 * E / (VB / 4))                                     \
+        return launch_flex_shape<MODE, T, VB, E, 128 / VB, ORD, CHECK>(a, ng, st);
+        FMM_FLEX(16, 4) FMM_FLEX(16, 8) FMM_FLEX(16, 16)
+        FMM_FLEX(8, 2) FMM_FLEX(8, 4) FMM_FLEX(8, 8) FMM_FLEX(8, 16)
+        FMM_FLEX(4, 1) FMM_FLEX(4, 2) FMM_FLEX(4, 4) FMM_FLEX(4, 8) FMM_FLEX(4, 16)
+#undef FMM_FLEX
+        return cudaErrorInvalidValue;
     }
+    // 12 elements up to r = 384 where vectors allow it (Erdos-Renyi, 60000 rows
+    // of 16, r = 300, bfloat16, FusedMM: 199 us with 16 elements, 166 with 12)
 #define FMM_FLEX(VB)                                                              \
-    if (vb == VB)                                                                 \
-        return e == 8 ? launch_flex_shape<MODE, T, VB, 8, ORD, CHECK>(a, ng, st)  \
-                      : launch_flex_shape<MODE, T, VB, 16, ORD, CHECK>(a, ng, st);
+    if (vb == VB) {                                                               \
+        if (a.r <= 32)                                                            \
+            return launch_flex_shape<MODE, T, VB, 8, 0, ORD, CHECK>(a, ng, st);   \
+        if (a.r <= 64)                                                            \
+            return launch_flex_shape<MODE, T, VB, 8, 8, ORD, CHECK>(a, ng, st);   \
+        if (a.r <= 128)                                                           \
+            return launch_flex_shape<MODE, T, VB, 8, 16, ORD, CHECK>(a, ng, st);  \
+        if (a.r <= 256)                                                           \
+            return launch_flex_shape<MODE, T, VB, 8, 32, ORD, CHECK>(a, ng, st);  \
+        if constexpr (VB / sizeof(T) <= 4)                                        \
+            if (a.r <= 384)                                                       \
+                return launch_flex_shape<MODE, T, VB, 12, 32, ORD, CHECK>(a, ng, st); \
+        return launch_flex_shape<MODE, T, VB, 16, 32, ORD, CHECK>(a, ng, st);     \
+    }
     FMM_FLEX(16)
     FMM_FLEX(8)
     FMM_FLEX(4)

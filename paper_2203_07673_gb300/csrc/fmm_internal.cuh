@@ -151,7 +151,8 @@ cudaError_t launch_flex_bf16(int mode, const PassArgs &a, int vb, int ng, cudaSt
 // vectorised widths.
 cudaError_t launch_wide_f32(int mode, const PassArgs &a, int n_wide, cudaStream_t st);
 cudaError_t launch_wide_bf16(int mode, const PassArgs &a, int n_wide, cudaStream_t st);
-// Widest row of the flexible pass (32 lanes of 16 elements).
+// Widest row of the flexible pass (32 lanes of 16 elements); the generic pass
+// takes only wider ones and relies on it.
 constexpr int32_t kFlexMaxR = 512;
 // Lanes of one group of the flexible pass for rows of r elements.
 int flex_lanes(int32_t r);

@@ -605,10 +605,17 @@ __device__ __forceinline__ float warp_allreduce(float v)
     return v;
 }
 
-// Generic pass for rows wider than the flexible pass takes (fmm_flex.cuh),
-// any alignment: one warp per row or chunk,
-// scalar loads strided by lane, the output row accumulated in place (each
-// lane owns the columns k = lane + 32 t, so no two lanes touch one word).
+// Generic pass for rows wider than the flexible pass takes (fmm_flex.cuh), any
+// alignment: one warp per row or chunk, scalar loads strided by lane, the
+// output row accumulated in place (each lane owns the columns k = lane + 32 t,
+// so no two lanes touch one word).  What bounds it is the chain of loads of one
+// nonzero after the other, so a step loads W elements of each operand before
+// it uses any, and FusedMM keeps the first 512 columns of its rows, the output's
+// among them, in registers.  SDDMM alone lost by it (313 -> 329 us) and is
+// left to the compiler.  Measured on GB300 (Erdos-Renyi, 60000 rows of 16,
+// r = 515, float32 / bfloat16, us): FusedMM 886 -> 444 / 1409 -> 282, SpMM
+// 3240 -> 783 / 1129 -> 337, adjoint over S 4009 -> 1003 / 2798 -> 826, over
+// S^T 1847 -> 1017 / 2368 -> 917.
 template <int MODE, typename T, bool CHECK = false>
 __global__ void __launch_bounds__(256) row_pass_generic(const PassArgs a)
 {
@@ -628,11 +635,23 @@ __global__ void __launch_bounds__(256) row_pass_generic(const PassArgs a)
     if (ACC)
         dst = slot >= 0 ? a.partials + (size_t)slot * r
                         : (a.out ? a.out + (size_t)row * r : nullptr);
+    // FusedMM holds the first 32 HEAD columns of its rows in registers (r is
+    // more than that: narrower rows take the flexible pass)
+    constexpr int HEAD = MODE == M_FUSED ? kFlexMaxR / 32 : 1;
     // the accumulating calls add into the output row as it stands
     if (dst && !(a.accumulate && slot < 0))
-        for (int k = lane; k < r; k += 32)
+        for (int k = lane + (MODE == M_FUSED ? 32 * HEAD : 0); k < r; k += 32)
             dst[k] = 0.f;
     const T *Li = L ? L + (size_t)row * r : nullptr;
+    float l0[HEAD] = {}, acc[HEAD] = {};
+    if constexpr (MODE == M_FUSED) {
+#pragma unroll
+        for (int t = 0; t < HEAD; ++t) {
+            l0[t] = widen<T>(Li[lane + 32 * t]);
+            if (a.accumulate && slot < 0 && dst)
+                acc[t] = dst[lane + 32 * t];
+        }
+    }
     for (int p = beg; p < end; ++p) {
         const int j = pass_col<CHECK>(a, p);
         if (CHECK && j < 0)
@@ -640,15 +659,54 @@ __global__ void __launch_bounds__(256) row_pass_generic(const PassArgs a)
         const int sidx = a.perm ? __ldg(a.perm + p) : p;
         const float sv = a.s ? __ldg(a.s + (a.s_direct ? p : sidx)) : 1.f;
         const T *Yj = Y + (size_t)j * r;
+        const float *Hj = MODE == M_BWD_COL ? a.H + (size_t)j * r
+                        : MODE == M_BWD_ROW ? a.H + (size_t)row * r : nullptr;
         float d = 0.f, w = 0.f;
-        if constexpr (MODE != M_SPMM) {
-            for (int k = lane; k < r; k += 32) {
-                const float yk = widen<T>(Yj[k]);
-                d = fmaf(widen<T>(Li[k]), yk, d);
-                if constexpr (MODE == M_BWD_ROW)
-                    w = fmaf(a.H[(size_t)row * r + k], yk, w);
-                if constexpr (MODE == M_BWD_COL)
-                    w = fmaf(a.H[(size_t)j * r + k], widen<T>(Li[k]), w);
+        // W elements a lane at a time, all loads of a step before their use
+        constexpr int W = 4;
+        if constexpr (MODE == M_FUSED) {
+            float y[HEAD];
+#pragma unroll
+            for (int t = 0; t < HEAD; ++t)
+                y[t] = widen<T>(__ldg(Yj + lane + 32 * t));
+#pragma unroll
+            for (int t = 0; t < HEAD; ++t)
+                d = fmaf(l0[t], y[t], d);
+            for (int k = lane + 32 * HEAD; k < r; k += 32)
+                d = fmaf(widen<T>(Li[k]), widen<T>(Yj[k]), d);
+            const float c = sv * warp_allreduce(d);
+#pragma unroll
+            for (int t = 0; t < HEAD; ++t)
+                acc[t] = fmaf(c, y[t], acc[t]);
+            if (dst)
+                for (int k = lane + 32 * HEAD; k < r; k += 32)
+                    dst[k] = fmaf(c, widen<T>(Yj[k]), dst[k]);
+            continue;
+        }
+        if constexpr (MODE == M_SDDMM) {
+            for (int k = lane; k < r; k += 32)
+                d = fmaf(widen<T>(Li[k]), widen<T>(Yj[k]), d);
+            d = warp_allreduce(d);
+        } else if constexpr (MODE != M_SPMM) {
+            for (int k = lane; k < r; k += 32 * W) {
+                float y[W], l[W], h[W];
+#pragma unroll
+                for (int t = 0; t < W; ++t) {
+                    const bool in = k + 32 * t < r;
+                    y[t] = in ? widen<T>(__ldg(Yj + k + 32 * t)) : 0.f;
+                    l[t] = in ? widen<T>(__ldg(Li + k + 32 * t)) : 0.f;
+                    if constexpr (MODE == M_BWD_ROW || MODE == M_BWD_COL)
+                        h[t] = in ? __ldg(Hj + k + 32 * t) : 0.f;
+                }
+#pragma unroll
+                for (int t = 0; t < W; ++t)
+                    if (k + 32 * t < r) {
+                        d = fmaf(l[t], y[t], d);
+                        if constexpr (MODE == M_BWD_ROW)
+                            w = fmaf(h[t], y[t], w);
+                        if constexpr (MODE == M_BWD_COL)
+                            w = fmaf(h[t], l[t], w);
+                    }
             }
             d = warp_allreduce(d);
             if constexpr (MODE == M_BWD_ROW || MODE == M_BWD_COL)
@@ -662,23 +720,34 @@ __global__ void __launch_bounds__(256) row_pass_generic(const PassArgs a)
                 a.nzout[sidx] = d * w;
         }
         if (dst) {
-            if constexpr (MODE == M_FUSED) {
-                const float c = sv * d;
-                for (int k = lane; k < r; k += 32)
-                    dst[k] = fmaf(c, widen<T>(Yj[k]), dst[k]);
-            } else if constexpr (MODE == M_SPMM) {
-                for (int k = lane; k < r; k += 32)
-                    dst[k] = fmaf(sv, widen<T>(Yj[k]), dst[k]);
-            } else if constexpr (MODE == M_BWD_ROW) {
-                const float c = sv * w;
-                for (int k = lane; k < r; k += 32)
-                    dst[k] = fmaf(c, widen<T>(Yj[k]), dst[k]);
-            } else if constexpr (MODE == M_BWD_COL) {
-                const float c1 = sv * d, c2 = sv * w;
-                for (int k = lane; k < r; k += 32)
-                    dst[k] = fmaf(c1, a.H[(size_t)j * r + k],
-                                  fmaf(c2, widen<T>(Yj[k]), dst[k]));
+            const float c = MODE == M_SPMM ? sv : sv * w;
+            const float c1 = sv * d;
+            for (int k = lane; k < r; k += 32 * W) {
+                float y[W], h[W], o[W];
+#pragma unroll
+                for (int t = 0; t < W; ++t) {
+                    const bool in = k + 32 * t < r;
+                    y[t] = in ? widen<T>(__ldg(Yj + k + 32 * t)) : 0.f;
+                    if constexpr (MODE == M_BWD_COL)
+                        h[t] = in ? __ldg(Hj + k + 32 * t) : 0.f;
+                    o[t] = in ? dst[k + 32 * t] : 0.f;
+                }
+#pragma unroll
+                for (int t = 0; t < W; ++t)
+                    if (k + 32 * t < r) {
+                        o[t] = fmaf(c, y[t], o[t]);
+                        if constexpr (MODE == M_BWD_COL)
+                            o[t] = fmaf(c1, h[t], o[t]);
+                        dst[k + 32 * t] = o[t];
+                    }
             }
+        }
+    }
+    if constexpr (MODE == M_FUSED) {
+        if (dst) {
+#pragma unroll
+            for (int t = 0; t < HEAD; ++t)
+                dst[lane + 32 * t] = acc[t];
         }
     }
 }

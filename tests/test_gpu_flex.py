@@ -66,3 +66,32 @@ def test_sums_of_partial_rows(hub, r):
     S = wl.random_csr(300, 280, np.random.default_rng(hub + r), mean_deg=6,
                       hubs=((0, hub), (1, 700), (2, 100), (299, 600)))
     run_all(S, {"split_nnz": 64}, r, torch.float32, seed=hub)
+
+
+@DTYPES
+@pytest.mark.parametrize("r", [12, 31, 65, 96, 128 + 4, 257, 300, 384, 385, 545, 1030])
+def test_long_rows_beside_short_ones(r, dtype):
+    """Rows around the length that gets a warp each, unsplit and in chunks, at
+    the edges of the elements per lane and past the widest row."""
+    hubs = tuple((i * 9, d) for i, d in enumerate((0, 1, 62, 63, 64, 65, 66, 127, 128, 255, 256, 257,
+                                                   600)))
+    S = wl.random_csr(400, 500, np.random.default_rng(r), mean_deg=4, empty_frac=0.1, hubs=hubs)
+    run_all(S, {}, r, dtype, seed=r)
+
+
+@DTYPES
+@pytest.mark.parametrize("r", [25, 300, 513, 545, 1030])
+def test_accumulating_call(r, dtype):
+    from paper_2203_07673_gb300 import fmm
+    S, opts = pattern("hubs", r)
+    rng = np.random.default_rng(r)
+    f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+    plan = fmm.Plan(torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda(), S.n, r,
+                    dtype, **opts)
+    vals, A, B, base = f(S.nnz), f(S.m, r).to(dtype), f(S.n, r).to(dtype), f(S.m, r)
+    out = base.clone()
+    fmm.fusedmm_acc(plan, vals, A, B, out=out)
+    v, A64, B64, b = vals.cpu().numpy(), host64(A), host64(B), host64(base)
+    ref = b + oracle.fusedmm(S.row_ptr, S.col_idx, v, A64, B64, S.n)
+    mag = np.abs(b) + oracle.fusedmm(S.row_ptr, S.col_idx, np.abs(v), np.abs(A64), np.abs(B64), S.n)
+    assert_close("out", out, ref, mag, r, int(S.degrees().max()) + 1)
