@@ -46,6 +46,7 @@ KERNEL_SOURCES = [os.path.join(ROOT, "paper_2203_07673_gb300", "csrc", f)
                             "fmm_staged.cuh", "fmm_staged_f32.cu", "fmm_staged_bf16.cu",
                             "fmm_pipe.cuh", "fmm_pipe_f32.cu", "fmm_pipe_bf16.cu",
                             "fmm_stream.cuh", "fmm_stream_f32.cu", "fmm_stream_bf16.cu",
+                            "fmm_values.cu", "fmm_wide.cuh",
                             "fmm_internal.cuh", "fmm_plan.cu")]
 
 
@@ -640,9 +641,9 @@ def run_fmm(args, rank, world, local_rank):
     dom_name, dom_bytes = calls[dom]
     achieved = dom_bytes / (call_ms[dom] / 1e3) / 1e9
     traffic, traffic_note = read_traffic(w["name"], dom_name, w["dtype"])
-    # the value permutation of a pass over S^T: one launch, or two (scatter
-    # into windows, gather inside them) above two windows of 2^23 slots
-    perm_launches = 0 if vals is None else (2 if S.nnz > 2 * (1 << 23) else 1)
+    # the value permutation of a pass over S^T: one launch, or two (into the
+    # tiles' order, then tile by tile) between 2^24 and 2^28 nonzeros
+    perm_launches = 0 if vals is None else (2 if 1 << 24 < S.nnz <= 1 << 28 else 1)
     launches = {"fmm_fusedmm": 1 + (1 if info["split_rows"] else 0),
                 "fmm_fusedmm_t": 1 + (1 if info["split_cols"] else 0) + perm_launches,
                 "fmm_fusedmm_bwd": 2 + (1 if info["split_rows"] else 0)
@@ -883,13 +884,14 @@ def run_dist15d(args, rank, world, local_rank):
     units = 2.0 * nnz_total * r
     # library launches per step: per phase one FusedMMA pass (+ its combine
     # where rows are split) and one FusedMMB pass (+ combine) after the value
-    # permutation (one launch, or two above two windows of 2^23 slots)
+    # permutation (one launch, or two between 2^24 and 2^28 nonzeros)
     per_step = 0
     for pl in d.plans:
         info = pl.info()
         nnz_l = int(info.get("nnz", 0))
         per_step += 1 + (1 if info["split_rows"] else 0)
-        per_step += 1 + (1 if info["split_cols"] else 0) + (2 if nnz_l > 2 * (1 << 23) else 1)
+        per_step += 1 + (1 if info["split_cols"] else 0) + (
+            2 if 1 << 24 < nnz_l <= 1 << 28 else 1)
     d.close()
     if rank == 0:
         print(json.dumps({

@@ -320,8 +320,8 @@ int fmm_spmm_t_acc(const fmm_plan *plan, const float *v, const void *A, float *o
  * Kernel variant of a plan's row passes (the codes of
  * fmm_plan_options.variant; 0 leaves a side unchanged).  variant applies to
  * passes over S, variant_t to passes over S^T.  The code of a plan's default
- * for both gives the default back, with its own choice per operation and size.  Used by the
- * autotuner; calls already queued are not affected.
+ * for both gives the default back, with its own choice per operation and
+ * size.  Used by the autotuner; calls already queued are not affected.
  */
 int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
 
@@ -435,8 +435,9 @@ int fmm_gat_project(int32_t rows, int32_t heads, int32_t rh, const float *X, con
  * device that loads the library's module until exit): the order of the rows
  * by length, and the partial rows of rows longer than ch nonzeros, which are
  * split into chunks of ch, at least 128 and more where the array has no room
- * for that many partial rows.  r > 65536 returns FMM_EOVERFLOW.  The array is shared by all calls: calls that overlap on the
- * GPU race and give wrong results, so order them on one stream.  Every
+ * for that many partial rows.  r > 65536 returns FMM_EOVERFLOW.  The array is
+ * shared by all calls: calls that overlap on the GPU race and give wrong
+ * results, so order them on one stream.  Every
  * call looks the array's address up (cudaGetSymbolAddress, which allocates
  * nothing) on the current device, so the call still finds it after
  * cudaDeviceReset; the first call on a device may load the library's module
