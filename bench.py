@@ -642,8 +642,8 @@ def run_fmm(args, rank, world, local_rank):
     achieved = dom_bytes / (call_ms[dom] / 1e3) / 1e9
     traffic, traffic_note = read_traffic(w["name"], dom_name, w["dtype"])
     # the value permutation of a pass over S^T: one launch, or two (into the
-    # tiles' order, then tile by tile) between 2^24 and 2^28 nonzeros
-    perm_launches = 0 if vals is None else (2 if 1 << 24 < S.nnz <= 1 << 28 else 1)
+    # order of tiles or windows, then inside each) above 2^24 nonzeros
+    perm_launches = 0 if vals is None else (2 if S.nnz > 1 << 24 else 1)
     launches = {"fmm_fusedmm": 1 + (1 if info["split_rows"] else 0),
                 "fmm_fusedmm_t": 1 + (1 if info["split_cols"] else 0) + perm_launches,
                 "fmm_fusedmm_bwd": 2 + (1 if info["split_rows"] else 0)
@@ -884,14 +884,13 @@ def run_dist15d(args, rank, world, local_rank):
     units = 2.0 * nnz_total * r
     # library launches per step: per phase one FusedMMA pass (+ its combine
     # where rows are split) and one FusedMMB pass (+ combine) after the value
-    # permutation (one launch, or two between 2^24 and 2^28 nonzeros)
+    # permutation (one launch, or two above 2^24 nonzeros)
     per_step = 0
     for pl in d.plans:
         info = pl.info()
         nnz_l = int(info.get("nnz", 0))
         per_step += 1 + (1 if info["split_rows"] else 0)
-        per_step += 1 + (1 if info["split_cols"] else 0) + (
-            2 if 1 << 24 < nnz_l <= 1 << 28 else 1)
+        per_step += 1 + (1 if info["split_cols"] else 0) + (2 if nnz_l > 1 << 24 else 1)
     d.close()
     if rank == 0:
         print(json.dumps({
