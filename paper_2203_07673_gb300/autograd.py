@@ -16,6 +16,21 @@ import torch
 from . import fmm
 
 
+def gradients(plan, transpose, vals, A, B, G, need):
+    """(dA, dB, ds), None where ``need`` is False; raises for operands the plan
+    does not take (the native adjoint hands those over to it)."""
+    if plan.r <= 512:   # gradients rounded to A's dtype as they are stored
+        fn = fmm.fusedmm_t_bwd_typed if transpose else fmm.fusedmm_bwd_typed
+    else:
+        fn = fmm.fusedmm_t_bwd if transpose else fmm.fusedmm_bwd
+    dA, dB, ds = fn(plan, vals, A, B, G, need)
+    if dA is not None and dA.dtype != A.dtype:
+        dA = dA.to(A.dtype)
+    if dB is not None and dB.dtype != B.dtype:
+        dB = dB.to(B.dtype)
+    return dA, dB, ds
+
+
 class FusedMMFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, plan, vals, A, B, transpose=False):
@@ -35,15 +50,7 @@ class FusedMMFunction(torch.autograd.Function):
                 vals is not None and ctx.needs_input_grad[1])
         if not any(need):
             return None, None, None, None, None
-        if ctx.plan.r <= 512:   # gradients rounded to A's dtype as they are stored
-            fn = fmm.fusedmm_t_bwd_typed if ctx.transpose else fmm.fusedmm_bwd_typed
-        else:
-            fn = fmm.fusedmm_t_bwd if ctx.transpose else fmm.fusedmm_bwd
-        dA, dB, ds = fn(ctx.plan, vals, A, B, G, need)
-        if dA is not None and dA.dtype != A.dtype:
-            dA = dA.to(A.dtype)
-        if dB is not None and dB.dtype != B.dtype:
-            dB = dB.to(B.dtype)
+        dA, dB, ds = gradients(ctx.plan, ctx.transpose, vals, A, B, G, need)
         return None, ds, dA, dB, None
 
 
@@ -52,7 +59,7 @@ def fusedmm(plan, vals, A, B, transpose: bool = False):
     if plan.fast is not None:
         # the same function in native code (csrc/torch_calls.cpp), for ordinary
         # tensors outside of modes and transforms
-        out = fmm._calls.autograd(plan.fast, plan, vals, A, B, transpose)
+        out = fmm._calls.autograd(plan.fast, plan, vals, A, B, transpose, gradients)
         if out is not NotImplemented:
             return out
     return FusedMMFunction.apply(plan, vals, A, B, transpose)

@@ -148,6 +148,17 @@ const PlanCall kCalls[] = {
     {"fmm_fusedmm_t", "vAB", 'N', fmm_fusedmm_t, nullptr},
 };
 
+bool operand(char kind, const Tensor &t, const Plan &p)
+{
+    switch (kind) {
+    case 'v': case 'x': case 'V': return plain(t, at::kFloat, p.device) && is_list(t, p.nnz);
+    case 'A': return plain(t, p.dtype, p.device) && is_rows(t, p.m, p.r);
+    case 'B': return plain(t, p.dtype, p.device) && is_rows(t, p.n, p.r);
+    case 'M': return plain(t, at::kFloat, p.device) && is_rows(t, p.m, p.r);
+    default: return plain(t, at::kFloat, p.device) && is_rows(t, p.n, p.r);
+    }
+}
+
 bool operand(char kind, PyObject *o, const Plan &p, Tensor &t)
 {
     if (o == Py_None)
@@ -156,13 +167,7 @@ bool operand(char kind, PyObject *o, const Plan &p, Tensor &t)
     if (!q)
         return false;
     t = *q;
-    switch (kind) {
-    case 'v': case 'x': case 'V': return plain(t, at::kFloat, p.device) && is_list(t, p.nnz);
-    case 'A': return plain(t, p.dtype, p.device) && is_rows(t, p.m, p.r);
-    case 'B': return plain(t, p.dtype, p.device) && is_rows(t, p.n, p.r);
-    case 'M': return plain(t, at::kFloat, p.device) && is_rows(t, p.m, p.r);
-    default: return plain(t, at::kFloat, p.device) && is_rows(t, p.n, p.r);
-    }
+    return operand(kind, t, p);
 }
 
 PyObject *plan_call(const PlanCall &c, PyObject *const *args, Py_ssize_t n)
@@ -241,30 +246,69 @@ PyObject *cg_update(PyObject *, PyObject *const *args, Py_ssize_t n)
 
 // -------------------------------------------------------------- autograd
 
-// Keeps the Python plan (and with it the C plan) alive in a graph.
+struct Locked {   // the interpreter lock, taken for a scope
+    PyGILState_STATE s = PyGILState_Ensure();
+    ~Locked() { PyGILState_Release(s); }
+};
+
+// Keeps the Python plan (and with it the C plan) alive in a graph, and the
+// Python adjoint for operands that this one does not take.
 struct PlanRef : torch::CustomClassHolder {
     PlanPtr plan;
-    PyObject *owner;
-    PlanRef(PlanPtr p, PyObject *o) : plan(std::move(p)), owner(o) { Py_INCREF(owner); }
+    PyObject *owner, *gradients;
+    PlanRef(PlanPtr p, PyObject *o, PyObject *g) : plan(std::move(p)), owner(o), gradients(g)
+    {
+        Py_INCREF(owner);
+        Py_INCREF(gradients);
+    }
     ~PlanRef() override
     {
         if (!Py_IsInitialized())
             return;
-        const PyGILState_STATE s = PyGILState_Ensure();
+        const Locked lock;
         Py_DECREF(owner);
-        PyGILState_Release(s);
+        Py_DECREF(gradients);
     }
 };
+
+// The Python exception that is set, for a thread that gives up the lock.
+[[noreturn]] void throw_python_error()
+{
+    python_error e;
+    e.persist();
+    throw e;
+}
 
 // FmmError on a thread without the lock.
 [[noreturn]] void throw_status(int status, const char *where)
 {
-    const PyGILState_STATE s = PyGILState_Ensure();
+    const Locked lock;
     raise_status(status, where);
-    python_error e;
-    e.persist();
-    PyGILState_Release(s);
-    throw e;
+    throw_python_error();
+}
+
+// gradients(plan, transpose, vals, A, B, G, need) of autograd.py.
+tensor_list python_gradients(const PlanRef &ref, bool transpose, const Tensor &vals, const Tensor &A,
+                             const Tensor &B, const Tensor &G, bool need_A, bool need_B, bool need_s)
+{
+    const Locked lock;
+    PyObject *r = PyObject_CallFunction(
+        ref.gradients, "OONNNN(NNN)", ref.owner, transpose ? Py_True : Py_False,
+        THPVariable_Wrap(vals), THPVariable_Wrap(A), THPVariable_Wrap(B), THPVariable_Wrap(G),
+        PyBool_FromLong(need_A), PyBool_FromLong(need_B), PyBool_FromLong(need_s));
+    if (!r)
+        throw_python_error();
+    Tensor d[3];
+    for (int i = 0; i < 3; ++i) {
+        PyObject *x = PySequence_GetItem(r, i);
+        if (x && THPVariable_Check(x))
+            d[i] = THPVariable_Unpack(x);
+        Py_XDECREF(x);
+    }
+    Py_DECREF(r);
+    if (PyErr_Occurred())
+        throw_python_error();
+    return {d[0], d[1], d[2], Tensor(), Tensor()};
 }
 
 struct FusedMM : torch::autograd::Function<FusedMM> {
@@ -289,7 +333,8 @@ struct FusedMM : torch::autograd::Function<FusedMM> {
     static tensor_list backward(AutogradContext *ctx, tensor_list grads)
     {
         const auto holder = ctx->saved_data["plan"].toCapsule();
-        const Plan &p = *static_cast<const PlanRef *>(holder.get())->plan;
+        const PlanRef &ref = *static_cast<const PlanRef *>(holder.get());
+        const Plan &p = *ref.plan;
         const bool transpose = ctx->saved_data["transpose"].toBool();
         const auto saved = ctx->get_saved_variables();
         const Tensor &vals = saved[0], &A = saved[1], &B = saved[2];
@@ -300,6 +345,11 @@ struct FusedMM : torch::autograd::Function<FusedMM> {
         const bool need_A = ctx->needs_input_grad(0), need_B = ctx->needs_input_grad(1);
         Tensor ds, dA, dB;
         if (need_s || need_A || need_B) {
+            // what a saved-tensor hook gave back may have any layout, shape,
+            // dtype or device: the Python path raises its error
+            if ((vals.defined() && !operand('v', vals, p)) || !operand('A', A, p) ||
+                !operand('B', B, p) || !operand(transpose ? 'N' : 'M', G, p))
+                return python_gradients(ref, transpose, vals, A, B, G, need_A, need_B, need_s);
             const bool typed = p.dtype != at::kFloat && p.r <= kTypedMaxR;
             const at::ScalarType dt = typed ? p.dtype : at::kFloat;
             if (need_s)
@@ -328,11 +378,11 @@ struct FusedMM : torch::autograd::Function<FusedMM> {
     }
 };
 
-// autograd(plan capsule, plan object, vals, A, B, transpose)
+// autograd(plan capsule, plan object, vals, A, B, transpose, gradients)
 PyObject *autograd(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     HANDLE_TH_ERRORS
-    const PlanPtr *pp = n == 6 ? plan_of(args[0]) : nullptr;
+    const PlanPtr *pp = n == 7 ? plan_of(args[0]) : nullptr;
     if (!pp || !plain_mode())
         return not_implemented();
     const Plan &p = **pp;
@@ -345,7 +395,7 @@ PyObject *autograd(PyObject *, PyObject *const *args, Py_ssize_t n)
     const int transpose = PyObject_IsTrue(args[5]);
     if (transpose < 0)
         return nullptr;
-    auto ref = c10::make_intrusive<PlanRef>(*pp, args[1]);
+    auto ref = c10::make_intrusive<PlanRef>(*pp, args[1], args[6]);
     Tensor out;
     {
         Released unlocked;

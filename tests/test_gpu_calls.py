@@ -124,6 +124,41 @@ def test_saved_tensors():
         torch.autograd.grad(out, B, G)
 
 
+@pytest.mark.parametrize("which", ["vals", "A", "B"])
+@pytest.mark.parametrize("unpack", ["strides", "expanded", "narrower", "dtype", "host"])
+@pytest.mark.parametrize("transpose", [False, True], ids=["A", "B"])
+def test_unpacked_tensors_are_checked(transpose, unpack, which):
+    """A saved-tensor hook may give back any tensor: operands that the call
+    would refuse are refused in the adjoint too, with the same error, and the
+    same values in the right layout are taken."""
+    from paper_2203_07673_gb300 import autograd
+    plan, v, A, B, Gm, Gn = make()
+    G = Gn if transpose else Gm
+    leaves = dict(vals=v, A=A, B=B)
+    for t in leaves.values():
+        t.requires_grad_(True)
+    bad = leaves[which].detach()
+    bad = {"strides": lambda t: t.repeat_interleave(2, -1)[..., ::2],
+           "expanded": lambda t: t[:1].expand(t.shape), "narrower": lambda t: t[:-1].contiguous(),
+           "dtype": lambda t: t.double(), "host": lambda t: t.cpu()}[unpack](bad)
+
+    def step(swap):
+        packed = []
+        with torch.autograd.graph.saved_tensors_hooks(
+                lambda t: packed.append(t) or len(packed) - 1,
+                lambda i: bad if swap and packed[i].shape == leaves[which].shape
+                and packed[i].data_ptr() == leaves[which].data_ptr() else packed[i]):
+            out = autograd.fusedmm(plan, v, A, B, transpose=transpose)
+        assert len(packed) == 3
+        return torch.autograd.grad(out, (v, A, B), G)
+    with pytest.raises((TypeError, ValueError)) as want:
+        slow(plan, step, True)
+    with pytest.raises(type(want.value)) as got:
+        step(True)
+    assert str(got.value) == str(want.value)
+    assert all(torch.equal(x, y) for x, y in zip(step(False), slow(plan, step, False)))
+
+
 def test_other_ways_to_differentiate():
     from paper_2203_07673_gb300 import autograd
     plan, v, A, B, G, _ = make()
