@@ -26,7 +26,12 @@
 // lane, coalesced) handed out by shuffles; the current and the next block
 // are held, which covers a prefetch distance of up to one block.  Nonzeros
 // past the end of a row get value 0 and a zero row, so every batch runs the
-// same instructions and contributes exactly nothing.
+// same instructions and contributes exactly nothing, as long as the local row
+// is finite: 0 times an infinity or a NaN would put NaN into every element.
+// Warps with such a row take ring_rows_singly, which has no such positions: a
+// few instructions and a vote per row (leaving the positions out in the loop, a
+// comparison and a select per nonzero, took 2.80 ms in place of 2.59 for both
+// products of the Zipf rows, bfloat16, r = 64).
 //
 // Row layout: with two or more 16-byte words per lane, a lane owns
 // consecutive words of a row (lane l: words l VPL ... l VPL + VPL - 1), so a
@@ -95,6 +100,139 @@ constexpr int kPipeBlock = 32;
 // thread): the register ring trades rows in flight per team against teams
 // per SM.
 //
+// The row word that word v of lane lig of a group holds.
+template <typename T, int R, int VPL>
+__device__ __forceinline__ int pipe_word(int lig, int v)
+{
+    return VPL % 2 == 0 ? lig * VPL + v : v * TeamShape<T, R, VPL, 1>::G + lig;
+}
+
+// Stores the lane's elements of a finished row, or of a chunk's partial row.
+template <int MODE, typename T, int R, int VPL>
+__device__ __forceinline__ void pipe_store(const PassArgs &a, int row, int slot, int lig,
+                                           const float2 *acc2)
+{
+    constexpr int EPV = TeamShape<T, R, VPL, 1>::EPV, W2 = EPV / 2;
+    const Loader ld;
+    if constexpr ((MODE == M_BWD_ROW || MODE == M_BWD_COL) && sizeof(T) == 2) {
+        if (a.out16 && slot < 0) {
+#pragma unroll
+            for (int v = 0; v < VPL; ++v)
+                store_bf16x8(a.out16 + (size_t)row * R + pipe_word<T, R, VPL>(lig, v) * 8,
+                             reinterpret_cast<const float *>(&acc2[v * W2]));
+            return;
+        }
+    }
+    float *dst = slot >= 0 ? a.partials + (size_t)slot * R
+                           : (a.out ? a.out + (size_t)row * R : nullptr);
+    if (!dst)
+        return;
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) {
+#pragma unroll
+        for (int w = 0; w < W2; w += 2) {
+            const int k = pipe_word<T, R, VPL>(lig, v) * EPV + 2 * w;
+            const float2 p0 = acc2[v * W2 + w], p1 = acc2[v * W2 + w + 1];
+            out_store4(ld, dst + k, make_float4(p0.x, p0.y, p1.x, p1.y), a.accumulate && slot < 0);
+        }
+    }
+}
+
+// The rows of a warp one nonzero at a time, in the order of sums of
+// pipe_pass_body and without positions past their ends.  Every lane of the warp
+// calls it.
+template <int MODE, typename T, int R, int VPL, bool CHECK>
+__device__ __forceinline__ void ring_rows_singly(const PassArgs &a, int row, int beg, int end,
+                                                 int slot, bool active)
+{
+    using TS = TeamShape<T, R, VPL, 1>;
+    constexpr int G = TS::G, EPV = TS::EPV, W2 = EPV / 2, E2 = VPL * W2;
+    constexpr bool HAS_H = MODE == M_BWD_ROW || MODE == M_BWD_COL;
+    const int lig = threadIdx.x & (G - 1);
+    const Loader ld;
+    auto load = [&](const T *rows, int i, float2 *f) {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+            unpack2<T>(ld.u4(reinterpret_cast<const uint4 *>(rows + (size_t)i * R) +
+                                 pipe_word<T, R, VPL>(lig, v), true), f + v * W2);
+    };
+    auto load_h = [&](int i, float2 *f) {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+#pragma unroll
+            for (int q = 0; q < EPV / 4; ++q) {
+                const float4 x = ld.f4(a.H + (size_t)i * R + pipe_word<T, R, VPL>(lig, v) * EPV + 4 * q,
+                                       true);
+                f[v * W2 + 2 * q] = make_float2(x.x, x.y);
+                f[v * W2 + 2 * q + 1] = make_float2(x.z, x.w);
+            }
+    };
+    // <x, z>: even and odd elements of the lane, their sum, the group's lanes
+    auto dot = [&](const float2 *x, const float2 *z) {
+        float2 t2 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < E2; ++e) t2 = ffma2(x[e], z[e], t2);
+        float d = t2.x + t2.y;
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+        return d;
+    };
+    float2 l2[E2], h2[HAS_H ? E2 : 1], y2[E2], acc2[E2];
+#pragma unroll
+    for (int e = 0; e < E2; ++e) {
+        l2[e] = y2[e] = acc2[e] = make_float2(0.f, 0.f);
+        if constexpr (HAS_H) h2[e] = make_float2(0.f, 0.f);
+    }
+    const int n = end - beg;   // 0 where the team is not active
+    if (n > 0) {
+        load(static_cast<const T *>(a.L), row, l2);
+        if constexpr (MODE == M_BWD_ROW) load_h(row, h2);
+    }
+    const int wn = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
+    for (int k = 0; k < wn; ++k) {
+        const int p = beg + k;
+        const int j = k < n ? pass_col<CHECK>(a, p) : -1;
+        int sp = p;
+        float s = 0.f;
+        if (j >= 0) {
+            if (a.perm && (MODE == M_BWD_ROW || !a.s_direct))
+                sp = ld.idx(a.perm + p);
+            s = a.s ? ld.val(a.s + (a.s_direct ? p : sp)) : 1.f;
+            load(static_cast<const T *>(a.Y), j, y2);
+            if constexpr (MODE == M_BWD_COL) load_h(j, h2);
+        }
+        // (after the end of a row, the sums of the last nonzero's rows, unused)
+        const float d = dot(l2, y2);
+        float w = 0.f;
+        if constexpr (MODE == M_BWD_ROW) w = dot(h2, y2);
+        if constexpr (MODE == M_BWD_COL) w = dot(h2, l2);
+        if (j < 0)
+            continue;
+        if (MODE == M_BWD_ROW && a.nzout && lig == 0)
+            nz_store<MODE>(a, sp, d * w);
+        const float c1 = s * d, c2 = MODE == M_FUSED ? c1 : s * w;
+#pragma unroll
+        for (int e = 0; e < E2; ++e) {
+            acc2[e] = ffma2(make_float2(c2, c2), y2[e], acc2[e]);
+            if constexpr (MODE == M_BWD_COL)
+                acc2[e] = ffma2(make_float2(c1, c1), h2[e], acc2[e]);
+        }
+    }
+    if (active)
+        pipe_store<MODE, T, R, VPL>(a, row, slot, lig, acc2);
+}
+
+// The same as a call.  The adjoints call it, FusedMM has it inline: each way
+// leaves the loop of its pass as fast as it was (inline in the adjoints, the
+// R-MAT training step takes 5.47 ms in place of 5.40; called from FusedMM, the
+// Zipf rows 2.71 in place of 2.59).
+template <int MODE, typename T, int R, int VPL, bool CHECK>
+__device__ __noinline__ void ring_rows_singly_call(const PassArgs a, int row, int beg, int end,
+                                                   int slot, bool active)
+{
+    ring_rows_singly<MODE, T, R, VPL, CHECK>(a, row, beg, end, slot, active);
+}
+
 // pipe_pass_body does the work of team `gid` (every lane of the warp must call
 // it; lanes whose team is not active only join the shuffles).
 template <int MODE, typename T, int R, int VPL, int U, int RING, int REFILL, bool CHECK>
@@ -121,8 +259,7 @@ __device__ __forceinline__ void pipe_pass_body(const PassArgs &a, long long gid,
     const int lane = threadIdx.x & 31;
     const int lig = lane & (G - 1);
     const int tbase = lane & ~(G - 1);
-    // the row word that word v of this lane holds
-    auto widx = [lig](int v) { return WIDE ? lig * VPL + v : v * G + lig; };
+    auto widx = [lig](int v) { return pipe_word<T, R, VPL>(lig, v); };
     const Loader ld;
 
     int row = 0, beg = 0, end = 0, slot = -1;
@@ -262,6 +399,22 @@ __device__ __forceinline__ void pipe_pass_body(const PassArgs &a, long long gid,
 #pragma unroll
     for (int b = 0; b < RING - 1 + REFILL; ++b)
         issue_all(b, jc, b);
+    if constexpr (ACC && HAS_L) {
+        // 0 times every element of the local rows: NaN where one is not finite
+        float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < E2; ++e) {
+            z = ffma2(l2[e], make_float2(0.f, 0.f), z);
+            if constexpr (LOCAL_H) z = ffma2(h2[e], make_float2(0.f, 0.f), z);
+        }
+        if (__any_sync(0xffffffffu, z.x + z.y != 0.f)) {
+            if constexpr (MODE == M_FUSED)
+                ring_rows_singly<MODE, T, R, VPL, CHECK>(a, row, beg, end, slot, active);
+            else
+                ring_rows_singly_call<MODE, T, R, VPL, CHECK>(a, row, beg, end, slot, active);
+            return;
+        }
+    }
 
     for (int bk = 0; bk < wblocks; ++bk) {
 #pragma unroll
@@ -407,31 +560,8 @@ __device__ __forceinline__ void pipe_pass_body(const PassArgs &a, long long gid,
     }
 
     if constexpr (ACC) {
-        if (active) {
-            float *dst = slot >= 0 ? a.partials + (size_t)slot * R
-                                   : (a.out ? a.out + (size_t)row * R : nullptr);
-            if constexpr (TWO && sizeof(T) == 2) {
-                if (a.out16 && slot < 0) {
-#pragma unroll
-                    for (int v = 0; v < VPL; ++v)
-                        store_bf16x8(a.out16 + (size_t)row * R + widx(v) * 8,
-                                     reinterpret_cast<const float *>(&acc2[v * W2]));
-                    dst = nullptr;
-                }
-            }
-            if (dst) {
-#pragma unroll
-                for (int v = 0; v < VPL; ++v) {
-#pragma unroll
-                    for (int w = 0; w < W2; w += 2) {
-                        const int k = widx(v) * EPV + 2 * w;
-                        const float2 p0 = acc2[v * W2 + w], p1 = acc2[v * W2 + w + 1];
-                        out_store4(ld, dst + k, make_float4(p0.x, p0.y, p1.x, p1.y),
-                                   a.accumulate && slot < 0);
-                    }
-                }
-            }
-        }
+        if (active)
+            pipe_store<MODE, T, R, VPL>(a, row, slot, lig, acc2);
     }
 }
 

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(256, MB) stream_pass_kernel(const PassArgs a)
                 for (int off = G / 2; off > 0; off >>= 1)
                     d += __shfl_xor_sync(0xffffffffu, d, off);
                 if constexpr (MODE == M_FUSED) {
-                    const float c = sv * d;
+                    const float c = q < n ? sv * d : 0.f;   // (d may be NaN past the end)
                     const float2 c2 = make_float2(c, c);
 #pragma unroll
                     for (int e = 0; e < E2; ++e)
