@@ -644,10 +644,10 @@ def run_fmm(args, rank, world, local_rank):
     # the value permutation of a pass over S^T: one launch, or two (into the
     # order of tiles or windows, then inside each) above 2^24 nonzeros
     perm_launches = 0 if vals is None else (2 if S.nnz > 1 << 24 else 1)
-    launches = {"fmm_fusedmm": 1 + (1 if info["split_rows"] else 0),
-                "fmm_fusedmm_t": 1 + (1 if info["split_cols"] else 0) + perm_launches,
-                "fmm_fusedmm_bwd": 2 + (1 if info["split_rows"] else 0)
-                + (1 if info["split_cols"] else 0) + perm_launches}
+    launches = {"fmm_fusedmm": 1 + (1 if info["row_chunks"] else 0),
+                "fmm_fusedmm_t": 1 + (1 if info["col_chunks"] else 0) + perm_launches,
+                "fmm_fusedmm_bwd": 2 + (1 if info["row_chunks"] else 0)
+                + (1 if info["col_chunks"] else 0) + perm_launches}
     h2d = A_h.numel() * A_h.element_size() + B_h.numel() * B_h.element_size() + (
         0 if vals_h is None else vals_h.numel() * 4) + (0 if G_h is None else G_h.numel() * 4)
     d2h = (out_h.numel() + second_h.numel()) * 4 + (
@@ -889,8 +889,8 @@ def run_dist15d(args, rank, world, local_rank):
     for pl in d.plans:
         info = pl.info()
         nnz_l = int(info.get("nnz", 0))
-        per_step += 1 + (1 if info["split_rows"] else 0)
-        per_step += 1 + (1 if info["split_cols"] else 0) + (2 if nnz_l > 1 << 24 else 1)
+        per_step += 1 + (1 if info["row_chunks"] else 0)
+        per_step += 1 + (1 if info["col_chunks"] else 0) + (2 if nnz_l > 1 << 24 else 1)
     d.close()
     if rank == 0:
         print(json.dumps({
@@ -1240,8 +1240,8 @@ def run_als(args, rank, world, local_rank):
         # row update; the B side's SpMM^T first permutes c; split rows add
         # a combine per pass over S
         "gpu_launches": K * (2 * (3 + 2 * iters) + 1 + (
-            (2 + iters) if plan.info()["split_rows"] else 0) + (
-            (2 + iters) if plan.info()["split_cols"] else 0)),
+            (2 + iters) if plan.info()["row_chunks"] else 0) + (
+            (2 + iters) if plan.info()["col_chunks"] else 0)),
         "clocks": clk,
     }
     if not args.no_cpu_baseline:
@@ -1393,7 +1393,7 @@ def run_gat(args, rank, world, local_rank):
                 "layer": "X W (torch.matmul) + projections + attention"},
         "e2e": {"value": nnz * r / (e2e_ms / 1e3), "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms},
-        "gpu_launches": args.steps * (1 + (1 if info["split_rows"] else 0)), "clocks": clk,
+        "gpu_launches": args.steps * (1 + (1 if info["row_chunks"] else 0)), "clocks": clk,
     }
     if not args.no_cpu_baseline:
         line["cpu_baseline"] = gat_oracle_sample(rp, ci, f, g, Hp, heads, r, args.cpu_seconds)

@@ -102,10 +102,12 @@ typedef struct fmm_plan_options {
                                  summed in a fixed order; 0 = default:
                                  nnz / (4 x the teams of lanes that run at
                                  once for the kernel variant), clamped to
-                                 [256, 8192].  With a split_nnz that no row
-                                 (column) exceeds the plan counts as unsplit,
-                                 but its passes still cut rows longer than
-                                 the default size                             */
+                                 [256, 8192].  A split_nnz above nnz sets no
+                                 limit: rows are taken in chunks of the
+                                 default size, but none counts as split
+                                 (split_rows, fmm_batch_create).  The length
+                                 of the longest row and column keeps every
+                                 one whole                                    */
     int32_t variant;          /* kernel variant of the vectorised row passes:
                                  0 = chosen by the plan; else V*100 + N*10 + U
                                  with V = vectors per lane (as a multiple of
@@ -162,10 +164,11 @@ typedef struct fmm_plan_info {
     int64_t nnz;
     int32_t max_row_nnz;      /* longest row of S                          */
     int32_t max_col_nnz;      /* longest column of S (-1 without S^T)      */
-    int32_t split_rows;       /* rows of S split into chunks               */
-    int32_t split_cols;       /* columns of S split into chunks            */
-    int32_t row_chunks;       /* chunks over the split rows                */
-    int32_t col_chunks;       /* chunks over the split columns             */
+    int32_t split_rows;       /* rows of S split into chunks (0 where the
+                                 split_nnz given set no limit)             */
+    int32_t split_cols;       /* columns of S, in the same way             */
+    int32_t row_chunks;       /* chunks that the passes over S take        */
+    int32_t col_chunks;       /* chunks that the passes over S^T take      */
     int32_t split_nnz;        /* chunk size in nonzeros                    */
     int32_t variant;          /* kernel variant code of passes over S      */
     int32_t variant_t;        /* kernel variant code of passes over S^T    */
@@ -334,8 +337,9 @@ int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
  * B (n x r), out (m x r) receive FusedMMA; G (m x r), dA, dB, ds receive its
  * adjoint.  All plans must share one dtype and the current device, have r in
  * {32, 64, 128, 256}, and have no split rows or columns (create them with a
- * split_nnz at least the longest row and column); dense pointers must be
- * 16-byte aligned.  Items without G, or without any gradient output, make a
+ * split_nnz above nnz, which leaves the cutting of hub rows to the library, or
+ * at least the longest row and column, which keeps them whole); dense pointers
+ * must be 16-byte aligned.  Items without G, or without any gradient output, make a
  * forward-only batch.  The batch stores the pointers: they must stay valid
  * and the buffers at those addresses are read and written by every launch.
  *

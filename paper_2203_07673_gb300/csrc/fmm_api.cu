@@ -448,11 +448,10 @@ int fmm_plan_get_info(const fmm_plan *p, fmm_plan_info *info)
     info->nnz = p->nnz;
     info->max_row_nnz = p->rows.max_nnz;
     info->max_col_nnz = p->has_t ? p->cols.max_nnz : -1;
-    // rows cut although no row exceeds the plan's split_nnz do not count
-    info->split_rows = p->rows.split_asked ? p->rows.n_split : 0;
-    info->split_cols = p->cols.split_asked ? p->cols.n_split : 0;
-    info->row_chunks = p->rows.split_asked ? p->rows.n_chunks : 0;
-    info->col_chunks = p->cols.split_asked ? p->cols.n_chunks : 0;
+    info->split_rows = p->no_limit ? 0 : p->rows.n_split;
+    info->split_cols = p->no_limit ? 0 : p->cols.n_split;
+    info->row_chunks = p->rows.n_chunks;
+    info->col_chunks = p->cols.n_chunks;
     info->split_nnz = p->split_nnz;
     info->variant = encode_variant(p->rows.variant);
     info->variant_t = p->has_t ? encode_variant(p->cols.variant) : 0;

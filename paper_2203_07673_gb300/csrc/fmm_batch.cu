@@ -11,9 +11,9 @@
 // one launch.  The counter is cleared by a memset queued before each launch,
 // so both phases can be captured in a CUDA graph and replayed.
 //
-// Rows above the default split size are taken in the chunks of their plan
-// (plans must have no rows longer than their own split_nnz), with partial
-// rows in the batch's own memory, summed in chunk order by a second kernel.
+// Plans whose split_nnz set no limit take rows above the default split size in
+// chunks, here as in their own calls, with partial rows in the batch's own
+// memory, summed in chunk order by a second kernel.
 // Results are bitwise those of the per-matrix calls with the same variants.
 //
 // Units are handed out matrix by matrix, the matrices with the most work
@@ -429,8 +429,7 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
             set_error_msg("batch items need r in {32, 64, 128, 256}");
             return FMM_EUNSUPPORTED;
         }
-        if ((p->rows.n_split && p->rows.split_asked) ||
-            (p->has_t && p->cols.n_split && p->cols.split_asked)) {
+        if (!p->no_limit && (p->rows.n_split || (p->has_t && p->cols.n_split))) {
             set_error_msg("batch plans must have no split rows (create them with a large split_nnz)");
             return FMM_EUNSUPPORTED;
         }

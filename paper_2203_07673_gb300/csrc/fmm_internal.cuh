@@ -45,8 +45,6 @@ struct Side {
     // both products, 2.32 -> 2.27).
     int4 *items = nullptr;
     int32_t n_split = 0;              // rows split into chunks
-    bool split_asked = true;          // whether the rows in chunks are longer than
-                                      // the plan's split_nnz (see build_side)
     int32_t n_light = 0;              // rows - n_split
     int32_t n_chunks = 0;
     int4 *split = nullptr;            // {row, first chunk, chunk count, unused}
@@ -258,7 +256,8 @@ struct fmm_plan {
     int32_t m = 0, n = 0, r = 0, dtype = 0;
     int64_t nnz = 0;
     uint32_t flags = 0;
-    int32_t split_nnz = 512;
+    int32_t split_nnz = 512;   // nonzeros per chunk
+    bool no_limit = false;     // rows in chunks do not count as split
     int32_t variant = 0;              // requested variant code (0 = default)
     bool has_t = false;
     fmm::Side rows;   // S

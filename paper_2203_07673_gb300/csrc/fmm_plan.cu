@@ -425,13 +425,8 @@ static int build_runs(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
     return FMM_OK;
 }
 
-// split_nnz: the plan's; dflt: the default for the pattern.  A split_nnz
-// that no row exceeds (a plan for a batch, whose rows count as whole) still
-// cuts the rows above the default size: one lane group on a hub row of 10^4
-// nonzeros took 4 ms, longer than the rest of its pass (R-MAT 2 10^5
-// vertices).  The info then reports no split rows (split_asked).
 static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t split_nnz,
-                      int32_t dflt, int32_t r, Temps &tmp, cudaStream_t st, fmm_plan *plan)
+                      int32_t r, Temps &tmp, cudaStream_t st, fmm_plan *plan)
 {
     side.rows = rows;
     side.row_ptr = row_ptr;
@@ -441,20 +436,6 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
     row_keys_kernel<<<blocks_for(rows, 256), 256, 0, st>>>(row_ptr, rows, split_nnz, tmp.ka,
                                                            tmp.va, tmp.counters);
     FMM_TRY(cudaGetLastError(), "row keys");
-    if (split_nnz > dflt) {
-        int32_t seen[2];
-        FMM_TRY(cudaMemcpyAsync(seen, tmp.counters, sizeof(seen), cudaMemcpyDeviceToHost, st),
-                "read counters");
-        FMM_TRY(cudaStreamSynchronize(st), "plan sync");
-        if (seen[0] == 0 && seen[1] > dflt) {
-            side.split_asked = false;
-            split_nnz = dflt;
-            FMM_TRY(cudaMemsetAsync(tmp.counters, 0, 2 * sizeof(int32_t), st), "memset");
-            row_keys_kernel<<<blocks_for(rows, 256), 256, 0, st>>>(row_ptr, rows, split_nnz, tmp.ka,
-                                                                   tmp.va, tmp.counters);
-            FMM_TRY(cudaGetLastError(), "row keys");
-        }
-    }
     bool in_b = false;
     FMM_TRY(radix_sort(tmp.ka, tmp.va, tmp.kb, tmp.vb, rows, 8, tmp.ghist, st, &in_b),
             "row order sort");
@@ -631,8 +612,15 @@ int create_plan(const fmm_csr *S, int32_t r, int32_t dtype, const fmm_plan_optio
     const KernelVariant row_variant =
         p->variant ? decode_variant(p->variant)
                    : default_variant(r, dtype, S->m ? (double)S->nnz / S->m : 0.0);
-    const int32_t dflt_split = default_split_nnz(S->nnz, r, dtype, row_variant);
-    p->split_nnz = opt && opt->split_nnz > 0 ? opt->split_nnz : dflt_split;
+    // a split_nnz above nnz sets no limit (plans for a batch, whose rows must
+    // not count as split): the rows are still taken in chunks of the default
+    // size, since one lane group on a hub row of 10^4 nonzeros took 4 ms, longer
+    // than the rest of its pass (R-MAT 2 10^5 vertices).  Up to nnz it is what
+    // the caller says, the longest row included, which keeps every row whole.
+    const int32_t asked = opt ? opt->split_nnz : 0;
+    p->no_limit = (int64_t)asked > S->nnz;
+    p->split_nnz = asked > 0 && !p->no_limit ? asked
+                                             : default_split_nnz(S->nnz, r, dtype, row_variant);
     cudaGetDevice(&p->device);
     Temps tmp;
     const int64_t N = std::max<int64_t>({(int64_t)S->m, (int64_t)S->n, S->nnz, 1});
@@ -656,7 +644,7 @@ int create_plan(const fmm_csr *S, int32_t r, int32_t dtype, const fmm_plan_optio
     PLAN_TRY(dmalloc(&p->err, 1, p), "allocate error word");
     PLAN_TRY(cudaMemsetAsync(p->err, 0, sizeof(int32_t), st), "clear error word");
 
-    rc = build_side(p->rows, S->row_ptr, S->m, p->split_nnz, dflt_split, r, tmp, st, p);
+    rc = build_side(p->rows, S->row_ptr, S->m, p->split_nnz, r, tmp, st, p);
     if (rc) return fail(rc);
     p->rows.col_idx = S->col_idx;
     p->rows.perm = nullptr;
@@ -725,7 +713,7 @@ int create_plan(const fmm_csr *S, int32_t r, int32_t dtype, const fmm_plan_optio
                 p->perm_t, p->win_pos1, S->nnz, p->win_pos2);
             PLAN_TRY(cudaGetLastError(), "window positions");
         }
-        rc = build_side(p->cols, p->row_ptr_t, S->n, p->split_nnz, dflt_split, r, tmp, st, p);
+        rc = build_side(p->cols, p->row_ptr_t, S->n, p->split_nnz, r, tmp, st, p);
         if (rc) return fail(rc);
         p->cols.col_idx = p->col_idx_t;
         p->cols.perm = p->perm_t;

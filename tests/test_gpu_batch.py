@@ -251,3 +251,40 @@ def test_batch_of_default_bfloat16_plans(r, offset):
             err = np.abs(it[k].double().cpu().numpy() - x)
             assert np.all(err <= 2 * (2 * r + deg + 4) * U32 * m + 1e-30), k
     batch.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+def test_split_nnz_and_what_the_info_says(dtype):
+    """split_nnz up to nnz is the caller's: rows whole from the longest on, cut
+    below it, whatever the default; above nnz it sets no limit, and the info
+    tells the chunks and their size."""
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(5)
+    S = wl.random_csr(300, 250, rng, mean_deg=5, hubs=((0, 900), (5, 400)))
+    longest = max(int(S.degrees().max()), int(np.bincount(S.col_idx, minlength=S.n).max()))
+    deg, cdeg = S.degrees(), np.bincount(S.col_idx, minlength=S.n)
+    rp, ci = torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda()
+    f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+    A, B, out = f(S.m, 64).to(dtype), f(S.n, 64).to(dtype), torch.empty(S.m, 64, device="cuda")
+    chunks = lambda d, k: int(np.ceil(d[d > k] / k).sum())
+    for split, size in ((longest - 1, longest - 1), (longest, None), (S.nnz, None),
+                        (S.nnz + 1, 256), (1 << 30, 256)):
+        plan = fmm.Plan(rp, ci, S.n, 64, dtype, split_nnz=split)
+        i = plan.info()
+        if size is None:
+            assert i["split_rows"] == i["split_cols"] == i["row_chunks"] == i["col_chunks"] == 0
+        else:
+            assert i["split_nnz"] == size
+            assert (i["row_chunks"], i["col_chunks"]) == (chunks(deg, size), chunks(cdeg, size))
+            assert i["split_rows"] == ((deg > size).sum() if split <= S.nnz else 0)
+        item = dict(plan=plan, A=A, B=B, out=out)
+        if split == longest - 1:
+            with pytest.raises(fmm.FmmError):
+                fmm.Batch([item])
+            continue
+        batch = fmm.Batch([item])
+        batch.forward()
+        assert relF(out.double().cpu().numpy(),
+                    oracle.fusedmm(S.row_ptr, S.col_idx, None, A.double().cpu().numpy(),
+                                   B.double().cpu().numpy(), S.n)) <= 1e-5
+        batch.close()
