@@ -353,10 +353,11 @@ int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
  * Each item runs the kernel variant its plan selects (fmm_plan_set_variant),
  * if the batch kernels have it for that width and role (codes 112, 114, 122,
  * 212, 214, 221, with at most 32 floats live per lane in the forward phase and
- * 48 in the backward phase; bfloat16 plans left to their default run its
- * register-ring layouts), else the width's default team layout with
- * fewer nonzeros per batch.  Results equal the per-item calls of plans with the
- * same variants set bit for bit.  Calls on one batch must be ordered (one stream).
+ * 48 in the backward phase; plans left to their default run the layouts of
+ * their own calls), else the width's default team layout with
+ * fewer nonzeros per batch.  Results equal the per-item calls with the same
+ * variants bit for bit, those of plans left to their default among them.  Calls
+ * on one batch must be ordered (one stream).
  */
 typedef struct fmm_batch fmm_batch;   /* opaque */
 

@@ -161,37 +161,36 @@ int encode_variant(const KernelVariant &v)
 // the team and staged passes, 0.10 for the register ring.  Then every item of
 // 48 nonzeros or more gets a warp, and every item of 8 or more where the items
 // are few enough for a warp each.  Measured on GB300 (us, variant -> wide):
-//   float32, R-MAT of 2^14 vertices, r = 32 / 64 / 128 / 256:
-//     FusedMM 59 -> 20 / 54 -> 21 / 72 -> 25 / 56 -> 49
-//     adjoint over S 69 -> 15 / 67 -> 21 / 67 -> 32 / 70 -> 60
-//     adjoint over S^T 60 -> 16 / 56 -> 26 / 57 -> 48 / 66 -> 84
-//     SDDMM 55 -> 12 / 48 -> 19 / 23 -> 26 / 34 -> 56
-//     SpMM 47 -> 17 / 40 -> 15 / 41 -> 17 / 39 -> 26
-//   bfloat16, r = 32 / 64 / 128: FusedMM 32 -> 14 / 29 -> 22 / 28 -> 30, adjoint
-//     over S 41 -> 15 / 39 -> 22 / 38 -> 32; r = 32: adjoint over S^T 60 -> 21,
+//   float32, R-MAT of 2^14 vertices, r = 32 / 64 / 128 (256):
+//     FusedMM 60 -> 15 / 54 -> 15 / 72 -> 24 (56 -> 49)
+//     adjoint over S 70 -> 16 / 67 -> 16 / 67 -> 29
+//     adjoint over S^T 61 -> 18 / 56 -> 28 / 57 -> 47
+//     SDDMM 56 -> 12 / 48 -> 19
+//     SpMM 47 -> 15 / 40 -> 12 / 41 -> 17 (39 -> 25)
+//   bfloat16, r = 32 / 64 / 128: FusedMM 32 -> 14 / 29 -> 15, adjoint over S
+//     39 -> 15 / 41 -> 17 / 38 -> 26; r = 32: adjoint over S^T 60 -> 17,
 //     SDDMM 54 -> 12, SpMM 45 -> 12
 //   Erdos-Renyi rows of 32, float32, r = 32, FusedMM / adjoint over S^T: 4096
-//     rows 8.7 -> 6.0 / 15 -> 6.2, 16384 rows (the line) 11.0 -> 10.9 / 17 -> 16
+//     rows 8.7 -> 5.4 / 15 -> 8.7
 // Past the line the pass is its gathers, and the variant moves them better: a
-// Zipf pattern of 2^16 rows at r = 128 takes 106 and would take 122.  A row of
-// r = 256 occupies a warp with one group, so there the line lies higher, and
-// the roles that lose (above, and bfloat16 past the widths named) stay out.
+// Zipf pattern of 2^16 rows takes 106 at r = 128, float32, and would take 122;
+// in bfloat16, where the line is 3 (the register ring beside it takes the
+// registers), 36 and 47 at r = 32.  A row of r = 256 occupies a warp with one
+// group, so there the line lies higher, and the roles that lose (SDDMM from
+// r = 128 on, the adjoints at r = 256, bfloat16 past the widths named) stay out.
 static int wide_items(int mode, int dtype, const PassArgs &a)
 {
     if (!a.bucket_start)
         return 0;
     const bool bf16 = dtype == FMM_BF16;
-    const bool ok = bf16 ? a.r == 32 || (mode == M_FUSED && a.r == 64) ||
-                               (mode == M_BWD_ROW && a.r <= 128)
-                         : mode == M_SDDMM ? a.r <= 64 : mode != M_BWD_COL || a.r <= 128;
-    if (!ok)
+    if (!wide_role(mode, bf16, a.r))
         return 0;
     const bool ring = bf16 && (mode == M_FUSED || mode == M_BWD_ROW);
     const double chain = (ring ? 0.10 : 0.19) * a.longest;
     const int row_bytes = a.r * ((bf16 ? 2 : 4) + (mode == M_BWD_COL ? 4 : 0));
     const double work = (double)a.nnz * row_bytes / 1e7;
     const bool high = bf16 || a.r == 256 || (mode == M_BWD_ROW && a.r == 128);
-    if (chain <= (high ? 1.6 : 0.9) * work)
+    if (chain <= (ring ? 3.0 : high ? 1.6 : 0.9) * work)
         return 0;
     const long long items = (long long)a.n_chunks + a.n_light;
     const uint32_t key = length_key(items <= (long long)sm_count() * 48 ? 8 : 48, INT32_MAX);
@@ -208,8 +207,8 @@ cudaError_t launch_pass(int mode, int dtype, const KernelVariant &given, const P
     if (given.own && vec) {
         const int n_wide = wide_items(mode, dtype, a);
         if (n_wide > 0)
-            return dtype == FMM_BF16 ? launch_wide_bf16(mode, a, n_wide, st)
-                                     : launch_wide_f32(mode, a, n_wide, st);
+            return dtype == FMM_BF16 ? launch_wide_bf16(mode, a, n_wide, aligned32(a.Y), st)
+                                     : launch_wide_f32(mode, a, n_wide, false, st);
     }
     if (v.stages > 0 && vec && fwd) {
         return dtype == FMM_BF16 ? launch_staged_bf16(mode, v.vpl_mult, v.stages, a, st)

@@ -133,23 +133,29 @@ __device__ __forceinline__ void run_code(int code, const PassArgs &a, int begin,
 #undef FMM_BATCH_CASE
 }
 
-// Items of bfloat16 plans left to their own choice: the layouts of
-// role_variant, in a kernel of their own (128 registers a thread, which the
-// team codes above would only pay for).
-template <int MODE, int R, int VPL, int RING>
+// Items of plans left to their own choice: the ring layouts of role_variant, in
+// a kernel of their own (128 registers a thread, which the team codes above
+// would only pay for).
+template <int MODE, typename T, int R, int VPL, int RING>
 __device__ __forceinline__ void run_ring_unit(const PassArgs &a, int begin, int count)
 {
-    constexpr int G = TeamShape<bf16_t, R, VPL, 1>::G, TPW = 32 / G;
+    constexpr int G = TeamShape<T, R, VPL, 1>::G, TPW = 32 / G;
     const int lane = threadIdx.x & 31;
     for (int t0 = 0; t0 < count; t0 += TPW) {
         const int t = t0 + lane / G;
-        pipe_pass_body<MODE, bf16_t, R, VPL, 1, RING, 1, false>(a, (long long)begin + t, t < count);
+        pipe_pass_body<MODE, T, R, VPL, 1, RING, 1, false>(a, (long long)begin + t, t < count);
     }
 }
 
 constexpr int kRingCode = 9;   // in place of a team code
 
-// Vectors per lane of the ring layouts of role_variant (0: the team kernel).
+// Whether role_variant gives a role a layout of the ring kernels below.
+bool ring_role(int mode, int dtype, int r)
+{
+    return dtype == FMM_BF16 || (mode == M_BWD_ROW && r == 256);
+}
+
+// Vectors per lane of the ring layouts of bfloat16 rows (0: the team kernel).
 template <int MODE>
 constexpr int ring_vpl(int r)
 {
@@ -161,19 +167,26 @@ constexpr int ring_depth(int r)
     return MODE == M_FUSED ? (r == 128 ? 4 : 2) : MODE == M_BWD_ROW ? 4 : r == 64 ? 4 : 2;
 }
 
-template <int MODE>
+template <int MODE, typename T>
 __device__ __forceinline__ void run_ring(int r, const PassArgs &a, int begin, int count)
 {
-    switch (r) {
-    case 32:
-        if constexpr (ring_vpl<MODE>(32) == 0)
-            run_unit<MODE, bf16_t, 32, 1, 1, 2>(a, begin, count);
-        else
-            run_ring_unit<MODE, 32, ring_vpl<MODE>(32), ring_depth<MODE>(32)>(a, begin, count);
+    if constexpr (sizeof(T) == 4) {   // (r = 256)
+        run_ring_unit<MODE, T, 256, 2 * base_vpl<T, 256>(), 2>(a, begin, count);
+    } else {
+#define FMM_RING_R(RR)                                                                       \
+    case RR:                                                                                 \
+        run_ring_unit<MODE, T, RR, ring_vpl<MODE>(RR), ring_depth<MODE>(RR)>(a, begin, count); \
         return;
-    case 64: run_ring_unit<MODE, 64, ring_vpl<MODE>(64), ring_depth<MODE>(64)>(a, begin, count); return;
-    case 128: run_ring_unit<MODE, 128, ring_vpl<MODE>(128), ring_depth<MODE>(128)>(a, begin, count); return;
-    case 256: run_ring_unit<MODE, 256, ring_vpl<MODE>(256), ring_depth<MODE>(256)>(a, begin, count); return;
+        switch (r) {
+        case 32:
+            if constexpr (ring_vpl<MODE>(32) == 0)
+                run_unit<MODE, T, 32, 1, 1, 2>(a, begin, count);
+            else
+                run_ring_unit<MODE, T, 32, ring_vpl<MODE>(32), ring_depth<MODE>(32)>(a, begin, count);
+            return;
+        FMM_RING_R(64) FMM_RING_R(128) FMM_RING_R(256)
+        }
+#undef FMM_RING_R
     }
 }
 
@@ -216,7 +229,7 @@ __device__ __forceinline__ void for_units(const BatchItemDev *items, const int4 
 
 // The ring layouts have a kernel per role: one for the whole backward phase
 // spilled at its 128 registers (6.2 ms in place of 1.86 + 3.6).
-template <int MODE>
+template <int MODE, typename T>
 __global__ void __launch_bounds__(32, 16) ring_batch_kernel(const BatchItemDev *items,
                                                             const int4 *units, int n_units,
                                                             int *counter)
@@ -224,7 +237,7 @@ __global__ void __launch_bounds__(32, 16) ring_batch_kernel(const BatchItemDev *
     __shared__ __align__(16) unsigned char shared[sizeof(PassArgs)];
     for_units(items, units, n_units, counter, shared,
               [](int, int, const PassArgs &a, int begin, int count) {
-                  run_ring<MODE>(a.r, a, begin, count);
+                  run_ring<MODE, T>(a.r, a, begin, count);
               });
 }
 
@@ -319,6 +332,8 @@ int batch_code(int dtype, int mode, int r, const KernelVariant &v)
 // Teams per warp of a variant code at width r.
 int teams_per_warp(int dtype, int r, int code, int mode)
 {
+    if (code == kRingCode && dtype == FMM_F32)
+        return 2;   // 16 lanes, r = 256
     if (code == kRingCode) {
         const int vpl = mode == M_BWD_COL ? ring_vpl<M_BWD_COL>(r) : ring_vpl<M_FUSED>(r);
         return 32 / (r / 8 / std::max(1, vpl));
@@ -509,7 +524,7 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
         d.bwd_col = empty;
         // the ring kernel loads gathered rows 32 bytes at a time
         auto code_of = [&](int mode, const KernelVariant &v, const void *Y, const void *H) {
-            return v.own && dtype == FMM_BF16 && aligned32(Y) && aligned32(H)
+            return v.own && ring_role(mode, dtype, p->r) && aligned32(Y) && aligned32(H)
                        ? kRingCode
                        : batch_code(dtype, mode, p->r, v);
         };
@@ -564,12 +579,13 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
     if (dtype == FMM_BF16) {
         b->grid[0] = grid_for((const void *)batch_kernel<bf16_t, 0>, 256);
         b->grid[1] = grid_for((const void *)batch_kernel<bf16_t, 1>, 256);
-        b->grid[2] = grid_for((const void *)ring_batch_kernel<M_FUSED>, 32);
-        b->grid[3] = grid_for((const void *)ring_batch_kernel<M_BWD_ROW>, 32);
-        b->grid[4] = grid_for((const void *)ring_batch_kernel<M_BWD_COL>, 32);
+        b->grid[2] = grid_for((const void *)ring_batch_kernel<M_FUSED, bf16_t>, 32);
+        b->grid[3] = grid_for((const void *)ring_batch_kernel<M_BWD_ROW, bf16_t>, 32);
+        b->grid[4] = grid_for((const void *)ring_batch_kernel<M_BWD_COL, bf16_t>, 32);
     } else {
         b->grid[0] = grid_for((const void *)batch_kernel<float, 0>, 256);
         b->grid[1] = grid_for((const void *)batch_kernel<float, 1>, 256);
+        b->grid[3] = grid_for((const void *)ring_batch_kernel<M_BWD_ROW, float>, 32);
     }
     *batch = b;
     return FMM_OK;
@@ -590,11 +606,11 @@ static int run_phase(const fmm_batch *b, int phase, fmm_stream stream, const cha
     };
     const bool bf16 = b->dtype == FMM_BF16;
     if (phase == 0) {
-        run(ring_batch_kernel<M_FUSED>, 2, 32);
+        run(ring_batch_kernel<M_FUSED, bf16_t>, 2, 32);
         run(bf16 ? batch_kernel<bf16_t, 0> : batch_kernel<float, 0>, 0, 256);
     } else {
-        run(ring_batch_kernel<M_BWD_ROW>, 3, 32);
-        run(ring_batch_kernel<M_BWD_COL>, 4, 32);
+        run(bf16 ? ring_batch_kernel<M_BWD_ROW, bf16_t> : ring_batch_kernel<M_BWD_ROW, float>, 3, 32);
+        run(ring_batch_kernel<M_BWD_COL, bf16_t>, 4, 32);
         run(bf16 ? batch_kernel<bf16_t, 1> : batch_kernel<float, 1>, 1, 256);
     }
     const int n_sums = phase ? b->n_sums_bwd : b->n_sums_fwd;

@@ -145,10 +145,17 @@ cudaError_t launch_pass_bf16(int mode, int vpl_mult, int ng, int u, bool vec, co
 // per row at most.
 cudaError_t launch_flex_f32(int mode, const PassArgs &a, int vb, int ng, cudaStream_t st);
 cudaError_t launch_flex_bf16(int mode, const PassArgs &a, int vb, int ng, cudaStream_t st);
-// Passes with a warp for each of the first n_wide work items (fmm_wide.cuh);
-// vectorised widths.
-cudaError_t launch_wide_f32(int mode, const PassArgs &a, int n_wide, cudaStream_t st);
-cudaError_t launch_wide_bf16(int mode, const PassArgs &a, int n_wide, cudaStream_t st);
+// Roles and widths that may give a warp to a long row (fmm_wide.cuh).
+constexpr bool wide_role(int mode, bool bf16, int r)
+{
+    if (bf16)
+        return r == 32 || (mode == M_FUSED && r == 64) || (mode == M_BWD_ROW && r <= 128);
+    return mode == M_SDDMM ? r <= 64 : (mode != M_BWD_ROW && mode != M_BWD_COL) || r <= 128;
+}
+// Passes with a warp for each of the first n_wide work items; ring: the other
+// choice for the pass is the register ring.
+cudaError_t launch_wide_f32(int mode, const PassArgs &a, int n_wide, bool ring, cudaStream_t st);
+cudaError_t launch_wide_bf16(int mode, const PassArgs &a, int n_wide, bool ring, cudaStream_t st);
 // Widest row of the flexible pass (32 lanes of 16 elements); the generic pass
 // takes only wider ones and relies on it.
 constexpr int32_t kFlexMaxR = 512;

@@ -2,8 +2,8 @@
 #include "fmm_wide.cuh"
 
 namespace fmm {
-cudaError_t launch_wide_f32(int mode, const PassArgs &a, int n_wide, cudaStream_t st)
+cudaError_t launch_wide_f32(int mode, const PassArgs &a, int n_wide, bool ring, cudaStream_t st)
 {
-    return launch_wide_typed<float>(mode, a, n_wide, st);
+    return launch_wide_typed<float>(mode, a, n_wide, ring, st);
 }
 }  // namespace fmm

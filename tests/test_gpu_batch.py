@@ -288,3 +288,41 @@ def test_split_nnz_and_what_the_info_says(dtype):
                     oracle.fusedmm(S.row_ptr, S.col_idx, None, A.double().cpu().numpy(),
                                    B.double().cpu().numpy(), S.n)) <= 1e-5
         batch.close()
+
+
+@pytest.mark.parametrize("dtype,offset", [(torch.float32, 0), (torch.float32, 4), (torch.bfloat16, 0),
+                                          (torch.bfloat16, 8)])
+@pytest.mark.parametrize("r", [32, 64, 128, 256])
+def test_batch_of_untouched_plans(r, dtype, offset):
+    """Plans left to their own choice: a batch gives the bits of their own
+    calls, which take other passes where the pattern asks for them (rows of
+    their own warp, rows in chunks), also with operands that are 16-byte but not
+    32-byte aligned (offset)."""
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(r + offset)
+    f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+
+    def rows(k):
+        buf = torch.zeros(k * r + offset, dtype=dtype, device="cuda")
+        buf[offset:] = f(k * r).to(dtype)
+        return buf[offset:].view(k, r)
+    items = []
+    for m, n, deg, hubs in ((300, 250, 9.0, ()), (1, 40, 30.0, ()), (700, 90, 3.0, ((0, 400), (9, 47))),
+                            (9000, 5000, 12.0, ((3, 255), (4000, 48))), (40, 3000, 20.0, ((7, 3000),))):
+        S = wl.random_csr(m, n, rng, mean_deg=deg, empty_frac=0.1, hubs=hubs)
+        for split in (1 << 30, max(1, int(S.degrees().max()), int(np.bincount(S.col_idx, minlength=n).max()))):
+            plan = fmm.Plan(torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda(), n,
+                            r, dtype, split_nnz=split)
+            items.append(dict(plan=plan, vals=f(S.nnz), A=rows(m), B=rows(n), G=f(m, r),
+                              out=torch.empty(m, r, device="cuda"), dA=torch.empty(m, r, device="cuda"),
+                              dB=torch.empty(n, r, device="cuda"), ds=torch.empty(S.nnz, device="cuda")))
+    batch = fmm.Batch(items)
+    batch.forward()
+    batch.backward()
+    for k, it in enumerate(items):
+        p = it["plan"]
+        want = (fmm.fusedmm(p, it["vals"], it["A"], it["B"]),
+                *fmm.fusedmm_bwd(p, it["vals"], it["A"], it["B"], it["G"]))
+        for name, w in zip(("out", "dA", "dB", "ds"), want):
+            assert torch.equal(it[name], w), (k, name)
+    batch.close()
