@@ -323,8 +323,9 @@ int fmm_spmm_t_acc(const fmm_plan *plan, const float *v, const void *A, float *o
  * Kernel variant of a plan's row passes (the codes of
  * fmm_plan_options.variant; 0 leaves a side unchanged).  variant applies to
  * passes over S, variant_t to passes over S^T.  The code of a plan's default
- * for both gives the default back, with its own choice per operation and
- * size.  Used by the autotuner; calls already queued are not affected.
+ * gives a side the default back, with its own choice per operation and size
+ * (fmm_plan_options.variant sets that code's layout alone).  Used by the
+ * autotuner; calls already queued are not affected.
  */
 int fmm_plan_set_variant(fmm_plan *plan, int32_t variant, int32_t variant_t);
 

@@ -411,13 +411,15 @@ int fmm_plan_set_variant(fmm_plan *p, int32_t variant, int32_t variant_t)
         set_error_msg("invalid plan or variant code");
         return FMM_EINVAL;
     }
-    // the code of the plan's own choice on both sides gives that choice back
+    // the code of the plan's own choice gives a side that choice back (as a
+    // layout of its own the code can be given to fmm_plan_create): a tuner that
+    // times a code on both sides and keeps it on one keeps what it timed
     const KernelVariant own = default_variant(p->r, p->dtype, 0.0);
-    const bool back = variant == variant_t && variant == encode_variant(own);
+    auto of = [&](int32_t code) { return code == encode_variant(own) ? own : decode_variant(code); };
     if (variant)
-        p->rows.variant = back ? own : decode_variant(variant);
+        p->rows.variant = of(variant);
     if (variant_t)
-        p->cols.variant = back ? own : decode_variant(variant_t);
+        p->cols.variant = of(variant_t);
     return FMM_OK;
 }
 

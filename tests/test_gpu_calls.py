@@ -248,3 +248,32 @@ def test_threads():
     for t in threads:
         t.join()
     assert not failed, failed
+
+
+@pytest.mark.parametrize("dtype,r,own,other", [(torch.bfloat16, 64, 32212, 112), (torch.float32, 256, 112, 122)])
+def test_default_code_gives_a_side_its_own_choice_back(dtype, r, own, other):
+    """fmm_plan_set_variant with the code of a plan's default on one side: that
+    side runs what an untouched plan runs (another layout than the code's in one
+    of the adjoints, which shows in its bits), whatever the other side has."""
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(r)
+    S = wl.random_csr(500, 400, rng, mean_deg=12, hubs=((3, 200),))
+    f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+    v, A, B, G = f(S.nnz), f(S.m, r).to(dtype), f(S.n, r).to(dtype), f(S.m, r)
+
+    def grads(*codes, **kw):
+        plan = fmm.Plan(torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda(), S.n, r,
+                        dtype, **kw)
+        assert kw or plan.info()["variant"] == plan.info()["variant_t"] == own
+        for c in codes:
+            plan.set_variant(*c)
+        out = fmm.fusedmm_bwd(plan, v, A, B, G)
+        plan.close()
+        return out
+    side = 1 if dtype == torch.bfloat16 else 0   # dB by the columns, dA by the rows
+    want, plain = grads()[side], grads(variant=own)[side]
+    assert not torch.equal(want, plain)
+    pair = lambda mine, theirs: (theirs, mine) if side else (mine, theirs)
+    for codes in ([pair(own, other)], [pair(own, 0)], [(own, own)], [pair(other, other), pair(own, 0)]):
+        assert torch.equal(grads(*codes)[side], want), codes
+    assert not torch.equal(grads(pair(other, own))[side], want)
