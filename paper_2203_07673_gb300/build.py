@@ -69,11 +69,22 @@ def _run(cmd, what):
         raise RuntimeError(f"{cmd[0]} failed for {what}:\n{res.stderr}")
 
 
+def _drop_calls():
+    """Removes the module of the call path (and its stamp)."""
+    for path in (CALLS + ".stamp", CALLS):
+        if os.path.exists(path):
+            os.remove(path)
+
+
 def _compile_calls(force):
     """Compiles csrc/torch_calls.cpp against the installed PyTorch; returns the
-    object file, PyTorch's directory and whether anything changed."""
+    object file, PyTorch's directory and the key of both, or None where the
+    module is up to date.  A module of another key is removed first."""
     src, obj = os.path.join(CSRC, "torch_calls.cpp"), os.path.join(OUT, "torch_calls.o")
-    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    spec = importlib.util.find_spec("torch")
+    if spec is None:
+        raise RuntimeError("PyTorch is not installed")
+    torch_dir = os.path.dirname(spec.origin)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     inc = [INCLUDE, os.path.join(torch_dir, "include"),
            os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
@@ -83,25 +94,24 @@ def _compile_calls(force):
     for path in (src, os.path.join(INCLUDE, "fmm.h"), os.path.join(torch_dir, "version.py")):
         with open(path, "rb") as fh:
             h.update(fh.read())
-    stamp = obj + ".stamp"
-    if not force and os.path.exists(obj) and os.path.exists(stamp):
+    stamp = CALLS + ".stamp"   # written once the module is linked
+    if not force and os.path.exists(CALLS) and os.path.exists(stamp):
         with open(stamp) as fh:
             if fh.read() == h.hexdigest():
-                return obj, torch_dir, False
+                return None
+    _drop_calls()
     _run(cmd, src)
-    with open(stamp, "w") as fh:
-        fh.write(h.hexdigest())
-    return obj, torch_dir, True
+    return obj, torch_dir, h.hexdigest()
 
 
-def _link_calls(obj, torch_dir, changed):
-    if not changed and os.path.exists(CALLS):
-        return
+def _link_calls(obj, torch_dir, key):
     tmp = CALLS + f".tmp{os.getpid()}"
     _run([CXX, "-shared", obj, "-o", tmp, f"-L{os.path.join(torch_dir, 'lib')}", "-lc10",
           "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python", f"-L{OUT}", "-l:libfmm.so",
           "-Wl,-rpath,$ORIGIN"], CALLS)
     os.replace(tmp, CALLS)
+    with open(CALLS + ".stamp", "w") as fh:
+        fh.write(key)
 
 
 def build_library(force: bool = False, extra_flags=(), verbose: bool = False) -> str:
@@ -122,9 +132,12 @@ def build_library(force: bool = False, extra_flags=(), verbose: bool = False) ->
             raise RuntimeError(f"link failed:\n{res.stderr}")
         os.replace(tmp, LIB)
     try:
-        _link_calls(*calls.result())
-    except RuntimeError as e:
+        built = calls.result()
+        if built is not None:
+            _link_calls(*built)
+    except (RuntimeError, OSError) as e:
         # every call then takes its path in Python: slower, the same results
+        _drop_calls()
         print(f"{CALLS} not built: {e}", file=sys.stderr)
     if verbose:
         print(LIB)
