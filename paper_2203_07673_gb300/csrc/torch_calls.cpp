@@ -29,6 +29,7 @@
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/csrc/jit/frontend/tracer.h>
+#include <torch/version.h>
 
 #include "fmm.h"
 
@@ -467,4 +468,13 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "fmm_calls", nullptr, -1, kMethods
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit_fmm_calls(void) { return PyModule_Create(&kModule); }
+PyMODINIT_FUNC PyInit_fmm_calls(void)
+{
+    PyObject *m = PyModule_Create(&kModule);
+    // the PyTorch it is built for: fmm.py uses it with no other
+    if (m && PyModule_AddStringConstant(m, "torch_version", TORCH_VERSION) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

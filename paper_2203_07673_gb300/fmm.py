@@ -16,7 +16,9 @@ import ctypes
 import importlib.machinery
 import importlib.util
 import os
+import re
 import threading
+import warnings
 
 import torch
 
@@ -103,11 +105,21 @@ _calls = None   # the native call path, once the library is loaded (if it is bui
 
 
 def _load_calls():
+    """The native call path, or None where it is not built, does not load or is
+    of another PyTorch: every call then takes its path in Python."""
     if not os.path.exists(CALLS_PATH):
         return None
     loader = importlib.machinery.ExtensionFileLoader("fmm_calls", CALLS_PATH)
-    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("fmm_calls", loader))
-    loader.exec_module(mod)
+    try:
+        mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("fmm_calls", loader))
+        loader.exec_module(mod)
+    except ImportError as e:
+        warnings.warn(f"{CALLS_PATH} does not load ({e}); calls take their path in Python")
+        return None
+    if mod.torch_version != re.match(r"[\d.]*\d|", str(torch.__version__)).group():
+        warnings.warn(f"{CALLS_PATH} is built for PyTorch {mod.torch_version}, this is "
+                      f"{torch.__version__}; calls take their path in Python")
+        return None
     mod.set_check(_check)
     return mod
 
@@ -126,9 +138,9 @@ def lib() -> ctypes.CDLL:
                 fn = getattr(handle, name)
                 fn.argtypes = args
                 fn.restype = res
-            _lib = handle
             if _calls is None:
                 _calls = _load_calls()
+            _lib = handle
     return _lib
 
 

@@ -1,12 +1,14 @@
 """The native call module is optional: whatever stops its build, the library is
 built all the same, no earlier module stays behind to be loaded, and the next
-build makes it."""
+build makes it; a module that does not load, or is of another PyTorch, is left
+out."""
 import os
 import stat
 
 import pytest
+import torch
 
-from paper_2203_07673_gb300 import build
+from paper_2203_07673_gb300 import build, fmm
 
 
 @pytest.fixture
@@ -59,3 +61,24 @@ def test_no_pytorch(tree, monkeypatch, capsys):
     monkeypatch.setattr(build.importlib.util, "find_spec", lambda name: None)
     assert os.path.exists(build.build_library())
     assert not calls.exists() and "PyTorch is not installed" in capsys.readouterr().err
+
+
+def test_a_module_that_does_not_load(tmp_path, monkeypatch):
+    """The library loads without it, at the first call as at the second."""
+    bad = tmp_path / "fmm_calls.so"
+    bad.write_text("not a module")
+    monkeypatch.setattr(fmm, "CALLS_PATH", str(bad))
+    monkeypatch.setattr(fmm, "_lib", None)
+    monkeypatch.setattr(fmm, "_calls", None)
+    with pytest.warns(UserWarning, match="does not load"):
+        assert fmm.lib().fmm_version() > 0
+    assert fmm._calls is None and fmm.lib().fmm_version() > 0
+
+
+def test_a_module_of_another_pytorch(monkeypatch):
+    if not os.path.exists(fmm.CALLS_PATH):
+        pytest.skip("the module is not built")
+    assert fmm._load_calls() is not None
+    monkeypatch.setattr(torch, "__version__", "1.0.0+cpu")
+    with pytest.warns(UserWarning, match="built for PyTorch"):
+        assert fmm._load_calls() is None
