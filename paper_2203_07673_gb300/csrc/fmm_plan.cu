@@ -430,6 +430,7 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
 {
     side.rows = rows;
     side.row_ptr = row_ptr;
+    side.bucket_start.assign(257, 0);
     if (rows == 0)
         return FMM_OK;
     FMM_TRY(cudaMemsetAsync(tmp.counters, 0, 2 * sizeof(int32_t), st), "memset");
@@ -442,7 +443,6 @@ static int build_side(Side &side, const int32_t *row_ptr, int32_t rows, int32_t 
     const int32_t *order = reinterpret_cast<const int32_t *>(in_b ? tmp.vb : tmp.va);
     // start of every length key in the order: the scanned digit offsets of the
     // sort's first tile (entry key * ntiles of the histogram)
-    side.bucket_start.assign(257, 0);
     if (rows > 1) {
         const int64_t ntiles = (rows + RS_TILE - 1) / RS_TILE;
         uint32_t starts[256];

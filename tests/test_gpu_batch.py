@@ -326,3 +326,41 @@ def test_batch_of_untouched_plans(r, dtype, offset):
         for name, w in zip(("out", "dA", "dB", "ds"), want):
             assert torch.equal(it[name], w), (k, name)
     batch.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+def test_batch_with_empty_matrices(dtype):
+    """Matrices without rows, without columns and without either beside others:
+    their outputs are zeros or nothing, the others those of their own calls, and
+    a matrix without columns whose dB is given has an adjoint."""
+    import ctypes
+    from paper_2203_07673_gb300 import fmm
+    rng = np.random.default_rng(2)
+    r = 32
+    f = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).cuda()
+    items = []
+    for m, n, deg in ((0, 50, 0.0), (40, 30, 4.0), (30, 0, 0.0), (0, 0, 0.0)):
+        S = wl.random_csr(m, n, rng, mean_deg=deg) if deg else wl.CSR(
+            m, n, np.zeros(m + 1, np.int32), np.zeros(0, np.int32))
+        plan = fmm.Plan(torch.from_numpy(S.row_ptr).cuda(), torch.from_numpy(S.col_idx).cuda(), n, r,
+                        dtype, split_nnz=1 << 30)
+        items.append(dict(plan=plan, vals=f(S.nnz), A=f(m, r).to(dtype), B=f(n, r).to(dtype), G=f(m, r),
+                          out=torch.full((m, r), np.nan, device="cuda"),
+                          dA=torch.full((m, r), np.nan, device="cuda")))
+    batch = fmm.Batch(items)
+    batch.forward()
+    for it in items:
+        assert torch.equal(it["out"], fmm.fusedmm(it["plan"], it["vals"], it["A"], it["B"]))
+    batch.close()
+    it, spare = items[2], torch.zeros(4 * r, device="cuda")
+    ptr = lambda t: t.data_ptr()
+    arr = (fmm._BatchItem * 1)(fmm._BatchItem(it["plan"].handle, None, ptr(it["A"]), None, ptr(it["out"]),
+                                              ptr(it["G"]), ptr(it["dA"]), ptr(spare), None))
+    out = ctypes.c_void_p()
+    assert fmm.lib().fmm_batch_create(arr, 1, fmm._stream(), ctypes.byref(out)) == fmm.FMM_OK
+    it["out"].fill_(float("nan"))
+    for call in (fmm.lib().fmm_batch_forward, fmm.lib().fmm_batch_backward):
+        assert call(out, fmm._stream()) == fmm.FMM_OK
+    torch.cuda.synchronize()
+    assert not it["out"].any() and not it["dA"].any() and not spare.any()
+    assert fmm.lib().fmm_batch_destroy(out) == fmm.FMM_OK
