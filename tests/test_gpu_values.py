@@ -40,3 +40,29 @@ def test_values_reach_their_columns(nnz, kind, shift):
     plan.set_values(v)
     assert torch.equal(fmm.spmm_t(plan, v, torch.ones(m, 4, device="cuda")), got)
     plan.close()
+
+
+@pytest.mark.parametrize("side", [3000, 4200, 16400])
+def test_every_value_keeps_its_row(side):
+    """All three ways to the order of S^T: a single gather (9.0M nonzeros),
+    through shared memory (17.6M) and in windows (269M, above 2^28).  A full
+    pattern with the columns of each row in an order of its own, and operand
+    rows that differ, so that two values changed about show even inside a
+    column; integers small enough for every sum to be exact."""
+    from paper_2203_07673_gb300 import fmm
+    g = torch.Generator(device="cuda").manual_seed(side)
+    i = torch.arange(side, device="cuda")
+    cols = torch.cat([(i * 1009 + 37 * r) % side for r in range(side)]).int()
+    assert side % 1009 != 0
+    plan = fmm.Plan((torch.arange(side + 1, device="cuda") * side).int(), cols, side, 32)
+    v = torch.randint(0, 8, (side * side,), generator=g, device="cuda").float()
+    A = torch.randint(0, 64, (side, 32), generator=g, device="cuda").float()
+    dense = torch.empty(side, side, device="cuda")
+    dense.scatter_(1, cols.view(side, side).long(), v.view(side, side))
+    want = dense.double().t() @ A.double()
+    assert want.max() < 2 ** 24
+    del dense
+    assert torch.equal(fmm.spmm_t(plan, v, A).double(), want)
+    plan.set_values(v)
+    assert torch.equal(fmm.spmm_t(plan, v, A).double(), want)
+    plan.close()
