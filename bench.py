@@ -46,7 +46,8 @@ KERNEL_SOURCES = [os.path.join(ROOT, "paper_2203_07673_gb300", "csrc", f)
                             "fmm_staged.cuh", "fmm_staged_f32.cu", "fmm_staged_bf16.cu",
                             "fmm_pipe.cuh", "fmm_pipe_f32.cu", "fmm_pipe_bf16.cu",
                             "fmm_stream.cuh", "fmm_stream_f32.cu", "fmm_stream_bf16.cu",
-                            "fmm_values.cu", "fmm_wide.cuh",
+                            "fmm_values.cu", "fmm_flex.cuh", "fmm_wide.cuh",
+                            "fmm_wide_f32.cu", "fmm_wide_bf16.cu",
                             "fmm_internal.cuh", "fmm_plan.cu")]
 
 

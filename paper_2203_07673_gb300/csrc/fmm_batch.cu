@@ -2,19 +2,21 @@
 //
 // Every matrix of a batch keeps its own plan (pattern, S^T, row order).  A
 // batch lists, for each matrix and each row pass of a phase, work units of
-// consecutive teams (rows in the plan's longest-first order).  Units of all
-// matrices are sorted longest-rows-first and handed out by a device counter:
-// every warp of a grid sized to fill the GPU pops a unit, runs the team
-// kernel body of that matrix's row width and kernel variant on it, and pops
-// the next, until the list is empty.  Forward (FusedMMA of every matrix) is
-// one launch; backward (dA and ds over S, dB over S^T, for every matrix) is
-// one launch.  The counter is cleared by a memset queued before each launch,
-// so both phases can be captured in a CUDA graph and replayed.
+// consecutive teams (chunks, then rows in the plan's longest-first order).  The
+// units are handed out by a device counter: every warp of a grid sized to fill
+// the GPU pops a unit, runs the pass body of that matrix's row width and layout
+// on it, and pops the next, until the list is empty.  There is a list, a counter
+// and a persistent kernel for the team layouts of each phase and for the
+// register-ring layouts of each role, so forward (FusedMMA of every matrix) is
+// one launch or two, backward (dA and ds over S, dB over S^T) up to three; a
+// last kernel sums partial rows.  The counters are cleared by a memset queued
+// before each phase, so both can be captured in a CUDA graph and replayed.
 //
 // Plans whose split_nnz set no limit take rows above the default split size in
 // chunks, here as in their own calls, with partial rows in the batch's own
-// memory, summed in chunk order by a second kernel.
-// Results are bitwise those of the per-matrix calls with the same variants.
+// memory, summed in chunk order.  Results are bitwise those of the per-matrix
+// calls: the layouts are those of the plan, and the passes that a call may take
+// in their place (fmm_wide.cuh) keep their order of sums.
 //
 // Units are handed out matrix by matrix, the matrices with the most work
 // first, and inside a matrix chunks first and then the longest rows: the
@@ -373,8 +375,8 @@ void make_units(std::vector<int4> &out, const Side &side, int item, int code, in
     }
 }
 
-// The split rows of one pass as (partial rows, output row, chunks) for
-// combine_kernel; rows without an output have none.
+// The rows in chunks of one pass as (partial rows, output row, chunks) for
+// batch_sum_kernel; passes without an output have none.
 void make_sums(std::vector<BatchSum> &out, const Side &side, const float *partials, float *dst,
                int32_t r)
 {

@@ -769,10 +769,12 @@ KernelVariant default_variant(int32_t r, int32_t dtype, double avg_nnz)
     if (dtype == FMM_BF16 && fast_r(r))
         v = ring_variant(2, r == 128 ? 4 : 2);
     // float32 rows of r = 128 (512 bytes): the staged pass with a ring of 4
-    // gathered rows per team, 3-4 % faster on Erdos-Renyi rows at the DRAM
-    // roofline (it needs no register spill); where gathers mostly hit L2 the
-    // extra trip through shared memory costs more than the deeper ring
-    // gains, and the team kernel stays
+    // gathered rows per team, 3-5 % faster than the team kernel where the
+    // gathered operand is larger than L2 (it needs no register spill;
+    // Erdos-Renyi rows of 32, 2^18 / 2^19 / 2^20 rows: 404 -> 393 us, 1011 ->
+    // 956, 2354 -> 2279).  It is taken for smaller operands too, whose gathers
+    // hit L2 and where the trip through shared memory costs more than the ring
+    // gains (2^17 rows: 147 -> 199, R-MAT 2^17: 97 -> 114)
     if (dtype == FMM_F32 && r == 128)
         v.stages = 4;
     v.own = true;

@@ -524,8 +524,8 @@ class _BatchItem(ctypes.Structure):
 
 
 class Batch:
-    """fmm_batch: FusedMMA (and its adjoint) of many plans in one persistent
-    launch per phase.  ``items`` is a list of dicts with keys plan, vals, A,
+    """fmm_batch: FusedMMA (and its adjoint) of many plans in a few persistent
+    launches per phase.  ``items`` is a list of dicts with keys plan, vals, A,
     B, out and optionally G, dA, dB, ds (tensors on the plans' device).  The
     batch keeps references to every tensor; their storage must not move."""
 
