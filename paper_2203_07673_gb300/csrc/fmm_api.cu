@@ -193,21 +193,26 @@ static int wide_items(int mode, int dtype, const PassArgs &a)
     if (chain <= (ring ? 3.0 : high ? 1.6 : 0.9) * work)
         return 0;
     const long long items = (long long)a.n_chunks + a.n_light;
-    const uint32_t key = length_key(items <= (long long)sm_count() * 48 ? 8 : 48, INT32_MAX);
+    // (at r = 256 an SM holds twelve such warps: 2000 Erdos-Renyi rows of 16 took
+    // 10.6 us in two waves, 8.1 by the variant)
+    const long long few = (long long)sm_count() * (a.r == 256 ? 12 : 48);
+    const uint32_t key = length_key(items <= few ? 8 : 48, INT32_MAX);
     return a.n_chunks + a.bucket_start[key + 1] - a.bucket_start[1];
 }
 
 cudaError_t launch_pass(int mode, int dtype, const KernelVariant &given, const PassArgs &a,
                         cudaStream_t st)
 {
-    const KernelVariant v = given.own ? role_variant(mode, a.r, dtype) : given;
+    const long long items = std::max<long long>(1, (long long)a.n_chunks + a.n_light);
+    const KernelVariant v =
+        given.own ? role_variant(mode, a.r, dtype, (double)a.nnz / items, a.longest) : given;
     const bool vec = fast_r(a.r) && aligned16(a.L) && aligned16(a.Y) && aligned16(a.H) &&
                      aligned16(a.out) && aligned16(a.out16) && aligned16(a.partials);
     const bool fwd = mode == M_FUSED || mode == M_SDDMM || mode == M_SPMM;
     if (given.own && vec) {
         const int n_wide = wide_items(mode, dtype, a);
         if (n_wide > 0)
-            return dtype == FMM_BF16 ? launch_wide_bf16(mode, a, n_wide, aligned32(a.Y), st)
+            return dtype == FMM_BF16 ? launch_wide_bf16(mode, a, n_wide, v.ring > 0 && aligned32(a.Y), st)
                                      : launch_wide_f32(mode, a, n_wide, false, st);
     }
     if (v.stages > 0 && vec && fwd) {

@@ -151,10 +151,16 @@ __device__ __forceinline__ void run_ring_unit(const PassArgs &a, int begin, int 
 
 constexpr int kRingCode = 9;   // in place of a team code
 
-// Whether role_variant gives a role a layout of the ring kernels below.
-bool ring_role(int mode, int dtype, int r)
+// Whether the own choice of a pass over `side` is a layout of the ring kernels
+// below (the adjoint over S^T of bfloat16 r = 32 by the team body).
+bool ring_role(int mode, int dtype, int r, const Side &side, int64_t nnz)
 {
-    return dtype == FMM_BF16 || (mode == M_BWD_ROW && r == 256);
+    if (dtype == FMM_F32 && (mode != M_BWD_ROW || r != 256))
+        return false;
+    if (mode == M_BWD_COL && r == 32)
+        return true;
+    const long long items = std::max<long long>(1, (long long)side.n_chunks + side.n_light);
+    return role_variant(mode, r, dtype, (double)nnz / items, side.longest).ring > 0;
 }
 
 // Vectors per lane of the ring layouts of bfloat16 rows (0: the team kernel).
@@ -527,20 +533,21 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
         PassArgs empty{};
         d.bwd_col = empty;
         // the ring kernel loads gathered rows 32 bytes at a time
-        auto code_of = [&](int mode, const KernelVariant &v, const void *Y, const void *H) {
-            return v.own && ring_role(mode, dtype, p->r) && aligned32(Y) && aligned32(H)
+        auto code_of = [&](int mode, const Side &side, const void *Y, const void *H) {
+            return side.variant.own && ring_role(mode, dtype, p->r, side, p->nnz) && aligned32(Y) &&
+                           aligned32(H)
                        ? kRingCode
-                       : batch_code(dtype, mode, p->r, v);
+                       : batch_code(dtype, mode, p->r, side.variant);
         };
         auto list = [&](int kind, int code) -> std::vector<int4> & {
             return units[code == kRingCode ? 2 + kind : kind != U_FWD];
         };
-        const int cf = code_of(M_FUSED, p->rows.variant, it.B, nullptr);
+        const int cf = code_of(M_FUSED, p->rows, it.B, nullptr);
         const int rcode = p->r << 16;
         make_units(list(U_FWD, cf), p->rows, i, 4 * (rcode | cf) + U_FWD, teams_per_warp(dtype, p->r, cf, M_FUSED),
                    unit_nnz);
         if (bwd) {
-            const int cr = code_of(M_BWD_ROW, p->rows.variant, it.B, nullptr);
+            const int cr = code_of(M_BWD_ROW, p->rows, it.B, nullptr);
             make_sums(sums_b, p->rows, next_partials, it.dA, p->r);
             next_partials += (size_t)p->rows.n_chunks * p->r;
             if (it.dA || it.ds)
@@ -550,7 +557,7 @@ int fmm_batch_create(const fmm_batch_item *items, int32_t count, fmm_stream stre
                 fill(d.bwd_col, p->cols, it.vals, it.B, it.A, it.G, it.dB, nullptr);
                 make_sums(sums_b, p->cols, next_partials, it.dB, p->r);
                 next_partials += (size_t)p->cols.n_chunks * p->r;
-                const int cc = code_of(M_BWD_COL, p->cols.variant, it.A, it.G);
+                const int cc = code_of(M_BWD_COL, p->cols, it.A, it.G);
                 make_units(list(U_BWD_COL, cc), p->cols, i, 4 * (rcode | cc) + U_BWD_COL,
                            teams_per_warp(dtype, p->r, cc, M_BWD_COL), unit_nnz);
             }

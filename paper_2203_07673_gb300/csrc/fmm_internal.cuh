@@ -238,8 +238,9 @@ int encode_variant(const KernelVariant &v);
 // Default kernel variant of a pass over rows of width r (dtype, average
 // nonzeros per row).
 KernelVariant default_variant(int32_t r, int32_t dtype, double avg_nnz);
-// The same per role (default_variant is that of FusedMM).
-KernelVariant role_variant(int mode, int32_t r, int32_t dtype);
+// The same per role (default_variant is that of FusedMM), for work items of avg
+// nonzeros on average and `longest` at most.
+KernelVariant role_variant(int mode, int32_t r, int32_t dtype, double avg, int32_t longest);
 // The team kernel's layout for a width (one group per row, 8 elements per
 // lane, 2 nonzeros per batch): the default of the batch kernels.
 KernelVariant team_default_variant(int32_t r, int32_t dtype);

@@ -802,25 +802,39 @@ KernelVariant default_variant(int32_t r, int32_t dtype, double avg_nnz)
 // pass -> .754 .081) and of r = 256 (.394 .218 -> .381 .193), adjoint over S of
 // r = 256 (.623 .345 -> .537 .313); the other roles lose with a ring (FusedMM
 // also has to keep its order of sums, see fmm_flex.cuh).
-KernelVariant role_variant(int mode, int32_t r, int32_t dtype)
+// Where the rows of a pattern (avg nonzeros per work item, longest the longest)
+// take the ring's gain away, the pass keeps the width's default (us, ring and
+// default; rows of k nonzeros each, R-MAT 2^18 and Zipf rows of that average):
+//   float32 SDDMM, r = 128, below 14 a row: k = 4 128 87, 8 158 128, 12 197 172,
+//     16 92 109; R-MAT 8 129 106, 15 194 213; Zipf 8 100 84, 16 149 164
+//   float32, r = 256, from 18 on where rows are alike (none above four times the
+//     average): SDDMM k = 16 225 253, 20 301 282, 32 404 387, Erdos-Renyi of 2^16
+//     rows of 32 164 127, Zipf rows of 24, 2^12 rows, 28 45; adjoint over S k = 16
+//     356 406, 20 464 438, 32 622 540, R-MAT 29 830 958, Zipf 60 1197 1408
+//   bfloat16, r = 32, rows of 4 at most: FusedMM k = 4 25.5 21.1, 6 28.0 28.9,
+//     adjoint over S 33.0 27.8, 37.4 39.8
+KernelVariant role_variant(int mode, int32_t r, int32_t dtype, double avg, int32_t longest)
 {
     KernelVariant v = default_variant(r, dtype, 0.0);
     if (!fast_r(r))
         return v;
     if (dtype == FMM_BF16) {
-        if (mode == M_BWD_ROW)
+        if (r == 32 && longest <= 4)
+            v = team_default_variant(r, dtype);
+        else if (mode == M_BWD_ROW)
             v = ring_variant(2, 4);
         else if (mode == M_BWD_COL)
             v = r == 32 ? team_default_variant(r, dtype)
                         : r == 64 ? ring_variant(1, 4) : ring_variant(2, 2);
         else if (mode != M_FUSED)
             v = r == 32 ? team_default_variant(r, dtype) : ring_variant(2, 2);
-    } else if (mode == M_SDDMM && r >= 128) {
+    } else if (r == 128 && mode == M_SDDMM && avg >= 14) {
         v = ring_variant(2, 2);
         v.u = 2;
-        v.mb = r == 128 ? 3 : 2;
-    } else if (mode == M_BWD_ROW && r == 256) {
+        v.mb = 3;
+    } else if (r == 256 && (mode == M_SDDMM || mode == M_BWD_ROW) && (avg < 18 || longest > 4 * avg)) {
         v = ring_variant(2, 2);
+        v.u = mode == M_SDDMM ? 2 : 1;
     }
     v.own = true;
     return v;

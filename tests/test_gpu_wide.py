@@ -50,3 +50,14 @@ def test_float32_order(m, r, code):
             call(own, vals, *x, out=got)
             call(team, vals, *x, out=want)
             assert torch.equal(got, want), (name, acc)
+
+
+@pytest.mark.parametrize("dtype,r", [(torch.float32, 128), (torch.float32, 256), (torch.bfloat16, 32)])
+@pytest.mark.parametrize("k", [1, 4, 5, 13, 14, 17, 18, 40])
+def test_rows_alike(k, dtype, r):
+    """Patterns of k nonzeros in every row, on both sides of the averages at which
+    SDDMM and the adjoints of a plan left to its own choice change their layout,
+    and with one long row, which changes it back."""
+    rng = np.random.default_rng(k)
+    run_all(wl.er_exact_degree(700, 300, k, rng), {}, r, dtype, seed=k)
+    run_all(wl.random_csr(700, 300, rng, mean_deg=k, hubs=((5, 250),)), {}, r, dtype, seed=k)
