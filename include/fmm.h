@@ -152,9 +152,10 @@ typedef struct fmm_plan_options {
                                  Default: 32212 for bfloat16 rows (32412 for
                                  r = 128), 1042 for float32 rows of r = 128,
                                  else that team layout; SDDMM, SpMM and the
-                                 adjoints of a plan left to its default, and
-                                 passes bound by their longest rows, may run
-                                 another layout                              */
+                                 adjoints of a plan left to its default,
+                                 passes over rows of a few nonzeros and passes
+                                 bound by their longest rows may run another
+                                 layout                                      */
 } fmm_plan_options;
 
 typedef struct fmm_plan fmm_plan;   /* opaque */
