@@ -55,3 +55,19 @@ def test_widths_and_chunk_edges(r, dtype):
 
 def test_no_nonzeros():
     check(csr(np.zeros(1500, np.int64), 7, np.random.default_rng(0)), 64, torch.float32, 0)
+
+
+@pytest.mark.parametrize("m,hub", [(1, 5000), (31, 129), (4095, 700), (4096, 128), (4097, 700),
+                                   (4096, 262000), (4096, 262200), (4000, 300000)])
+def test_few_rows(m, hub):
+    """The order of the rows by one block, up to 4096 rows and 4096 chunk slots (2
+    nnz / 128), and by the kernels above either."""
+    rng = np.random.default_rng(m + hub)
+    deg = np.zeros(m, np.int64) if hub > 200000 else rng.integers(0, 300, m) * (rng.random(m) < 0.3)
+    deg[m // 2] = hub
+    check(csr(deg, 211, rng), 32, torch.float32, m)
+    check(csr(deg, 211, rng), 20, torch.bfloat16, m)
+
+
+def test_rows_of_one_length():
+    check(csr(np.full(3000, 17, np.int64), 211, np.random.default_rng(1)), 128, torch.float32, 3)
